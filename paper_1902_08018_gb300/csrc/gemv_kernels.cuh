@@ -18,6 +18,7 @@
 
 #include <cstdint>
 
+#include "decode_out.cuh"
 #include "wz1_decode.cuh"
 
 namespace whff {
@@ -255,49 +256,53 @@ static __global__ void splitk_epilogue_kernel(const double* __restrict__ ws, int
 }
 
 // ------------------------------------------------------------- decode only
-template <int NW32>
-__global__ void wz1_decompress_kernel(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BN,
-                                      int64_t nblocks, double* __restrict__ out, int64_t ldo) {
-  __shared__ uint32_t planes[kPlaneWords];  // the decoder's plane words, a column per thread
+// Thread per block (WZ1) or per 16-byte chunk (scaled); results as decode_out.cuh says.
+template <int NW32, bool VEC>
+__global__ void __launch_bounds__(kDecodeThreads)
+    wz1_decompress_kernel(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BN, int64_t nblocks,
+                          double* __restrict__ out, int64_t ldo) {
+  __shared__ __align__(16) uint32_t planes[kPlaneWords];  // the decoder's plane words, a column per thread
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nblocks) return;
-  const int64_t I = b / BN, J = b - (b / BN) * BN;
+  const bool live = b < nblocks;
+  int64_t I = 0, J = 0;
+  unit_of(live ? b : nblocks - 1, BN, I, J);
+  uint2 d[16];
   uint32_t w[NW32 + 2];
-  load_block<NW32>(stream, b, w);
+  load_block<NW32>(stream, live ? b : nblocks - 1, w);
   int32_t q[16];
   int emax;
-  const bool nz = decode_block<NW32>(w, planes + threadIdx.x, q, emax);
-  const double scale = nz ? ldexp(1.0, emax - 26) : 0.0;
+  (void)decode_block<NW32>(w, planes + threadIdx.x, q, emax);  // a zero block's q are zeros
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int64_t row = 4 * I + r;
-    if (row >= M) break;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int64_t col = 4 * J + c;
-      if (col < N) out[row * ldo + col] = (double)__int2float_rn(q[4 * r + c]) * scale;
-    }
-  }
+  for (int k = 0; k < 16; ++k) d[k] = f64_from_f32(__int2float_rn(q[k]), emax - 26);
+  if constexpr (!VEC) __syncthreads();  // the plane words have been read: their memory turns the rows round
+  static_assert(kPlaneWords * 4 >= (kDecodeThreads / 32) * 512 * 8, "a warp's 4 x 128 doubles each");
+  store_units<VEC, 4, 4>(d, live, I, J, BN, M, N, out, ldo,
+                         reinterpret_cast<double*>(planes) + (threadIdx.x >> 5) * 512);
 }
 
-template <int FMT>
-__global__ void scaled_decompress_kernel(const uint8_t* __restrict__ payload, const float* __restrict__ scales,
-                                         int64_t M, int64_t N, int64_t ld, int64_t TN, double* __restrict__ out,
-                                         int64_t ldo) {
+template <int FMT, bool VEC>
+__global__ void __launch_bounds__(256)
+    scaled_decompress_kernel(const uint8_t* __restrict__ payload, const float* __restrict__ scales, int64_t M,
+                             int64_t N, int64_t ld, int64_t TN, double* __restrict__ out, int64_t ldo) {
   using T = ScaledTraits<FMT>;
   constexpr int V = T::V;
   constexpr int EB = scaled_elem_bytes<FMT>();
+  __shared__ double turn[VEC ? 1 : 8 * 32 * V];
   const int64_t chunks_per_row = ld / V;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= M * chunks_per_row) return;
-  const int64_t row = t / chunks_per_row, c = (t - row * chunks_per_row) * V;
+  const bool live = t < M * chunks_per_row;
+  int64_t row = 0, j = 0;
+  unit_of(live ? t : M * chunks_per_row - 1, chunks_per_row, row, j);
+  const int64_t c = j * V;
   const uint4 raw = __ldcs(reinterpret_cast<const uint4*>(payload + ((uint64_t)row * ld + c) * EB));
   float f[V];
   T::decode(raw, f);
-  const double s = (double)__ldg(scales + (row / 128) * TN + c / 128);
+  const float s = __ldg(scales + (row / 128) * TN + c / 128);
+  uint2 d[V];
 #pragma unroll
-  for (int v = 0; v < V; ++v)
-    if (c + v < N) out[row * ldo + c + v] = s * (double)f[v];
+  for (int v = 0; v < V; ++v) d[v] = f64_product(f[v], s);
+  store_units<VEC, 1, V>(d, live, row, j, chunks_per_row, M, N, out, ldo,
+                         turn + (VEC ? 0 : (threadIdx.x >> 5) * 32 * V));
 }
 
 }  // namespace dev

@@ -1026,12 +1026,14 @@ extern "C" int whff_decompress(whff_handle* h, double* out, int64_t ldo, void* s
   const cudaStream_t st = as_stream(stream);
   const auto& b = h->info;
   const int threads = 256;
+  const bool vec = dev::out_vec_ok(out, ldo);  // 32-byte stores
   if (b.fmt == WHFF_FMT_ZFP) {
     const int64_t nb = h->BM * h->BN;
     const unsigned grid = (unsigned)((nb + threads - 1) / threads);
 #define DZ(R_)                                                                                          \
   case R_:                                                                                              \
-    dev::wz1_decompress_kernel<R_ / 2><<<grid, threads, 0, st>>>(h->d_stream, b.M, b.N, h->BN, nb, out, ldo); \
+    if (vec) dev::wz1_decompress_kernel<R_ / 2, true><<<grid, threads, 0, st>>>(h->d_stream, b.M, b.N, h->BN, nb, out, ldo); \
+    else dev::wz1_decompress_kernel<R_ / 2, false><<<grid, threads, 0, st>>>(h->d_stream, b.M, b.N, h->BN, nb, out, ldo); \
     break;
     switch (b.rate) {
       DZ(4) DZ(8) DZ(12) DZ(16) DZ(20) DZ(24) DZ(28) DZ(32) DZ(36) DZ(40) DZ(44) DZ(48) DZ(52) DZ(56) DZ(60) DZ(64)
@@ -1064,14 +1066,19 @@ extern "C" int whff_decompress(whff_handle* h, double* out, int64_t ldo, void* s
     const int V = scaled_vec(b.fmt);
     const int64_t work = b.M * (ld / V);
     const unsigned grid = (unsigned)((work + threads - 1) / threads);
-    if (b.fmt == WHFF_FMT_BF16)
-      dev::scaled_decompress_kernel<2><<<grid, threads, 0, st>>>(h->d_stream, scales, b.M, b.N, ld, TN, out, ldo);
-    else if (b.fmt == WHFF_FMT_FP16)
-      dev::scaled_decompress_kernel<3><<<grid, threads, 0, st>>>(h->d_stream, scales, b.M, b.N, ld, TN, out, ldo);
-    else if (b.fmt == WHFF_FMT_FP8E4M3)
-      dev::scaled_decompress_kernel<4><<<grid, threads, 0, st>>>(h->d_stream, scales, b.M, b.N, ld, TN, out, ldo);
-    else
-      dev::scaled_decompress_kernel<7><<<grid, threads, 0, st>>>(h->d_stream, scales, b.M, b.N, ld, TN, out, ldo);
+#define DS(F_)                                                                                                     \
+  if (vec) dev::scaled_decompress_kernel<F_, true><<<grid, threads, 0, st>>>(h->d_stream, scales, b.M, b.N, ld, TN, out, ldo); \
+  else dev::scaled_decompress_kernel<F_, false><<<grid, threads, 0, st>>>(h->d_stream, scales, b.M, b.N, ld, TN, out, ldo);
+    if (b.fmt == WHFF_FMT_BF16) {
+      DS(2)
+    } else if (b.fmt == WHFF_FMT_FP16) {
+      DS(3)
+    } else if (b.fmt == WHFF_FMT_FP8E4M3) {
+      DS(4)
+    } else {
+      DS(7)
+    }
+#undef DS
   }
   WHFF_CUDA_TRY(cudaGetLastError());
   return WHFF_OK;

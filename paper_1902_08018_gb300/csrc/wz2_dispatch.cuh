@@ -100,10 +100,10 @@ template <int RATE>
 int wz2_decompress(const uint8_t* stream, int64_t M, int64_t N, int64_t BN, int64_t nblocks, double* out,
                    int64_t ldo, bool lift, cudaStream_t st) {
   const unsigned grid = (unsigned)((nblocks + 255) / 256);
-  if (lift)
-    dev::wz2_decompress_kernel<RATE, true><<<grid, 256, 0, st>>>(stream, M, N, BN, nblocks, out, ldo);
-  else
-    dev::wz2_decompress_kernel<RATE, false><<<grid, 256, 0, st>>>(stream, M, N, BN, nblocks, out, ldo);
+  const bool vec = dev::out_vec_ok(out, ldo);
+  auto kern = lift ? (vec ? &dev::wz2_decompress_kernel<RATE, true, true> : &dev::wz2_decompress_kernel<RATE, true, false>)
+                   : (vec ? &dev::wz2_decompress_kernel<RATE, false, true> : &dev::wz2_decompress_kernel<RATE, false, false>);
+  kern<<<grid, 256, 0, st>>>(stream, M, N, BN, nblocks, out, ldo);
   return 0;
 }
 

@@ -13,8 +13,10 @@
 // the FP64 epilogue.
 #pragma once
 #include <cstdint>
+#include <type_traits>
 #include <utility>
 
+#include "decode_out.cuh"
 #include "f32x2.cuh"
 #include "gemv_kernels.cuh"
 #include "wz2_batch.h"
@@ -723,56 +725,65 @@ static __global__ void wz2_batched_epilogue(const BatchEntry* __restrict__ entri
   if (e.state) e.state[row] = s;
 }
 
-template <int RATE, bool LIFT>
-__global__ void wz2_decompress_kernel(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BN,
-                                      int64_t nblocks, double* __restrict__ out, int64_t ldo) {
+// Decode only.  Thread per block; the inverse transform (2G) V (2G)^T is taken
+// in FP32 up to rate 20, where it is exact (|v| < 2^18 and the two passes grow
+// it by at most 25), and in integers at rate 24; the FP64 results are put
+// together and written as decode_out.cuh says.  Bound by the 8 bytes written
+// per entry.
+template <int RATE, bool LIFT, bool VEC>
+__global__ void __launch_bounds__(256)
+    wz2_decompress_kernel(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BN, int64_t nblocks,
+                          double* __restrict__ out, int64_t ldo) {
+  __shared__ double turn[VEC ? 1 : 8 * 512];
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nblocks) return;
-  const int64_t I = b / BN, J = b - (b / BN) * BN;
-  uint32_t w[Wz2Layout<RATE>::kWords];
-  wz2_load<RATE>(stream, b, w);
-  const int E = (int)(w[0] & 0xFFu);
-  const int K = (int)((w[0] >> 8) & 31u);
-  float f[16], Vf[16];
-  wz2_fields<RATE>(w, f);
-  wz2_unpermute<LIFT>(f, Vf);
-  int32_t T[16];
+  const bool live = b < nblocks;
+  int64_t I = 0, J = 0;
+  unit_of(live ? b : nblocks - 1, BN, I, J);
+  uint2 d[16];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) T[i] = (int32_t)Vf[i];  // exact: |v| < 2^22
-  double scale;
-  if (LIFT) {
-    // T = (2G) V (2G)^T, integers below 2^27: columns, then rows
+  for (int k = 0; k < 16; ++k) d[k] = make_uint2(0u, 0u);
+  if (live) {
+    uint32_t w[Wz2Layout<RATE>::kWords];
+    wz2_load<RATE>(stream, b, w);
+    const int E = (int)(w[0] & 0xFFu);
+    const int K = (int)((w[0] >> 8) & 31u);
+    if (E) {
+      float f[16], V[16];
+      wz2_fields<RATE>(w, f);
+      wz2_unpermute<LIFT>(f, V);
+      using T = std::conditional_t<(RATE <= 20), float, int32_t>;
+      T t[16];
 #pragma unroll
-    for (int pass = 0; pass < 2; ++pass) {
+      for (int i = 0; i < 16; ++i) t[i] = (T)V[i];  // exact: |v| < 2^22
+      if (LIFT) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int s0 = pass ? 1 : 4, s1 = pass ? 4 : 1;  // pass 0: along a (stride 4); pass 1: along b
-        int32_t& v0 = T[j * s1];
-        int32_t& v1 = T[j * s1 + s0];
-        int32_t& v2 = T[j * s1 + 2 * s0];
-        int32_t& v3 = T[j * s1 + 3 * s0];
-        const int32_t a = 2 * v0;
-        const int32_t r0 = a - v1 - v2, r1 = a - v1 + v2, r2 = a + v1 - v2 - v3, r3 = a + v1 + v2 + v3;
-        v0 = r0;
-        v1 = r1;
-        v2 = r2;
-        v3 = r3;
+        for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int s0 = pass ? 1 : 4, s1 = pass ? 4 : 1;  // pass 0: along a (stride 4); pass 1: along b
+            T& v0 = t[j * s1];
+            T& v1 = t[j * s1 + s0];
+            T& v2 = t[j * s1 + 2 * s0];
+            T& v3 = t[j * s1 + 3 * s0];
+            const T a = 2 * v0;
+            const T m = a - v1, p = a + v1;
+            const T r0 = m - v2, r1 = m + v2, q = p - v2, r3 = p + v2 + v3;
+            v0 = r0;
+            v1 = r1;
+            v2 = q - v3;
+            v3 = r3;
+          }
+        }
+      }
+      const int e = K + (E - 127) - (LIFT ? 30 : 24);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        if constexpr (RATE <= 20) d[i] = f64_from_f32(t[i], e);
+        else d[i] = f64_from_int(t[i], e);
       }
     }
-    scale = ldexp(1.0, K + (E - 127) - 30);
-  } else {
-    scale = ldexp(1.0, K + (E - 127) - 24);
   }
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int64_t row = 4 * I + r;
-    if (row >= M) break;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int64_t col = 4 * J + c;
-      if (col < N) out[row * ldo + col] = E ? (double)T[4 * r + c] * scale : 0.0;
-    }
-  }
+  store_units<VEC, 4, 4>(d, live, I, J, BN, M, N, out, ldo, turn + (VEC ? 0 : (threadIdx.x >> 5) * 512));
 }
 
 }  // namespace dev

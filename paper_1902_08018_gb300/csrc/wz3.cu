@@ -38,7 +38,8 @@ int wz3_occupancy(int R) {
 int wz3_decompress(const uint64_t* index, const uint8_t* area, int64_t M, int64_t N, double* out, int64_t ldo,
                    cudaStream_t st) {
   const int64_t BM = (M + 3) / 4, BN = (N + 3) / 4, RB = (BN + 31) / 32, nb = BM * BN;
-  dev::wz3_decompress_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(index, area, M, N, BN, RB, nb, out, ldo);
+  auto kern = dev::out_vec_ok(out, ldo) ? &dev::wz3_decompress_kernel<true> : &dev::wz3_decompress_kernel<false>;
+  kern<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(index, area, M, N, BN, RB, nb, out, ldo);
   return 0;
 }
 

@@ -193,14 +193,18 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? 4 : 1)
 }
 
 // Decode: thread per block, the exact definition -- T = (2G) V (2G)^T in
-// integers, times 2^(K+emax-30) in FP64 (exact) -- written row-major (ldo),
-// rows and columns past M, N dropped.
-static __global__ void wz3_decompress_kernel(const uint64_t* __restrict__ index, const uint8_t* __restrict__ area,
-                                             int64_t M, int64_t N, int64_t BN, int64_t RB, int64_t nblocks,
-                                             double* __restrict__ out, int64_t ldo) {
+// integers, times 2^(K+emax-30), exact in FP64 -- written row-major (ldo) as
+// decode_out.cuh says, rows and columns past M, N dropped.
+template <bool VEC>
+static __global__ void __launch_bounds__(256)
+    wz3_decompress_kernel(const uint64_t* __restrict__ index, const uint8_t* __restrict__ area, int64_t M, int64_t N,
+                          int64_t BN, int64_t RB, int64_t nblocks, double* __restrict__ out, int64_t ldo) {
+  __shared__ double turn[VEC ? 1 : 8 * 512];
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nblocks) return;
-  const int64_t I = b / BN, J = b - I * BN, run = J / 32;
+  const bool live = b < nblocks;
+  int64_t I = 0, J = 0;
+  unit_of(live ? b : nblocks - 1, BN, I, J);
+  const int64_t run = J / 32;
   const uint64_t e = index[I * RB + run];
   const int W = (int)(e >> 56);
   int64_t T[16];
@@ -241,13 +245,10 @@ static __global__ void wz3_decompress_kernel(const uint64_t* __restrict__ index,
             T[4 * r + 3] = s2 + x + yv + z;
     }
   }
+  uint2 d[16];
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int64_t gi = 4 * I + r, gj = 4 * J + c;
-      if (gi < M && gj < N) out[gi * ldo + gj] = zero ? 0.0 : ldexp((double)T[4 * r + c], scale_exp);
-    }
+  for (int k = 0; k < 16; ++k) d[k] = zero ? make_uint2(0u, 0u) : f64_from_int(T[k], scale_exp);
+  store_units<VEC, 4, 4>(d, live, I, J, BN, M, N, out, ldo, turn + (VEC ? 0 : (threadIdx.x >> 5) * 512));
 }
 
 }  // namespace dev
