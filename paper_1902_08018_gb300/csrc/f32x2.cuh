@@ -51,5 +51,41 @@ __device__ __forceinline__ void two_sum_acc2(float2& hi, float2& lo, float2 p) {
   lo = add_f2(lo, err);
 }
 
+// The same pairs held as 64-bit registers across a loop.
+using f32p = unsigned long long;
+__device__ __forceinline__ f32p pair_of(float a, float b) {
+  f32p d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ float2 halves_of(f32p a) {
+  float2 d;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(a));
+  return d;
+}
+__device__ __forceinline__ f32p add_p(f32p a, f32p b) {
+  f32p d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32p sub_p(f32p a, f32p b) {
+  f32p d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32p fma_p(f32p a, f32p b, f32p c) {
+  f32p d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+// TwoSum of q s into (hi, lo), s a power of two: the product is exact, so the
+// scaling rides in two of the FMAs (-bp = hi - s' is as exact as bp).
+__device__ __forceinline__ void two_sum_scaled_p(f32p& hi, f32p& lo, f32p q, f32p s) {
+  const f32p t = fma_p(q, s, hi), nbp = sub_p(hi, t);
+  const f32p err = add_p(sub_p(hi, add_p(t, nbp)), fma_p(q, s, nbp));
+  hi = t;
+  lo = add_p(lo, err);
+}
+
 }  // namespace dev
 }  // namespace whff

@@ -66,6 +66,29 @@ __device__ __forceinline__ double warp_sum_pair(float hi, float lo) {
   return (double)hi + (double)lo;
 }
 
+// Totals over the warp of 32 compensated pairs per lane: lane l returns that of
+// pair l.  Each level hands half of the pairs to the partner lane and adds the
+// half that it keeps (TwoSum, as warp_sum_pair), so the 32 totals take 31 pair
+// additions instead of 32 butterflies of five.
+__device__ __forceinline__ double warp_sum_pairs32(float (&hi)[32], float (&lo)[32], int lane) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < o; ++k) {
+      const float h2 = __shfl_xor_sync(0xffffffffu, up ? hi[k] : hi[k + o], o);
+      const float l2 = __shfl_xor_sync(0xffffffffu, up ? lo[k] : lo[k + o], o);
+      const float h = up ? hi[k + o] : hi[k], l = up ? lo[k + o] : lo[k];
+      const float s = h + h2;
+      const float bp = s - h;
+      const float e = (h - (s - bp)) + (h2 - bp);
+      hi[k] = s;
+      lo[k] = (l + l2) + e;
+    }
+  }
+  return (double)hi[0] + (double)lo[0];
+}
+
 // Fold a lane's (hi, lo) sums for 4 rows x R columns and write either the
 // final y (+ state) or the split-K partial.  Deterministic: fixed shuffle tree.
 template <int R>

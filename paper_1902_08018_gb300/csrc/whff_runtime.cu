@@ -74,6 +74,9 @@ struct whff_handle {
   const uint8_t* wz3_area = nullptr;
   int64_t wz3_RB = 0;           // runs per band
   int64_t band0 = 0;            // fixed accuracy: first band of a row view
+  int64_t wz3_L8 = 0;           // fixed accuracy, 8 columns: (group of 8 bands, run) units per CTA
+  int64_t wz3_ctas8 = 0;
+  int wz3_maxseg8 = 1;          // most CTAs sharing one group
   uint32_t wait_polls = whff::kWaitPolls;  // in-loop bounded waits of the tensor-core kernels
   cudaStream_t create_stream = nullptr;
 };
@@ -135,6 +138,22 @@ void choose_ranges(whff_handle* h) {
   h->chunk = U;
 }
 
+// Fixed accuracy, 8 columns: two CTAs per SM share the (group of 8 bands, run)
+// units in equal ranges, fewer where the partials of shared groups would not
+// fit the workspace (one CTA shares nothing).
+void plan_wz3_8(whff_handle* h) {
+  const int64_t RB = ceil_div(h->BN, 32), groups = ceil_div(h->BM, 8), units = groups * RB;
+  for (int64_t ctas = std::min<int64_t>(2 * h->sm_count, units);; ctas = std::max<int64_t>(1, ctas * 3 / 4)) {
+    h->wz3_L8 = ceil_div(units, ctas);
+    h->wz3_ctas8 = ceil_div(units, h->wz3_L8);
+    h->wz3_maxseg8 = 1;
+    for (int64_t G = 0; G < groups; ++G)
+      h->wz3_maxseg8 = std::max<int>(h->wz3_maxseg8,
+                                     (int)(((G + 1) * RB - 1) / h->wz3_L8 - (G * RB) / h->wz3_L8 + 1));
+    if (h->wz3_maxseg8 == 1 || (size_t)h->BM * (size_t)h->wz3_maxseg8 * 32 * 8 <= h->ws_bytes) break;
+  }
+}
+
 void choose_split(whff_handle* h) {
   if (h->info.fmt != WHFF_FMT_ZFP) {  // WZ2, WZ3 and scaled formats: persistent warp ranges
     choose_ranges(h);
@@ -176,9 +195,10 @@ size_t mma_ws_need(const whff_handle* h, int R) {
   return (size_t)ceil_div(h->info.M, 128) * (size_t)h->mma_maxseg * (size_t)R * 128 * 8;
 }
 
-// The lift's transformed x: 4 BN floats per right-hand side of a pass (up to 8).
+// The lift's transformed x: 4 BN floats per right-hand side of a pass (up to 8;
+// fixed accuracy lays it out in whole runs of 32 blocks).
 size_t xt_bytes(const whff_handle* h) {
-  return (size_t)4 * h->BN * std::min(h->max_rhs, kMaxRhsKernel) * sizeof(float);
+  return (size_t)4 * (is_wz3(h->info.fmt) ? 32 * ceil_div(h->BN, 32) : h->BN) * std::min(h->max_rhs, kMaxRhsKernel) * sizeof(float);
 }
 
 // Workspace bytes a CUDA-core pass of the plan needs.
@@ -306,8 +326,10 @@ int launch_pass(const whff_handle* h, const float* x, int R, int64_t ldx, double
       e = launch_scaled(h, x, R, ldx, vec, y, ldy, state, decay, st);
       break;
     case WHFF_FMT_FIXED_ACC: {
+      const bool wide = R == 8;
       Wz3Step a{h->wz3_index, h->wz3_area, h->band0, h->info.M, h->info.N, h->BM, h->BN, h->wz3_RB, x, ldx,
-                h->d_xt, R, h->range_len, h->maxseg, h->range_ctas, h->d_ws, y, ldy, state, decay};
+                h->d_xt, R, wide ? h->wz3_L8 : h->range_len, wide ? h->wz3_maxseg8 : h->maxseg,
+                wide ? h->wz3_ctas8 : h->range_ctas, h->d_ws, y, ldy, state, decay};
       e = wz3_launch(a, st) ? WHFF_EINVAL : WHFF_OK;
       if (e) set_error("whff_step: fixed-accuracy passes take 1 or 8 right-hand sides");
       break;
@@ -457,7 +479,7 @@ int create_impl(const BlobInfo& info, const uint8_t* src, int max_rhs, unsigned 
     const int occ = wz2_occ(info.rate, info.fmt == WHFF_FMT_FIXED_LIFT, h->unroll);
     h->ctas_per_sm = occ > 0 ? occ : 4;
   } else if (is_wz3(info.fmt)) {
-    const int occ = wz3_occupancy(1);
+    const int occ = wz3_occupancy();
     h->ctas_per_sm = occ > 0 ? occ : 4;
   } else if (!is_blocked(info.fmt)) {  // the kernel the fold default below picks
     const int occ = scaled_occupancy(info.fmt, scaled_ld(info.N) / scaled_vec(info.fmt) < 256);
@@ -501,6 +523,7 @@ int create_impl(const BlobInfo& info, const uint8_t* src, int max_rhs, unsigned 
   if (h->maxseg > 1)
     h->ws_bytes = (size_t)h->BM * (size_t)h->maxseg * (size_t)std::min(max_rhs, kMaxRhsKernel) * 4 * 8;
   h->ws_rhs = std::min(max_rhs, kMaxRhsKernel);
+  if (is_wz3(info.fmt)) plan_wz3_8(h);
   const bool wz2 = info.fmt == WHFF_FMT_FIXED_LIFT || info.fmt == WHFF_FMT_FIXED_BFP;
   const bool scaled16 = info.fmt == WHFF_FMT_BF16 || info.fmt == WHFF_FMT_FP16 || info.fmt == WHFF_FMT_FP8E4M3;
   if ((wz2 || scaled16) && max_rhs >= 2) {
@@ -688,6 +711,7 @@ int step_view(const whff_handle* h, int64_t row0, int64_t nrows, const float* x,
     v.ctas_per_sm = --c;
     choose_ranges(&v);
   }
+  if (is_wz3(fmt)) plan_wz3_8(&v);
   if (h->d_ws_mma) {
     int64_t ctas = (int64_t)h->sm_count * h->mma_occ;
     for (plan_mma(&v, ctas); mma_ws_need(&v, std::min(R, 32)) > h->ws_mma_cap && ctas > 1;

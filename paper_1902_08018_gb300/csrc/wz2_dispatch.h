@@ -160,9 +160,10 @@ int scaled_tma_map(void* out, const void* payload, int64_t M, int64_t ld, int fm
 // resident CTAs per SM for R <= 32 (0 on error); tma: the TMA-fed BF16 kernel
 int scaled_mma_occupancy(int fmt, bool tma);
 
-// Fixed-accuracy (WZ3) pass: (2G)^T x, then persistent warp ranges of L runs
-// over the pass's bands in band-major order, then (maxseg > 1) the segment
-// epilogue for bands shared by several ranges.  band0 is the first band of a
+// Fixed-accuracy (WZ3) pass: (2G)^T x, then persistent ranges (R = 1: a warp's,
+// of L runs of the pass's bands in band-major order; R = 8: a CTA's, of L
+// (group of 8 bands, run) units), then (maxseg > 1) the epilogue for bands
+// shared by several ranges.  band0 is the first band of a
 // row view within the matrix (its index is the matrix's).
 struct Wz3Step {
   const uint64_t* index;  // the matrix's run index (BM_total x RB)
@@ -173,7 +174,7 @@ struct Wz3Step {
   int64_t ldx;
   float* xt;  // scratch: (2G)^T x, 4 BN floats per right-hand side
   int R;      // 1 or 8
-  int64_t L;      // runs per warp range
+  int64_t L;      // R = 1: runs per warp range; R = 8: (group of 8 bands, run) units per CTA
   int maxseg;     // most ranges sharing one band
   int64_t ctas;   // grid size
   double* ws;     // BM x maxseg x R x 4 segment partials when maxseg > 1
@@ -183,7 +184,7 @@ struct Wz3Step {
   double decay;
 };
 int wz3_launch(const Wz3Step& a, cudaStream_t st);
-int wz3_occupancy(int R);  // resident CTAs per SM of the R-column kernel (0 on error)
+int wz3_occupancy();  // resident CTAs per SM of the R = 1 kernel (0 on error)
 int wz3_decompress(const uint64_t* index, const uint8_t* area, int64_t M, int64_t N, double* out, int64_t ldo,
                    cudaStream_t st);
 

@@ -79,7 +79,17 @@ __device__ __forceinline__ void wz3_load_run(const uint8_t* __restrict__ area, u
   const int W = (int)(e >> 56);
   const int nw = wz3_block_bytes(W) / 8;  // 64-bit words of a block (uniform over the warp)
   const uint2* p = reinterpret_cast<const uint2*>(area + (e & 0x00FFFFFFFFFFFFFFull)) + lane;
-  if (active && W != 0) {
+  if (nb == 32) {  // a whole run: constant offsets
+    if (W != 0) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k < nw) {
+          const uint2 v = __ldcs(p + k * 32);
+          w[2 * k] = v.x;
+          w[2 * k + 1] = v.y;
+        }
+    }
+  } else if (active && W != 0) {
 #pragma unroll
     for (int k = 0; k < 8; ++k)
       if (k < nw) {
@@ -95,31 +105,31 @@ __device__ __forceinline__ void wz3_load_run(const uint8_t* __restrict__ area, u
 // chunk J, ldt floats per column), then hi/lo[i][r] += p_i by TwoSum.  Rows
 // (0, 1) and (2, 3) go in packed FP32 pairs; each half rounds as the scalar
 // chain (product, three FMAs in b order, the scale, TwoSum) would.
-template <int R>
-__device__ __forceinline__ void wz3_accumulate(const uint32_t (&w)[16], int W, const float* __restrict__ xt,
-                                               int64_t ldt, int J, float (&hi)[4][R], float (&lo)[4][R]) {
+// wz3_values gives V[h][b] = (value (2h, b), value (2h + 1, b)) and s.
+__device__ __forceinline__ void wz3_values(const uint32_t (&w)[16], int W, float2 (&V)[2][4], float& s) {
   uint32_t t[16];
   wz3_fields_w(W, w, t);
-  float2 V[2][4];  // V[h][b] = (value (2h, b), value (2h + 1, b))
-  if (W <= 23) {  // exact: (2^23 + field) - (2^23 + 2^(W-1))
-    const float bias = 8388608.0f + (float)(1u << (W - 1));
-    const float2 b2 = make_float2(bias, bias);
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-      for (int b = 0; b < 4; ++b)
-        V[h][b] = sub_f2(make_float2(__uint_as_float(t[8 * h + b]), __uint_as_float(t[8 * h + 4 + b])), b2);
-  } else {  // the integer conversion, round to nearest
+  // exact: (2^23 + field) - (2^23 + 2^(W-1))
+  float bias = 8388608.0f + (float)(1u << (W - 1));
+  if (W > 23) {  // the integer conversion, round to nearest
     const uint32_t half = 1u << (W - 1);
+    bias = 0.f;
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-      for (int b = 0; b < 4; ++b)
-        V[h][b] = make_float2(__int2float_rn((int32_t)(t[8 * h + b] - half)),
-                              __int2float_rn((int32_t)(t[8 * h + 4 + b] - half)));
+    for (int k = 0; k < 16; ++k) t[k] = __float_as_uint(__int2float_rn((int32_t)(t[k] - half)));
   }
+  const float2 b2 = make_float2(bias, bias);
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+      V[h][b] = sub_f2(make_float2(__uint_as_float(t[8 * h + b]), __uint_as_float(t[8 * h + 4 + b])), b2);
   const uint32_t E = w[0] & 0xFFu, K = (w[0] >> 8) & 31u;
-  const float s = E ? __uint_as_float((E + K - 27u) << 23) : 0.f;  // 2^(E+K-154); E >= 28 for a nonzero block
+  s = E ? __uint_as_float((E + K - 27u) << 23) : 0.f;  // 2^(E+K-154); E >= 28 for a nonzero block
+}
+
+template <int R>
+__device__ __forceinline__ void wz3_accumulate(const float2 (&V)[2][4], float s, const float* __restrict__ xt,
+                                               int64_t ldt, int J, float (&hi)[4][R], float (&lo)[4][R]) {
   const float2 s2 = make_float2(s, s);
 #pragma unroll
   for (int r = 0; r < R; ++r) {
@@ -147,7 +157,7 @@ __device__ __forceinline__ void wz3_accumulate(const uint32_t (&w)[16], int W, c
 // ws[(I maxseg + seg) R + r][4] for the segment epilogue.  The index entry of
 // the next run is read while the lanes decode the current one.
 template <int R>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? 4 : 1)
+__global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
     wz3_gemv_kernel(const uint64_t* __restrict__ index, const uint8_t* __restrict__ area, int64_t M, int64_t BM,
                     int BN, int RB, const float* __restrict__ xt, int64_t ldt, int64_t L, int maxseg,
                     double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
@@ -175,7 +185,12 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? 4 : 1)
       const int W = (int)(e >> 56);
       uint32_t w[16];
       wz3_load_run(area, e, lane, nb, lane < nb, w);
-      if (W != 0 && lane < nb) wz3_accumulate<R>(w, W, xt, ldt, 32 * q + lane, hi, lo);  // a zero run adds 0
+      if (W != 0 && lane < nb) {  // a zero run adds 0
+        float2 V[2][4];
+        float s;
+        wz3_values(w, W, V, s);
+        wz3_accumulate<R>(V, s, xt, ldt, 32 * q + lane, hi, lo);
+      }
     }
     const int64_t g_lo = (I * RB) / L, g_hi = ((I + 1) * RB - 1) / L;
     if (g_lo == g_hi)
@@ -190,6 +205,165 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? 4 : 1)
     ++I;
     ub = ue;
   }
+}
+
+// Eight right-hand sides: the x of a block is 128 bytes, three times its stored
+// bits, so what x costs decides.  The eight warps of a CTA take the same runs of
+// eight neighbouring bands side by side and share the x chunks through L1; with
+// a range of one band after another to each warp every x chunk came from L2
+// (8.6 GB a pass at 32768^2).  CTA c takes units [c L, c L + L) of the sequence
+// (group of 8 bands, run), group-major; warp w the group's band w.
+// The chain of a row takes scalar FMAs (their operands need no doubling into
+// pairs; a packed instruction takes two issue cycles of the FMA pipe anyway), the
+// TwoSum packed ones on rows 2h and 2h + 1.
+// The 32 sums of a band (r, i) are folded over the lanes by warp_sum_pairs32,
+// lane 4 r + i ending with that of row i and column r: FP64 butterflies cost
+// 2600 cycles of GB300's FP64 pipe per band piece.
+// 8192^2 at 1e-7 (0.18 GB, one pass of 8 columns): 269 us and 12 us of segment
+// epilogue with warp ranges and FP64 folds, 105 us and 4 us this way, at 56 % of
+// the issue slots; the FMA pipe (128 FMAs and 96 packed ones per 32 blocks, and
+// the moves between them) is what bounds it now, at 57 us of pipe time.
+
+// (2G)^T x of 8 columns as the kernel reads it: for run q and column r the run's
+// 32 blocks, 16 bytes each, xt[((q 8 + r) 32 + block) 4 + b], so that every load
+// of a warp is 512 bytes in a row at a constant offset.  Thread per (q, r,
+// block); blocks past the last one get zeros.  The same FP32 operations as
+// wz2_xt_kernel.
+static __global__ void wz3_xt8_kernel(const float* __restrict__ x, int64_t ldx, int64_t N, int64_t RB,
+                                      float* __restrict__ xt) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= RB * 256) return;
+  const int blk = (int)t & 31, r = (int)(t >> 5) & 7;
+  const int64_t q = t >> 8, col = 4 * (32 * q + blk);
+  const float* xr = x + r * ldx + col;
+  float xv[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) xv[c] = col + c < N ? xr[c] : 0.f;
+  const float a = xv[0] + xv[1], b = xv[2] + xv[3], c = xv[0] + xv[2], d = xv[1] + xv[3];
+  reinterpret_cast<float4*>(xt)[t] = make_float4(2.f * (a + b), b - a, d - c, xv[3] - xv[2]);
+}
+
+// A block's products into the sums of 8 columns, hi/lo[h][r] the rows (2h, 2h + 1):
+// the chain of wz3_accumulate.  xq: the lane's block in the run's part of the x
+// that wz3_xt8_kernel lays out.
+__device__ __forceinline__ void wz3_accumulate8(const float2 (&V)[2][4], float s, const float* __restrict__ xq,
+                                                f32p (&hi)[2][8], f32p (&lo)[2][8]) {
+  const f32p s2 = pair_of(s, s);
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const float4 x = __ldg(reinterpret_cast<const float4*>(xq + 128 * r));
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float a = V[h][0].x * x.x, b = V[h][0].y * x.x;
+      a = fmaf(V[h][1].x, x.y, a), b = fmaf(V[h][1].y, x.y, b);
+      a = fmaf(V[h][2].x, x.z, a), b = fmaf(V[h][2].y, x.z, b);
+      a = fmaf(V[h][3].x, x.w, a), b = fmaf(V[h][3].y, x.w, b);
+      two_sum_scaled_p(hi[h][r], lo[h][r], pair_of(a, b), s2);
+    }
+  }
+}
+
+// Bring the run of index entry e to L2: a lane per 128-byte line.
+__device__ __forceinline__ void wz3_prefetch_run(const uint8_t* __restrict__ area, uint64_t e, int lane, int nb) {
+  const uint32_t bytes = (uint32_t)(nb * wz3_block_bytes((int)(e >> 56)));
+  const uint8_t* p = area + (e & 0x00FFFFFFFFFFFFFFull);
+  if (128 * (uint32_t)lane < bytes) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 128 * lane));
+}
+
+__device__ __forceinline__ int64_t wz3_groups(int64_t BM) { return (BM + 7) / 8; }
+
+// The lane's total z of (r, i), lane = 4 r + i, mixed with 2G over the rows
+// (lanes 4 r .. 4 r + 3): y of row i.
+__device__ __forceinline__ double wz3_mix_rows(double z, int lane) {
+  const int q = lane & ~3, i = lane & 3;
+  const double z0 = __shfl_sync(0xffffffffu, z, q), z1 = __shfl_sync(0xffffffffu, z, q + 1),
+               z2 = __shfl_sync(0xffffffffu, z, q + 2), z3 = __shfl_sync(0xffffffffu, z, q + 3);
+  double t = 2.0 * z0;
+  t = i < 2 ? t - z1 : t + z1;
+  t = i & 1 ? t + z2 : t - z2;
+  if (i >= 2) t = i == 2 ? t - z3 : t + z3;
+  return t * 0.125;
+}
+
+// y (and the state, column by column) of one band from its 32 totals.
+__device__ __forceinline__ void wz3_write_band8(double t, int lane, int64_t I, int64_t M, double* __restrict__ y,
+                                                int64_t ldy, double* __restrict__ state, double decay) {
+  const int64_t row = 4 * I + (lane & 3);
+  if (row < M) y[(int64_t)(lane >> 2) * ldy + row] = t;
+  if (state) {
+    double s = lane < 4 && row < M ? state[row] : 0.0;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) s = decay * s + __shfl_sync(0xffffffffu, t, 4 * r + (lane & 3));
+    if (lane < 4 && row < M) state[row] = s;
+  }
+}
+
+static __global__ void __launch_bounds__(kWarpsPerCta * 32, 2)
+    wz3_gemv8_kernel(const uint64_t* __restrict__ index, const uint8_t* __restrict__ area, int64_t M, int64_t BM,
+                     int BN, int RB, const float* __restrict__ xt, int64_t L, int maxseg, double* __restrict__ ws,
+                     double* __restrict__ y, int64_t ldy, double* __restrict__ state, double decay) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t u0 = (int64_t)blockIdx.x * L, u1 = min(wz3_groups(BM) * RB, u0 + L);
+  for (int64_t ub = u0; ub < u1;) {  // the range's piece of group G: runs [q0, q1) of each of its bands
+    const int64_t G = ub / RB, ue = min(u1, (G + 1) * RB);
+    const int q0 = (int)(ub - G * RB), q1 = (int)(ue - G * RB);
+    ub = ue;
+    const int64_t I = 8 * G + warp;
+    if (I >= BM) continue;  // whole warp
+    f32p hi[2][8], lo[2][8];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int r = 0; r < 8; ++r) hi[h][r] = lo[h][r] = 0;
+    const uint64_t* idx = index + I * RB;
+    uint64_t e0 = __ldg(idx + q0), e1 = __ldg(idx + min(q0 + 1, q1 - 1)), e2 = __ldg(idx + min(q0 + 2, q1 - 1));
+#pragma unroll 1
+    for (int q = q0; q < q1; ++q) {
+      const uint64_t e = e0;
+      e0 = e1, e1 = e2;
+      wz3_prefetch_run(area, e1, lane, min(32, BN - 32 * min(q + 2, q1 - 1)));
+      e2 = __ldg(idx + min(q + 3, q1 - 1));
+      const int W = (int)(e >> 56), left = BN - 32 * q;
+      if (W == 0 || lane >= left) continue;  // a zero run adds 0
+      uint32_t w[16];
+      wz3_load_run(area, e, lane, min(32, left), true, w);
+      float2 V[2][4];
+      float s;
+      wz3_values(w, W, V, s);
+      wz3_accumulate8(V, s, xt + 1024 * (int64_t)q + 4 * lane, hi, lo);
+    }
+    __syncwarp();
+    float h[32], l[32];
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const float2 a = halves_of(hi[k][r]), b = halves_of(lo[k][r]);
+        h[4 * r + 2 * k] = a.x, h[4 * r + 2 * k + 1] = a.y;
+        l[4 * r + 2 * k] = b.x, l[4 * r + 2 * k + 1] = b.y;
+      }
+    const double t = wz3_mix_rows(warp_sum_pairs32(h, l, lane), lane);
+    const int64_t c_lo = (G * RB) / L, c_hi = ((G + 1) * RB - 1) / L;
+    if (c_lo == c_hi)
+      wz3_write_band8(t, lane, I, M, y, ldy, state, decay);
+    else
+      ws[(I * maxseg + (blockIdx.x - c_lo)) * 32 + lane] = t;
+  }
+}
+
+// The bands of groups shared by several CTAs: their segments added in order.
+// A warp per (range boundary, band of the group it cuts); the first boundary
+// inside a group does the work.
+static __global__ void __launch_bounds__(256)
+    wz3_epilogue8_kernel(const double* __restrict__ ws, int64_t M, int64_t BM, int64_t RB, int64_t L, int maxseg,
+                         double* __restrict__ y, int64_t ldy, double* __restrict__ state, double decay) {
+  const int lane = threadIdx.x & 31;
+  const int64_t c = 1 + (int64_t)blockIdx.x, b = c * L;
+  const int64_t G = b / RB, I = 8 * G + (threadIdx.x >> 5);
+  if (b >= wz3_groups(BM) * RB || b % RB == 0 || (c - 1) * L > G * RB || I >= BM) return;
+  const int64_t c_lo = (G * RB) / L, c_hi = ((G + 1) * RB - 1) / L;
+  const double t = seq_sum_strided(ws + I * maxseg * 32 + lane, c_hi - c_lo + 1, 32);
+  wz3_write_band8(t, lane, I, M, y, ldy, state, decay);
 }
 
 // Decode: thread per block, the exact definition -- T = (2G) V (2G)^T in
