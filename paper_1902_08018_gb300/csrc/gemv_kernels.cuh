@@ -143,14 +143,25 @@ __device__ __forceinline__ float4 load_x4(const float* __restrict__ x, int64_t l
 }
 
 // --------------------------------------------------------------- WZ1 GEMV
+// Four warps to a block of the embedded coder's kernels: the SMs' shares of a
+// grid differ by less than with eight (10000^2 in three splits: 12.4 blocks per
+// SM, not 6.2), 36 warps fit an SM, and rate 64 fits 48 KB of shared memory.
+// wz1_gemv_kernel, rate 16, 10000^2 (0.2 GB), one column: 451 us with a group
+// test per iteration; 268 us with table lookups; 241 us with whole planes two at
+// a time and four-warp blocks.  1026 warp instructions per 32 blocks, bound by
+// the integer pipe (74 % busy): the parse about half of them, the bit transpose,
+// lift and products the rest.
+constexpr int kWz1Threads = 128;
 template <int NW32, int R>
-__global__ void __launch_bounds__(kWarpsPerCta * 32)
+__global__ void __launch_bounds__(kWz1Threads)
     wz1_gemv_kernel(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM, int64_t BN,
                     const float* __restrict__ x, int64_t ldx, bool x_vec_ok, int ksplit, int64_t jchunk,
                     double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
                     double decay) {
+  __shared__ Wz1Smem<NW32, kWz1Threads> sm;
+  wz1_smem_init(sm);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t I = (int64_t)blockIdx.x * kWarpsPerCta + warp;
+  const int64_t I = (int64_t)blockIdx.x * (kWz1Threads / 32) + warp;
   if (I >= BM) return;  // whole warp
   const int split = blockIdx.y;
   const int64_t J0 = (int64_t)split * jchunk;
@@ -162,15 +173,17 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32)
 #pragma unroll
     for (int r = 0; r < R; ++r) hi[i][r] = lo[i][r] = 0.f;
 
-  __shared__ uint32_t planes[kPlaneWords];  // the decoder's plane words, a column per thread
-  uint32_t* Ps = planes + threadIdx.x;
   const int64_t rowblk = I * BN;
+  uint32_t next[NW32];
+  if (J0 + lane < J1) load_block<NW32>(stream, rowblk + J0 + lane, next);
   for (int64_t J = J0 + lane; J < J1; J += 32) {
-    uint32_t w[NW32 + 2];
-    load_block<NW32>(stream, rowblk + J, w);
+    uint32_t w[NW32];
+#pragma unroll
+    for (int i = 0; i < NW32; ++i) w[i] = next[i];
+    if (J + 32 < J1) load_block<NW32>(stream, rowblk + J + 32, next);  // on its way while this one is decoded
     int32_t q[16];
     int emax;
-    const bool nz = decode_block<NW32>(w, Ps, q, emax);
+    const bool nz = decode_block(w, sm, q, emax);
     if (!nz) continue;
     const float scale = __int_as_float((emax - 26 + 127) << 23);  // 2^(emax-26), a normal float
     float a[16];
@@ -281,26 +294,27 @@ static __global__ void splitk_epilogue_kernel(const double* __restrict__ ws, int
 // ------------------------------------------------------------- decode only
 // Thread per block (WZ1) or per 16-byte chunk (scaled); results as decode_out.cuh says.
 template <int NW32, bool VEC>
-__global__ void __launch_bounds__(kDecodeThreads)
+__global__ void __launch_bounds__(kWz1Threads)
     wz1_decompress_kernel(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BN, int64_t nblocks,
                           double* __restrict__ out, int64_t ldo) {
-  __shared__ __align__(16) uint32_t planes[kPlaneWords];  // the decoder's plane words, a column per thread
+  using Smem = Wz1Smem<NW32, kWz1Threads>;
+  __shared__ __align__(16) Smem sm;
+  static_assert(sizeof(Smem) >= (kWz1Threads / 32) * 512 * 8, "turns the rows round: 4 x 128 doubles a warp");
+  wz1_smem_init(sm);
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool live = b < nblocks;
   int64_t I = 0, J = 0;
   unit_of(live ? b : nblocks - 1, BN, I, J);
-  uint2 d[16];
-  uint32_t w[NW32 + 2];
+  uint32_t w[NW32];
   load_block<NW32>(stream, live ? b : nblocks - 1, w);
   int32_t q[16];
   int emax;
-  (void)decode_block<NW32>(w, planes + threadIdx.x, q, emax);  // a zero block's q are zeros
+  const bool nz = decode_block(w, sm, q, emax);
+  uint2 d[16];
 #pragma unroll
-  for (int k = 0; k < 16; ++k) d[k] = f64_from_f32(__int2float_rn(q[k]), emax - 26);
-  if constexpr (!VEC) __syncthreads();  // the plane words have been read: their memory turns the rows round
-  static_assert(kPlaneWords * 4 >= (kDecodeThreads / 32) * 512 * 8, "a warp's 4 x 128 doubles each");
-  store_units<VEC, 4, 4>(d, live, I, J, BN, M, N, out, ldo,
-                         reinterpret_cast<double*>(planes) + (threadIdx.x >> 5) * 512);
+  for (int k = 0; k < 16; ++k) d[k] = nz ? f64_from_f32(__int2float_rn(q[k]), emax - 26) : make_uint2(0u, 0u);
+  if constexpr (!VEC) __syncthreads();  // the decoder's words have been read
+  store_units<VEC, 4, 4>(d, live, I, J, BN, M, N, out, ldo, reinterpret_cast<double*>(&sm) + (threadIdx.x >> 5) * 512);
 }
 
 template <int FMT, bool VEC>

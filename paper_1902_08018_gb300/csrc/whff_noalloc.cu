@@ -68,8 +68,9 @@ template <int NW32, int R>
 void launch(const uint8_t* s, int64_t M, int64_t N, int64_t BM, int64_t BN, const float* x, int64_t ldx, bool vec,
             int ksplit, int64_t chunk, double* ws, double* y, int64_t ldy, double* state, double decay,
             cudaStream_t st) {
-  dim3 grid((unsigned)((BM + whff::dev::kWarpsPerCta - 1) / whff::dev::kWarpsPerCta), (unsigned)ksplit);
-  whff::dev::wz1_gemv_kernel<NW32, R><<<grid, whff::dev::kWarpsPerCta * 32, 0, st>>>(
+  constexpr int kWarps = whff::dev::kWz1Threads / 32;
+  dim3 grid((unsigned)((BM + kWarps - 1) / kWarps), (unsigned)ksplit);
+  whff::dev::wz1_gemv_kernel<NW32, R><<<grid, whff::dev::kWz1Threads, 0, st>>>(
       s, M, N, BM, BN, x, ldx, vec, ksplit, chunk, ws, y, ldy, state, decay);
 }
 

@@ -211,8 +211,8 @@ size_t ws_need(const whff_handle* h) {
 template <int NW32>
 int launch_wz1_nw(const whff_handle* h, const float* x, int R, int64_t ldx, bool vec, double* y, int64_t ldy,
                   double* state, double decay, cudaStream_t st) {
-  dim3 grid((unsigned)((h->BM + dev::kWarpsPerCta - 1) / dev::kWarpsPerCta), (unsigned)h->ksplit);
-  dim3 block(dev::kWarpsPerCta * 32);
+  dim3 grid((unsigned)ceil_div(h->BM, dev::kWz1Threads / 32), (unsigned)h->ksplit);
+  dim3 block(dev::kWz1Threads);
   const uint8_t* s = h->d_stream;
   const auto& b = h->info;
 #define WZ1_CASE(RR)                                                                                      \
@@ -1053,6 +1053,7 @@ extern "C" int whff_decompress(whff_handle* h, double* out, int64_t ldo, void* s
   const bool vec = dev::out_vec_ok(out, ldo);  // 32-byte stores
   if (b.fmt == WHFF_FMT_ZFP) {
     const int64_t nb = h->BM * h->BN;
+    const int threads = dev::kWz1Threads;
     const unsigned grid = (unsigned)((nb + threads - 1) / threads);
 #define DZ(R_)                                                                                          \
   case R_:                                                                                              \

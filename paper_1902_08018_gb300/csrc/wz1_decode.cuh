@@ -6,6 +6,16 @@
 // coefficient implied) -> 32x16 bit-matrix transpose of the plane words into
 // one word per coefficient -> negabinary to two's complement -> inverse lift
 // (columns, then rows; mod 2^32, arithmetic shifts) -> 16 int32 values q.
+//
+// The parse is a chain of data-dependent steps that the 32 lanes of a warp take
+// at different places, so what counts is warp iterations: one table lookup
+// takes ten stream bits of a plane's group tests at once (nearly every plane is
+// one lookup, whatever the lane's bits are), and once every lane's coefficients
+// are all significant the rest is 16-bit planes, two to a 32-bit window.  The
+// stream words and the plane words sit in shared memory, a column per thread (a
+// lane's own index never conflicts).  One group test per iteration, 19 of 32
+// lanes active, took 1881 warp instructions per 32 blocks at rate 16 (10000^2: 451 us,
+// now 241; see wz1_gemv_kernel).
 // The decoded matrix entry is (float)q * 2^(emax-26) (round to nearest even).
 //
 // Sec. 5.2 observes that zfp decoding is sequential within a stream and that
@@ -37,129 +47,182 @@ __device__ __forceinline__ void inv_lift(uint32_t& a, uint32_t& b, uint32_t& c, 
   d = d1 + c;
 }
 
-// Delta swap of bit groups between two words of a bit matrix.
+// Swap of bit groups between two words of a bit matrix (s = 1, 2, 4; m the low
+// group of each pair): a keeps its low groups and takes b's low ones above them.
 __device__ __forceinline__ void dswap(uint32_t& a, uint32_t& b, int s, uint32_t m) {
-  uint32_t t = ((a >> s) ^ b) & m;
-  b ^= t;
-  a ^= t << s;
+  const uint32_t hi = a >> s;
+  a = (a & m) | ((b << s) & ~m);
+  b = (hi & m) | (b & ~m);
 }
 
-// Decode the plane stream (starting after the 9 header bits) of one block
-// whose NW32 little-endian 32-bit words are in w[0..NW32) followed by two zero
-// words.  Returns the 16 negabinary words u[k] in sequency order.
-//
-// The plane loop is not unrolled (one small loop body instead of 32 copies:
-// the unrolled form spent its time on instruction-cache misses), so the plane
-// words go to the thread's own column of a shared-memory array, Ps[j * ps]
-// for plane kmax - j, and come back for the bit-matrix transpose.
-template <int NW32>
-__device__ __forceinline__ void decode_planes(const uint32_t (&w)[NW32 + 2], uint32_t* __restrict__ Ps, int ps,
-                                              uint32_t (&u)[16]) {
-  constexpr int kMaxBits = 16 * NW32 * 2 - 9;  // 16*rate - 9, rate = 2*NW32
-  uint64_t win = ((uint64_t)w[1] << 32 | w[0]) >> 9;
-  int avail = 55;  // valid bits in win
-  int widx = 2;    // next word to append
-  int bits = kMaxBits;
-  auto refill = [&]() {
-    if (avail <= 32) {
-      win |= (uint64_t)w[widx] << avail;
-      ++widx;
-      avail += 32;
-    }
-  };
-  auto skip = [&](int c) {
-    win >>= c;
-    avail -= c;
-    bits -= c;
-  };
-
-  // Leading empty planes (a single zero group test each, while nothing is
-  // significant yet).  kmax = the first plane with a positive test.
-  int z0 = (uint32_t)win ? __ffs((uint32_t)win) - 1 : 32;
-  z0 = min(z0, bits);
-  skip(z0);
-  const int kmax = 31 - z0;
-
-  int n = 0, j = 0;
-#pragma unroll 1
-  for (; j <= kmax && bits > 0; ++j) {
-    refill();
-    const int m = min(n, bits);
-    uint32_t p = (uint32_t)win & ((1u << m) - 1u);
-    skip(m);
-#pragma unroll 1
-    while (n < 16 && bits > 0) {
-      refill();
-      const uint32_t v = (uint32_t)win;
-      if (!(v & 1u)) {  // negative group test: plane done
-        skip(1);
-        break;
-      }
-      const int avl = bits - 1;  // bits left after the test bit
-      const int run = 15 - n;    // explicit positions n..14 (15 is implied)
-      const uint32_t rest = v >> 1;
-      const int z = rest ? __ffs(rest) - 1 : 31;
-      if (z < run) {
-        if (z + 1 <= avl) {
-          p |= 1u << (n + z);
-          n += z + 1;
-          skip(z + 2);
-          continue;
-        }
-        skip(1 + avl);  // budget ends inside the zero run
-        break;
-      }
-      if (run <= avl) {  // positions n..14 zero, 15 implied one
-        p |= 1u << 15;
-        n = 16;
-        skip(1 + run);
+// Group tests of a plane, kTestBits stream bits at a time.  A plane's tests read
+// T S..S T S..S T ...: a test bit T (0 ends the plane), then one bit S per
+// position up to and including the first one.  The entry of (state, bits), the
+// state being before a T (0) or inside an S run (1): bits 0-11 the S bits in
+// order, 12 stopped inside an S run, 13 a zero T was met, byte 2 the stream bits
+// taken, byte 3 the number of S bits.
+constexpr int kTestBits = 10;
+constexpr int kTestEntries = 2 << kTestBits;
+constexpr uint32_t kInScan = 1u << 12, kPlaneDone = 1u << 13;
+struct TestTable {
+  uint32_t e[kTestEntries];
+};
+constexpr TestTable make_test_table() {
+  TestTable t{};
+  for (int i = 0; i < kTestEntries; ++i) {
+    bool scan = i >> kTestBits, end = false;
+    uint32_t out = 0, cnt = 0, pos = 0;
+    while (pos < (uint32_t)kTestBits && !end) {
+      const bool bit = (i >> pos) & 1;
+      ++pos;
+      if (!scan) {
+        scan = bit;
+        end = !bit;
       } else {
-        skip(1 + avl);
+        if (bit) out |= 1u << cnt;
+        ++cnt;
+        scan = !bit;
       }
-      break;
     }
-    Ps[j * ps] = p;
+    t.e[i] = out | (scan && !end ? kInScan : 0u) | (end ? kPlaneDone : 0u) | pos << 16 | cnt << 24;
+  }
+  return t;
+}
+static __device__ const TestTable kTestTable = make_test_table();
+
+// Shared memory of a block of TH threads decoding NW32-word blocks: per thread a
+// column of stream words (two zero words follow) and one of 16 plane pairs
+// (plane k in half k % 2 of word k / 2), and the table.
+template <int NW32, int TH>
+struct Wz1Smem {
+  uint32_t words[(NW32 + 2) * TH];
+  uint32_t planes[16 * TH];
+  uint32_t table[kTestEntries];
+};
+
+// Once per block, before the first decode; ends with a barrier.
+template <int NW32, int TH>
+__device__ __forceinline__ void wz1_smem_init(Wz1Smem<NW32, TH>& sm) {
+  for (int i = threadIdx.x; i < kTestEntries; i += TH) sm.table[i] = kTestTable.e[i];
+  sm.words[NW32 * TH + threadIdx.x] = sm.words[(NW32 + 1) * TH + threadIdx.x] = 0u;
+  __syncthreads();
+}
+
+// 32 stream bits from bit pos on (pos < 32 (NW32 + 1)); zeros past the block.
+template <int TH>
+__device__ __forceinline__ uint32_t wz1_window(const uint32_t* __restrict__ words, int pos) {
+  const uint32_t* p = words + (pos >> 5) * TH;
+  return __funnelshift_r(p[0], p[TH], pos);
+}
+
+// Decode the plane stream (after the 9 header bits) of the block whose words
+// are w: the 16 negabinary words u[k] in sequency order.  Bits past the budget
+// read as zeros, which end a plane as the budget does; only the implied last
+// coefficient has to look at the budget itself.
+template <int NW32, int TH>
+__device__ __forceinline__ void decode_planes(const uint32_t (&w)[NW32], Wz1Smem<NW32, TH>& sm, uint32_t (&u)[16]) {
+  constexpr int kEnd = 32 * NW32;  // 16*rate bits, rate = 2*NW32
+  uint32_t* words = sm.words + threadIdx.x;
+  uint32_t* planes = sm.planes + threadIdx.x;
+#pragma unroll
+  for (int i = 0; i < NW32; ++i) words[i * TH] = w[i];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) planes[i * TH] = 0u;
+  auto put = [&](int k, uint32_t p) {  // plane k
+    reinterpret_cast<uint16_t*>(planes + (k >> 1) * TH)[k & 1] = (uint16_t)p;
+  };
+
+  // leading empty planes: a zero test each, while nothing is significant yet
+  const uint32_t lead = wz1_window<TH>(words, 9);
+  const int z0 = lead ? __ffs(lead) - 1 : 32;
+  int pos = 9 + z0, k = 31 - z0, n = 0;
+#pragma unroll 1
+  for (; n < 16 && k >= 0 && pos < kEnd; --k) {  // n: coefficients significant so far
+    const uint32_t win = wz1_window<TH>(words, pos);
+    uint32_t p = win & ((1u << n) - 1u), src = win >> n;
+    pos += n;
+    int scan = 0;
+#pragma unroll 1
+    for (;;) {
+      const uint32_t e = sm.table[(scan << kTestBits) | (src & ((1u << kTestBits) - 1u))];
+      const int cnt = (int)(e >> 24), run = 15 - n;  // positions n..14 have bits of their own
+      uint32_t out = e & 0xFFFu;
+      if (cnt > run || (cnt == run && (e & kInScan))) {  // the scan went past position 14: 15 is implied
+        out &= (1u << run) - 1u;
+        pos += run + __popc(out) + (1 - scan);
+        p |= out << n;
+        if (pos <= kEnd) p |= 1u << 15;
+        n = 16;
+        break;
+      }
+      p |= out << n;
+      n += cnt;
+      pos += (int)((e >> 16) & 255u);
+      if (e & kPlaneDone) break;
+      scan = e & kInScan ? 1 : 0;
+      src = wz1_window<TH>(words, pos);
+    }
+    put(k, p);
+  }
+  if (!(k & 1) && k >= 0 && pos < kEnd) {  // whole planes: an even one alone ...
+    put(k, wz1_window<TH>(words, pos));
+    --k, pos += 16;
+  }
+  if (k >= 0 && pos < kEnd) {  // ... then (k, k - 1), one word of the stream and one of the planes at a time
+    const uint32_t* src = words + (pos >> 5) * TH;
+    uint32_t* dst = planes + (k >> 1) * TH;
+    const uint32_t* last = src + (min(k >> 1, (kEnd - 1 - pos) >> 5)) * TH;
+    uint32_t lo = *src;
+#pragma unroll 1
+    for (;;) {
+      const uint32_t hi = src[TH];
+      *dst = __byte_perm(__funnelshift_r(lo, hi, pos), 0u, 0x1032);
+      if (src == last) break;
+      lo = hi, src += TH, dst -= TH;
+    }
   }
 
-  // Transpose the 32 (plane) x 16 (coefficient) bit matrix: A[i] bit j = P[j] bit i
-  // (planes past the last decoded one are zero).
-  uint32_t P[32];
-#pragma unroll
-  for (int k = 0; k < 32; ++k) P[k] = k < j ? Ps[k * ps] : 0u;
+  // Transpose the 32 (plane) x 16 (coefficient) bit matrix: bit k of u[i] = bit
+  // i of plane k.  The index bits of word (w3 w2 w1 w0) and bit (b4 .. b0), at
+  // first plane (k4 k3 k2 k1) and (k0, c3 c2 c1 c0), are exchanged w3-b4, w3-b0,
+  // w2-b3, w1-b2, w0-b1; coefficient (c3 c2 c1 c0) ends in word (c0 c3 c2 c1).
   uint32_t A[16];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) A[i] = __byte_perm(P[i], P[i + 16], 0x5410);
+  for (int i = 0; i < 16; ++i) A[i] = planes[i * TH];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) dswap(A[k], A[k + 8], 8, 0x00FF00FFu);
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t a = A[i], b = A[i + 8];
+    A[i] = __byte_perm(a, b, 0x5410);
+    A[i + 8] = __byte_perm(a, b, 0x7632);
+  }
 #pragma unroll
-  for (int k = 0; k < 16; ++k)
-    if (!(k & 4)) dswap(A[k], A[k + 4], 4, 0x0F0F0F0Fu);
+  for (int i = 0; i < 8; ++i) dswap(A[i], A[i + 8], 1, 0x55555555u);
 #pragma unroll
-  for (int k = 0; k < 16; ++k)
-    if (!(k & 2)) dswap(A[k], A[k + 2], 2, 0x33333333u);
+  for (int i = 0; i < 16; ++i)
+    if (!(i & 4)) {
+      const uint32_t a = A[i], b = A[i + 4];
+      A[i] = __byte_perm(a, b, 0x6240);
+      A[i + 4] = __byte_perm(a, b, 0x7351);
+    }
 #pragma unroll
-  for (int k = 0; k < 16; ++k)
-    if (!(k & 1)) dswap(A[k], A[k + 1], 1, 0x55555555u);
-  // A[i] bit j is plane kmax - j: reverse and align so that bit k is plane k.
-  const int sh = 31 - kmax;  // 0..32
+  for (int i = 0; i < 16; ++i)
+    if (!(i & 2)) dswap(A[i], A[i + 2], 4, 0x0F0F0F0Fu);
 #pragma unroll
-  for (int i = 0; i < 16; ++i) u[i] = sh >= 32 ? 0u : (__brev(A[i]) >> sh);
+  for (int i = 0; i < 16; ++i)
+    if (!(i & 1)) dswap(A[i], A[i + 1], 2, 0x33333333u);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) u[i] = A[((i & 1) << 3) | (i >> 1)];
 }
 
-// Shared memory the decoder needs: one 32-word column per thread of a block
-// of kDecodeThreads threads.
-constexpr int kDecodeThreads = 256;
-constexpr int kPlaneWords = 32 * kDecodeThreads;
-
-// Decode one block: q (row-major) after the inverse transform, emax, nonzero.
-// Ps: the thread's column of a kPlaneWords-word shared array (stride kDecodeThreads).
-template <int NW32>
-__device__ __forceinline__ bool decode_block(const uint32_t (&w)[NW32 + 2], uint32_t* __restrict__ Ps, int32_t (&q)[16],
+// Decode one block: q (row-major) after the inverse transform, and emax; false
+// for a zero block, whose q mean nothing.
+template <int NW32, int TH>
+__device__ __forceinline__ bool decode_block(const uint32_t (&w)[NW32], Wz1Smem<NW32, TH>& sm, int32_t (&q)[16],
                                              int& emax) {
   const bool nz = w[0] & 1u;
   emax = (int)((w[0] >> 1) & 0xFFu) - 127;
   uint32_t u[16];
-  decode_planes<NW32>(w, Ps, kDecodeThreads, u);
+  decode_planes<NW32, TH>(w, sm, u);
   uint32_t c[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) c[seq_index(k)] = (u[k] ^ 0xAAAAAAAAu) - 0xAAAAAAAAu;
@@ -168,13 +231,13 @@ __device__ __forceinline__ bool decode_block(const uint32_t (&w)[NW32 + 2], uint
 #pragma unroll
   for (int r = 0; r < 4; ++r) inv_lift(c[4 * r], c[4 * r + 1], c[4 * r + 2], c[4 * r + 3]);
 #pragma unroll
-  for (int i = 0; i < 16; ++i) q[i] = nz ? (int32_t)c[i] : 0;
+  for (int i = 0; i < 16; ++i) q[i] = (int32_t)c[i];
   return nz;
 }
 
 // Load one block's words (2*rate bytes at a 2*rate-byte-aligned address).
 template <int NW32>
-__device__ __forceinline__ void load_block(const uint8_t* __restrict__ base, int64_t blk, uint32_t (&w)[NW32 + 2]) {
+__device__ __forceinline__ void load_block(const uint8_t* __restrict__ base, int64_t blk, uint32_t (&w)[NW32]) {
   const uint8_t* p = base + (uint64_t)blk * (uint64_t)(4 * NW32);
   if constexpr (NW32 % 4 == 0) {
 #pragma unroll
@@ -193,8 +256,6 @@ __device__ __forceinline__ void load_block(const uint8_t* __restrict__ base, int
       w[2 * i + 1] = v.y;
     }
   }
-  w[NW32] = 0;
-  w[NW32 + 1] = 0;
 }
 
 }  // namespace dev
