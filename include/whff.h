@@ -318,8 +318,9 @@ void whff_fields_destroy(whff_fields* f);
 /* Launch shape of the fixed-allocation (WZ2) kernels: blocks kept in flight
  * per lane (2, 4 or 8), resident CTAs per SM of the persistent grid, and the
  * fold flags: WHFF_FOLD_FP32_PAIRS folds a band's 32 lane sums as FP32
- * (hi, lo) pairs with TwoSum, widened once, instead of widening to FP64 and
- * adding in FP64 (cheaper on GB300's small FP64 pipe; pays on short bands);
+ * (hi, lo) pairs with TwoSum, good to about 2^-48 and widened once, instead of
+ * as triples that keep more than FP64's digits (fewer instructions; pays on
+ * short bands);
  * WHFF_FOLD_LANE_GROUPS lets four 8-lane groups of a warp take four bands at
  * once (short bands: tall matrices), with unroll 2 only.  Defaults: FP32
  * pairs below 4096 blocks per band, lane groups below 256.  Unroll does not

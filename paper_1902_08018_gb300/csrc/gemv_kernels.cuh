@@ -7,8 +7,8 @@
 // contiguous run of the compressed stream per iteration.  (The fixed-
 // allocation and scaled formats use the persistent range schedule of
 // wz2_kernels.cuh / scaled_kernels.cuh.)  Each lane keeps compensated FP32 sums
-// (TwoSum: hi + lo) per row and right-hand side; the warp folds them in FP64
-// with shuffles.  With one column range per band the warp finishes y and the
+// (TwoSum: hi + lo) per row and right-hand side; the warp folds them with
+// shuffles (fold.cuh) and widens the totals.  With one column range per band the warp finishes y and the
 // state itself; with several (split-K, for wide matrices whose few rows
 // cannot fill the GPU -- the cuBLAS failure mode of Sec. 5.1) the FP64
 // partials go to a workspace and a second kernel sums them in split order.
@@ -19,6 +19,7 @@
 #include <cstdint>
 
 #include "decode_out.cuh"
+#include "fold.cuh"
 #include "wz1_decode.cuh"
 
 namespace whff {
@@ -34,99 +35,115 @@ __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float p) {
   lo += err;
 }
 
-// Sum over aligned groups of GL lanes (GL = 32: the warp); every lane of a
-// group ends with its group's sum.  All 32 lanes must execute it.
-template <int GL = 32>
-__device__ __forceinline__ double warp_sum(double v) {
+// The band of values z (value k of the fold: column k / 4, row k % 4) that a lane
+// holds, written to y, the state (column by column) or the partials.
+// MIX 1: the lift's 2G mixing of a column's four rows and 2^-3; MIX 2: 2^3 (no
+// transform); MIX 0: as they are.  All 32 lanes call it; `lane` is the lane in
+// its group of GL.
+//   part != nullptr: value k goes to part[k] (mixed): a segment of a shared band;
+//   else row i of the band is row row0 + i of y (and of the state), below M.
+//   active = false: a group without a piece writes nothing.
+template <int MIX, int R, int GL>
+__device__ __forceinline__ void band_write(double (&z)[4 * R >= GL ? 4 * R / GL : 1], int lane, int64_t row0, int64_t M,
+                                           double* __restrict__ part, double* __restrict__ y, int64_t ldy,
+                                           double* __restrict__ state, double decay, bool active) {
+  constexpr unsigned kAll = 0xFFFFFFFFu;
+  constexpr int N = 4 * R;
+  constexpr int C = N >= GL ? N / GL : 1;  // values per lane
+  constexpr int S = N >= GL ? 1 : GL / N;  // lanes per value
+  const int first = fold_index<N, GL>(lane), base = (threadIdx.x & 31) - lane;
+  // the value k of the group: lane k / C * S holds it
+  auto from = [&](int k, int own) { return __shfl_sync(kAll, z[own], base + k / C * S); };
+  if (MIX == 1) {  // y = (2G) z * 2^-3, 2G rows (2,-1,-1,0), (2,-1,1,0), (2,1,-1,-1), (2,1,1,1)
+    double t[C];
+    const int q = first & ~3;
+    if constexpr (C >= 4) {  // whole columns in the lane
 #pragma unroll
-  for (int o = GL / 2; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Sum of the 32 lanes' compensated (hi, lo) pairs, in a fixed butterfly:
-// each level adds the partner's hi with TwoSum (its error is exact whatever
-// the operand order) and the partner's lo plainly, so every lane ends with
-// the same pair, good to about 2^-48.  FP32 work only: on GB300 the FP64
-// pipe is a small fraction of the FP32 one, and only the result is widened.
-// It pays where bands are short (tall matrices: many band sums per block
-// streamed); on long bands the FP64 butterfly above is a little faster, so
-// the choice is a per-matrix setting (see whff_set_config).
-template <int GL = 32>
-__device__ __forceinline__ double warp_sum_pair(float hi, float lo) {
+      for (int c = 0; c < C; ++c) {
+        const int i = c & 3, b = c & ~3;
+        double v = times_pow2(z[b], 1);
+        v = i < 2 ? v - z[b + 1] : v + z[b + 1];
+        v = i & 1 ? v + z[b + 2] : v - z[b + 2];
+        if (i >= 2) v = i == 2 ? v - z[b + 3] : v + z[b + 3];
+        t[c] = times_pow2(v, -3);
+      }
+    } else {
+      const double z0 = from(q, 0), z1 = from(q + 1, C == 2 ? 1 : 0), z2 = from(q + 2, 0),
+                   z3 = from(q + 3, C == 2 ? 1 : 0);
 #pragma unroll
-  for (int o = GL / 2; o; o >>= 1) {
-    const float h2 = __shfl_xor_sync(0xffffffffu, hi, o);
-    const float l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-    const float s = hi + h2;
-    const float bp = s - hi;
-    const float e = (hi - (s - bp)) + (h2 - bp);
-    hi = s;
-    lo = (lo + l2) + e;
-  }
-  return (double)hi + (double)lo;
-}
-
-// Totals over the warp of 32 compensated pairs per lane: lane l returns that of
-// pair l.  Each level hands half of the pairs to the partner lane and adds the
-// half that it keeps (TwoSum, as warp_sum_pair), so the 32 totals take 31 pair
-// additions instead of 32 butterflies of five.
-__device__ __forceinline__ double warp_sum_pairs32(float (&hi)[32], float (&lo)[32], int lane) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    const bool up = lane & o;
-#pragma unroll
-    for (int k = 0; k < o; ++k) {
-      const float h2 = __shfl_xor_sync(0xffffffffu, up ? hi[k] : hi[k + o], o);
-      const float l2 = __shfl_xor_sync(0xffffffffu, up ? lo[k] : lo[k + o], o);
-      const float h = up ? hi[k + o] : hi[k], l = up ? lo[k + o] : lo[k];
-      const float s = h + h2;
-      const float bp = s - h;
-      const float e = (h - (s - bp)) + (h2 - bp);
-      hi[k] = s;
-      lo[k] = (l + l2) + e;
-    }
-  }
-  return (double)hi[0] + (double)lo[0];
-}
-
-// Fold a lane's (hi, lo) sums for 4 rows x R columns and write either the
-// final y (+ state) or the split-K partial.  Deterministic: fixed shuffle tree.
-template <int R>
-__device__ __forceinline__ void finish_band(const float (&hi)[4][R], const float (&lo)[4][R], int lane, int64_t row0,
-                                            int64_t M, int split, int ksplit, int64_t Mpad, double* __restrict__ ws,
-                                            double* __restrict__ y, int64_t ldy, double* __restrict__ state,
-                                            double decay) {
-  double tot[4][R];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int r = 0; r < R; ++r) tot[i][r] = warp_sum((double)hi[i][r] + (double)lo[i][r]);
-  // lane (i*R + r) writes value (i, r)
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      if (lane != i * R + r) continue;
-      const int64_t row = row0 + i;
-      if (ksplit > 1) {
-        ws[((int64_t)split * R + r) * Mpad + row] = tot[i][r];
-      } else if (row < M) {
-        y[(int64_t)r * ldy + row] = tot[i][r];
+      for (int c = 0; c < C; ++c) {
+        const int i = (first + c) & 3;
+        double v = times_pow2(z0, 1) + negate_if(z1, i < 2);
+        v += negate_if(z2, !(i & 1));
+        v += i < 2 ? 0.0 : negate_if(z3, i == 2);
+        t[c] = times_pow2(v, -3);
       }
     }
-  if (ksplit == 1 && state != nullptr && lane < 4) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (lane != i) continue;
+    for (int c = 0; c < C; ++c) z[c] = t[c];
+  } else if (MIX == 2) {
+#pragma unroll
+    for (int c = 0; c < C; ++c) z[c] = times_pow2(z[c], 3);
+  }
+  const bool writer = active && lane % S == 0;
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    const int k = first + c;
+    const int64_t row = row0 + (k & 3);
+    if (!writer) continue;
+    if (part) part[k] = z[c];
+    else if (row < M) y[(int64_t)(k >> 2) * ldy + row] = z[c];
+  }
+  if (state != nullptr) {
+    if constexpr (R == 1) {
+      const int64_t row = row0 + (first & 3);
+      if (writer && !part && row < M) state[row] = decay * state[row] + z[0];
+    } else {  // lane i of the group gathers row i's columns in order
+      const int i = lane & 3;
       const int64_t row = row0 + i;
-      if (row < M) {
-        double s = state[row];
+      const bool mine = active && !part && lane < 4 && row < M;
+      double s = mine ? state[row] : 0.0;
 #pragma unroll
-        for (int r = 0; r < R; ++r) s = decay * s + tot[i][r];
-        state[row] = s;
+      for (int r = 0; r < R; ++r) {
+        double v;
+        if constexpr (C == 1) v = from(4 * r + i, 0);
+        else if constexpr (C == 2) {
+          const double a = from(4 * r + i, 0), b = from(4 * r + i, 1);
+          v = i & 1 ? b : a;
+        } else {
+          v = 0.0;
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const double a = from(4 * r + c, c);
+            if (i == c) v = a;
+          }
+        }
+        s = decay * s + v;
       }
+      if (mine) state[row] = s;
     }
   }
+}
+
+// Fold a lane's (hi, lo) sums for 4 rows x R columns over its group of GL lanes
+// (fold.cuh) and write them.  red32: the FP32 pair fold, else the triple one.
+template <int MIX, int R, int GL = 32>
+__device__ __forceinline__ void band_finish(const float (&hi)[4][R], const float (&lo)[4][R], int lane, int64_t row0,
+                                            int64_t M, double* __restrict__ part, double* __restrict__ y, int64_t ldy,
+                                            double* __restrict__ state, double decay, bool red32, bool active = true) {
+  constexpr int N = 4 * R;
+  float h[N], l[N];
+#pragma unroll
+  for (int k = 0; k < N; ++k) h[k] = hi[k & 3][k >> 2], l[k] = lo[k & 3][k >> 2];
+  double z[N >= GL ? N / GL : 1];
+  if (red32) fold_lanes<N, GL, false>(h, l, lane, z);
+  else fold_lanes<N, GL, true>(h, l, lane, z);
+  band_write<MIX, R, GL>(z, lane, row0, M, part, y, ldy, state, decay, active);
+}
+
+// a / b for non-negative operands, in 32 bits where they fit.
+__device__ __forceinline__ int64_t div64(int64_t a, int64_t b) {
+  return ((uint64_t)a | (uint64_t)b) >> 32 ? a / b : (int64_t)((uint32_t)a / (uint32_t)b);
 }
 
 // x[4J .. 4J+3] of column r, zero beyond N.
@@ -202,7 +219,11 @@ __global__ void __launch_bounds__(kWz1Threads)
       }
     }
   }
-  finish_band<R>(hi, lo, lane, 4 * I, M, split, ksplit, 4 * BM, ws, y, ldy, state, decay);
+  // several splits: the partial of column r, row i goes to ws[(split R + r) Mpad + i]; a column's
+  // rows are then consecutive, as in y
+  const bool part = ksplit > 1;
+  band_finish<0, R>(hi, lo, lane, 4 * I, part ? 4 * BM : M, nullptr, part ? ws + (int64_t)split * R * 4 * BM : y,
+                    part ? 4 * BM : ldy, part ? nullptr : state, decay, false);
 }
 
 // ------------------------------------------------------- scaled-format GEMV

@@ -171,31 +171,26 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32)
 #pragma unroll
       for (int r = 0; r < R; ++r) hi[i][r] = lo[i][r] = 0.f;
     if constexpr (GL == 32) {
-      const int64_t I = b0 / CB;
+      const int64_t I = div64(b0, CB);
       const int64_t piece_end = min(b1, (I + 1) * CB);
-      const int64_t g_lo = (I * CB) / L, g_hi = ((I + 1) * CB - 1) / L;
       scaled_piece<FMT, R, 32>(payload, scales, M, N, ld, TN, 4 * I, b0 - I * CB + lane, piece_end - I * CB, x,
                                ldx, x_fast, hi, lo);
-      if (g_lo == g_hi) {
-        band_finish<0, R>(hi, lo, lane, 4 * I, M, 0, 1, 4 * BM, ws, y, ldy, state, decay, red32);
-      } else {
-        band_finish<0, R>(hi, lo, lane, 4 * ((I * maxseg + (g - g_lo)) * R), M, 0, 2, 0, ws, y, ldy, state, decay,
-                          red32);
-      }
+      const int64_t g_lo = div64(I * CB, L), g_hi = div64((I + 1) * CB - 1, L);
+      band_finish<0, R>(hi, lo, lane, 4 * I, M, g_lo == g_hi ? nullptr : ws + (I * maxseg + (g - g_lo)) * R * 4, y, ldy,
+                        state, decay, red32);
       b0 = piece_end;
     } else {  // lane group lane / GL takes the piece of band b0 / CB + lane / GL
-      const int64_t I = b0 / CB + lane / GL;
+      const int64_t I0 = div64(b0, CB), I = I0 + lane / GL;
       const int64_t pb = max(b0, I * CB), pe = min(b1, (I + 1) * CB);
       const bool active = pb < pe;
-      const int64_t g_lo = (I * CB) / L, g_hi = ((I + 1) * CB - 1) / L;
       if (active)
         scaled_piece<FMT, R, GL>(payload, scales, M, N, ld, TN, 4 * I, pb - I * CB + gl, pe - I * CB, x, ldx, x_fast,
                                  hi, lo);
       // one call for all groups (the folds shuffle across the whole warp)
-      const bool whole = g_lo == g_hi;
-      band_finish<0, R, GL>(hi, lo, gl, whole ? 4 * I : 4 * ((I * maxseg + (g - g_lo)) * R), M, 0, whole ? 1 : 2,
-                            whole ? 4 * BM : 0, ws, y, ldy, state, decay, red32, active);
-      b0 = min(b1, (b0 / CB + NG) * CB);
+      const int64_t g_lo = div64(I * CB, L), g_hi = div64((I + 1) * CB - 1, L);
+      band_finish<0, R, GL>(hi, lo, gl, 4 * I, M, g_lo == g_hi ? nullptr : ws + (I * maxseg + (g - g_lo)) * R * 4, y,
+                            ldy, state, decay, red32, active);
+      b0 = min(b1, (I0 + NG) * CB);
     }
   }
 }
@@ -216,7 +211,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32)
     while (ei + 1 < nentries && entries[ei + 1].block_begin <= b0) ++ei;  // warp-uniform
     const BatchEntry& e = entries[ei];
     const int64_t local = b0 - e.block_begin;
-    const int64_t I = local / e.BN;
+    const int64_t I = div64(local, e.BN);
     const int64_t piece_end = min(b1, e.block_begin + (I + 1) * e.BN);
     int64_t g_lo, g_hi;
     batch_band_span(e, I, L, g_lo, g_hi);
@@ -229,12 +224,8 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32)
       for (int r = 0; r < R; ++r) hi[i][r] = lo[i][r] = 0.f;
     scaled_piece<FMT, R, 32>(e.stream, e.scales, e.M, e.N, e.ld, e.TN, 4 * I, local - I * e.BN + lane,
                              piece_end - e.block_begin - I * e.BN, e.x, e.ldx, x_fast, hi, lo);
-    if (g_lo == g_hi) {
-      band_finish<0, R>(hi, lo, lane, 4 * I, e.M, 0, 1, 4 * e.BM, e.ws, e.y, e.ldy, e.state, e.decay, false);
-    } else {
-      band_finish<0, R>(hi, lo, lane, 4 * ((I * e.maxseg + (g - g_lo)) * R), e.M, 0, 2, 0, e.ws, e.y, e.ldy,
-                        e.state, e.decay, false);
-    }
+    band_finish<0, R>(hi, lo, lane, 4 * I, e.M, g_lo == g_hi ? nullptr : e.ws + (I * e.maxseg + (g - g_lo)) * R * 4,
+                      e.y, e.ldy, e.state, e.decay, false);
     b0 = piece_end;
   }
 }

@@ -46,7 +46,7 @@ struct whff_handle {
   int ksplit = 1;
   int64_t chunk = 0;            // J blocks (WZ1) or columns (scaled) per split
   int ctas_per_sm = 4;          // resident CTAs per SM of the persistent kernels
-  bool red32 = false;           // WZ2 / scaled: fold lanes in FP32 pairs (short bands) instead of FP64
+  bool red32 = false;           // WZ2 / scaled: fold lanes in FP32 pairs (short bands) instead of triples
   bool groups8 = false;         // WZ2: four 8-lane groups per warp, one band each (short bands)
   int unroll = 2;               // WZ2: blocks in flight per lane (R = 1 kernel)
   bool bulk = false;            // WZ2, R = 1: blocks staged through shared memory by bulk copies
@@ -498,7 +498,7 @@ int create_impl(const BlobInfo& info, const uint8_t* src, int max_rhs, unsigned 
   }
   choose_split(h);
   // short bands (tall matrices) fold their lanes in FP32 pairs, long ones in
-  // FP64; very short ones give each band a group of 8 lanes.  BN counts a
+  // triples; very short ones give each band a group of 8 lanes.  BN counts a
   // band's lane work units: 4-column blocks (WZ2) or 16-byte chunks (scaled).
   h->red32 = info.fmt != WHFF_FMT_ZFP && h->BN < 4096;
   h->groups8 = info.fmt != WHFF_FMT_ZFP && h->BN < 256;
@@ -1247,7 +1247,7 @@ extern "C" int whff_tune(whff_handle* h, int iters, void* stream, double* best_m
   const int orig_f = (h->red32 ? WHFF_FOLD_FP32_PAIRS : 0) | (h->groups8 ? WHFF_FOLD_LANE_GROUPS : 0) |
                      (h->bulk ? WHFF_CONFIG_BULK : 0);
   double best = 1e30;
-  int bu = orig_u, bc = orig_c, bf = orig_f;
+  int bu = orig_u, bc = 1 << 20, bf = orig_f;
   int err = WHFF_OK;
   const bool lift = h->info.fmt == WHFF_FMT_FIXED_LIFT;
   // candidates: the top three CTA counts per SM x (unroll 2 with each of the four
@@ -1270,7 +1270,8 @@ extern "C" int whff_tune(whff_handle* h, int iters, void* stream, double* best_m
     if (err) break;
     float ms = 0.f;
     cudaEventElapsedTime(&ms, e0, e1);
-    if (ms / iters < best) {
+    // within the timing's noise of each other (1.5 %), the shape with fewer CTAs
+    if (c < bc ? ms / iters < 1.015 * best : c > bc ? 1.015 * ms / iters < best : ms / iters < best) {
       best = ms / iters;
       bu = u;
       bc = c;

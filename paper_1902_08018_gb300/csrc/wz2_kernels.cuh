@@ -148,94 +148,6 @@ __device__ __forceinline__ void wz2_unpermute(const float (&f)[16], float (&V)[1
   for (int k = 0; k < 16; ++k) V[LIFT ? seq_index(k) : k] = f[k];
 }
 
-// Fold a band's FP64 sums and map them to y: MIX 1 = the lift's 2G mixing
-// and 2^-3, MIX 2 = 2^3 (no transform), MIX 0 = identity (scaled formats).
-template <bool LIFT, int R, int GL = 32>
-__device__ __forceinline__ void wz2_finish(const float (&hi)[4][R], const float (&lo)[4][R], int lane, int64_t row0,
-                                           int64_t M, int split, int ksplit, int64_t Mpad, double* __restrict__ ws,
-                                           double* __restrict__ y, int64_t ldy, double* __restrict__ state,
-                                           double decay, bool red32, bool active = true);
-
-// red32: fold the lanes with the FP32 pair butterfly instead of FP64 (the
-// same bar; another rounding).  GL: lanes per band (32, or 8 when a warp
-// works on 4 bands at once); lane is the lane within its group, and a group
-// with no piece (active = false) folds zeros and writes nothing.  All 32
-// lanes must call it together.
-template <int MIX, int R, int GL = 32>
-__device__ __forceinline__ void band_finish(const float (&hi)[4][R], const float (&lo)[4][R], int lane, int64_t row0,
-                                            int64_t M, int split, int ksplit, int64_t Mpad, double* __restrict__ ws,
-                                            double* __restrict__ y, int64_t ldy, double* __restrict__ state,
-                                            double decay, bool red32, bool active = true) {
-  constexpr bool LIFT = MIX == 1;
-  double z[4][R];
-  if (red32) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int r = 0; r < R; ++r) z[i][r] = warp_sum_pair<GL>(hi[i][r], lo[i][r]);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int r = 0; r < R; ++r) z[i][r] = warp_sum<GL>((double)hi[i][r] + (double)lo[i][r]);
-  }
-  if (!active) return;
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    double t[4];
-    if (LIFT) {  // y = (2G) z * 2^-3, 2G rows (2,-1,-1,0), (2,-1,1,0), (2,1,-1,-1), (2,1,1,1)
-      const double a = 2.0 * z[0][r];
-      t[0] = (a - z[1][r] - z[2][r]) * 0.125;
-      t[1] = (a - z[1][r] + z[2][r]) * 0.125;
-      t[2] = (a + z[1][r] - z[2][r] - z[3][r]) * 0.125;
-      t[3] = (a + z[1][r] + z[2][r] + z[3][r]) * 0.125;
-    } else {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) t[i] = MIX == 2 ? z[i][r] * 8.0 : z[i][r];
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) z[i][r] = t[i];
-  }
-  // lane (i*R + r) mod GL writes value (i, r)
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      if (lane != (i * R + r) % GL) continue;
-      const int64_t row = row0 + i;
-      if (ksplit == 2) {  // segment partial: ws[row0 + r*4 + i] (row0 = 4*(band*maxseg+seg)*R)
-        ws[row0 + r * 4 + i] = z[i][r];
-      } else if (ksplit > 1) {
-        ws[((int64_t)split * R + r) * Mpad + row] = z[i][r];
-      } else if (row < M) {
-        y[(int64_t)r * ldy + row] = z[i][r];
-      }
-    }
-  if (ksplit == 1 && state != nullptr && lane < 4) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (lane != i) continue;
-      const int64_t row = row0 + i;
-      if (row < M) {
-        double s = state[row];
-#pragma unroll
-        for (int r = 0; r < R; ++r) s = decay * s + z[i][r];
-        state[row] = s;
-      }
-    }
-  }
-}
-
-// One block's contribution, scaled: p[i][r] = s * sum_b V[i][b] xt_r[b].
-template <bool LIFT, int R, int GL>
-__device__ __forceinline__ void wz2_finish(const float (&hi)[4][R], const float (&lo)[4][R], int lane, int64_t row0,
-                                           int64_t M, int split, int ksplit, int64_t Mpad, double* __restrict__ ws,
-                                           double* __restrict__ y, int64_t ldy, double* __restrict__ state,
-                                           double decay, bool red32, bool active) {
-  band_finish<LIFT ? 1 : 2, R, GL>(hi, lo, lane, row0, M, split, ksplit, Mpad, ws, y, ldy, state, decay, red32,
-                                   active);
-}
-
 // The stored-order field of row-major coefficient m (the inverse of seq_index).
 __device__ __forceinline__ constexpr int seq_field(int m) {
   constexpr int t[16] = {0, 1, 4, 5, 2, 3, 8, 9, 6, 10, 12, 13, 7, 11, 14, 15};
@@ -507,65 +419,51 @@ __device__ __forceinline__ void wz2_gemv_body(const uint8_t* __restrict__ stream
 #pragma unroll
       for (int r = 0; r < R; ++r) hi[i][r] = lo[i][r] = 0.f;
     if constexpr (GL == 32) {  // the warp takes the piece starting at b0
-      const int64_t I = b0 / BN;
+      const int64_t I = div64(b0, BN);
       const int64_t piece_end = min(b1, (I + 1) * BN);
-      const int64_t g_lo = (I * BN) / L, g_hi = ((I + 1) * BN - 1) / L;
       wz2_piece<RATE, LIFT, R, UNROLL, 32, LIFT>(stream + (uint64_t)(I * BN) * kBlockBytes, b0 - I * BN,
                                                  piece_end - I * BN, lane, x, ldx, N, x_fast, x_vec_ok, hi, lo);
-      if (g_lo == g_hi) {  // the whole band is in this range: finish it here
-        wz2_finish<LIFT, R>(hi, lo, lane, 4 * I, M, 0, 1, 4 * BM, ws, y, ldy, state, decay, red32);
-      } else {  // one segment of a shared band: ws[(band * maxseg + seg) * R + r][i]
-        wz2_finish<LIFT, R>(hi, lo, lane, 4 * ((I * maxseg + (g - g_lo)) * R), M, 0, 2, 0, ws, y, ldy, state,
-                            decay, red32);
-      }
+      // a band inside one range is finished here, a shared one leaves a segment:
+      // ws[(band * maxseg + seg) * R + r][i]
+      const int64_t g_lo = div64(I * BN, L), g_hi = div64((I + 1) * BN - 1, L);
+      band_finish<LIFT ? 1 : 2, R>(hi, lo, lane, 4 * I, M, g_lo == g_hi ? nullptr : ws + (I * maxseg + (g - g_lo)) * R * 4,
+                                   y, ldy, state, decay, red32);
       b0 = piece_end;
     } else {  // lane group lane / GL takes the piece of band b0 / BN + lane / GL
-      const int64_t I = b0 / BN + lane / GL;
+      const int64_t I0 = div64(b0, BN), I = I0 + lane / GL;
       const int64_t pb = max(b0, I * BN), pe = min(b1, (I + 1) * BN);
       const bool active = pb < pe;
-      const int64_t g_lo = (I * BN) / L, g_hi = ((I + 1) * BN - 1) / L;
       if (active)
         wz2_piece<RATE, LIFT, R, UNROLL, GL, LIFT>(stream + (uint64_t)(I * BN) * kBlockBytes, pb - I * BN,
                                                    pe - I * BN, gl, x, ldx, N, x_fast, x_vec_ok, hi, lo);
       // one call for all groups (the folds shuffle across the whole warp)
-      const bool whole = g_lo == g_hi;
-      wz2_finish<LIFT, R, GL>(hi, lo, gl, whole ? 4 * I : 4 * ((I * maxseg + (g - g_lo)) * R), M, 0, whole ? 1 : 2,
-                              whole ? 4 * BM : 0, ws, y, ldy, state, decay, red32, active);
-      b0 = min(b1, (b0 / BN + NG) * BN);
+      const int64_t g_lo = div64(I * BN, L), g_hi = div64((I + 1) * BN - 1, L);
+      band_finish<LIFT ? 1 : 2, R, GL>(hi, lo, gl, 4 * I, M,
+                                       g_lo == g_hi ? nullptr : ws + (I * maxseg + (g - g_lo)) * R * 4, y, ldy, state,
+                                       decay, red32, active);
+      b0 = min(b1, (I0 + NG) * BN);
     }
   }
 }
 
-// The persistent kernel (body above).  Its packed unroll-4 instantiation
-// (rates 8 and 12) is held to 3 resident CTAs per SM; every other one keeps
-// the compiler's default register budget.
+// CTAs per SM that the plans count on: those of the two-block kernel decide the
+// default warp ranges, and with them which blocks are paired before they enter
+// the sums, so they stay what they are -- a CTA more would change the last bits
+// of every result, and measures no better (rate 20, 8192^2: 37.0 us with 3,
+// 37.9 with 4).  The kernels are held to them.
+template <int RATE>
+__host__ __device__ constexpr int wz2_ctas_per_sm(int unroll) {
+  return unroll == 8 ? (RATE <= 8 ? 3 : RATE <= 20 ? 2 : 1) : unroll == 4 ? (RATE <= 16 ? 3 : 2) : RATE <= 16 ? 4 : 3;
+}
+
 template <int RATE, bool LIFT, int R, int UNROLL, int GL>
-__global__ void __launch_bounds__(kWarpsPerCta * 32)
+__global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? wz2_ctas_per_sm<RATE>(UNROLL) : 1)
     wz2_gemv_kernel(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM, int64_t BN,
                     const float* __restrict__ x, int64_t ldx, bool x_vec_ok, int64_t L, int maxseg,
                     double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
                     double decay, bool red32) {
   wz2_gemv_body<RATE, LIFT, R, UNROLL, GL>(stream, M, N, BM, BN, x, ldx, x_vec_ok, L, maxseg, ws, y, ldy, state,
                                            decay, red32);
-}
-
-template <int RATE, bool LIFT, int R, int UNROLL, int GL>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, 3)
-    wz2_gemv_kernel_o3(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM, int64_t BN,
-                       const float* __restrict__ x, int64_t ldx, bool x_vec_ok, int64_t L, int maxseg,
-                       double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
-                       double decay, bool red32) {
-  wz2_gemv_body<RATE, LIFT, R, UNROLL, GL>(stream, M, N, BM, BN, x, ldx, x_vec_ok, L, maxseg, ws, y, ldy, state,
-                                           decay, red32);
-}
-
-// The instantiation a launch uses.
-template <int RATE, bool LIFT, int R, int UNROLL, int GL>
-constexpr auto wz2_gemv_entry() {
-  if constexpr (wz2_packed<RATE>() && R == 1 && UNROLL == 4)
-    return &wz2_gemv_kernel_o3<RATE, LIFT, R, UNROLL, GL>;
-  else
-    return &wz2_gemv_kernel<RATE, LIFT, R, UNROLL, GL>;
 }
 
 // sum_{k < n} p[k * stride], added in k order; the loads of eight terms are
@@ -608,12 +506,12 @@ static __global__ void wz2_segment_epilogue(const double* __restrict__ ws, int64
   const int64_t g = 1 + (q >> 5);  // the boundary of this warp (warp-uniform)
   const int i = (int)((q & 31) >> 3), j = (int)(q & 7);
   const int64_t b = g * L, total = ((M + 3) / 4) * BN;
-  const int64_t I = b / BN;
+  const int64_t I = div64(b, BN);
   // a boundary inside band I, and the first one there (the previous one is not inside I)
-  const bool mine = b < total && b % BN != 0 && (g - 1) * L <= I * BN;
+  const bool mine = b < total && b != I * BN && (g - 1) * L <= I * BN;
   const int64_t row = 4 * I + i;
   const bool valid = mine && row < M;
-  const int64_t g_lo = (I * BN) / L, g_hi = ((I + 1) * BN - 1) / L;
+  const int64_t g_lo = div64(I * BN, L), g_hi = div64((I + 1) * BN - 1, L);
   double s = (valid && state) ? state[row] : 0.0;
   for (int r = 0; r < R; ++r) {
     double t = 0.0;
@@ -634,16 +532,18 @@ static __global__ void wz2_segment_epilogue(const double* __restrict__ ws, int64
 __device__ __forceinline__ void batch_band_span(const BatchEntry& e, int64_t I, int64_t L, int64_t& g_lo,
                                                 int64_t& g_hi) {
   const int64_t first = e.block_begin + I * e.BN;
-  g_lo = first / L;
-  g_hi = (first + e.BN - 1) / L;
+  g_lo = div64(first, L);
+  g_hi = div64(first + e.BN - 1, L);
 }
 
 // One persistent launch over all matrices of a batch that share a format,
 // rate and right-hand-side count: the global block order is the entries'
 // band-major orders one after another, split into contiguous warp ranges
 // exactly as for a single matrix.
+// One column: held to the CTAs per SM that its grid is made for (wz2_occupancy);
+// at three where the grid counts on four, a quarter of it ran alone at the end.
 template <int RATE, bool LIFT, int R, int UNROLL>
-__global__ void __launch_bounds__(kWarpsPerCta * 32)
+__global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? wz2_ctas_per_sm<RATE>(UNROLL) : 1)
     wz2_batched_kernel(const BatchEntry* __restrict__ entries, int nentries, int64_t total, int64_t L) {
   constexpr int64_t kBlockBytes = 4 * Wz2Layout<RATE>::kWords;
   const int lane = threadIdx.x & 31;
@@ -655,7 +555,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32)
     while (ei + 1 < nentries && entries[ei + 1].block_begin <= b0) ++ei;  // warp-uniform
     const BatchEntry& e = entries[ei];
     const int64_t local = b0 - e.block_begin;
-    const int64_t I = local / e.BN;
+    const int64_t I = div64(local, e.BN);
     const int64_t piece_end = min(b1, e.block_begin + (I + 1) * e.BN);
     int64_t g_lo, g_hi;
     batch_band_span(e, I, L, g_lo, g_hi);
@@ -669,12 +569,9 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32)
     wz2_piece<RATE, LIFT, R, UNROLL>(e.stream + (uint64_t)(I * e.BN) * kBlockBytes, local - I * e.BN,
                                      piece_end - e.block_begin - I * e.BN, lane, e.x, e.ldx, e.N, x_fast, x_vec_ok,
                                      hi, lo);
-    if (g_lo == g_hi) {
-      wz2_finish<LIFT, R>(hi, lo, lane, 4 * I, e.M, 0, 1, 4 * e.BM, e.ws, e.y, e.ldy, e.state, e.decay, false);
-    } else {
-      wz2_finish<LIFT, R>(hi, lo, lane, 4 * ((I * e.maxseg + (g - g_lo)) * R), e.M, 0, 2, 0, e.ws, e.y, e.ldy,
-                          e.state, e.decay, false);
-    }
+    band_finish<LIFT ? 1 : 2, R>(hi, lo, lane, 4 * I, e.M,
+                                 g_lo == g_hi ? nullptr : e.ws + (I * e.maxseg + (g - g_lo)) * R * 4, e.y, e.ldy,
+                                 e.state, e.decay, false);
     b0 = piece_end;
   }
 }

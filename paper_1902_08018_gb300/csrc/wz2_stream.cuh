@@ -85,7 +85,7 @@ __device__ __forceinline__ void cursor_next(StageCursor& c, int n, int64_t b1, i
 }
 
 template <int RATE, bool LIFT>
-__global__ void __launch_bounds__(kWarpsPerCta * 32)
+__global__ void __launch_bounds__(kWarpsPerCta * 32, 3)
     wz2_stream_kernel(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM, int64_t BN,
                       const float* __restrict__ x, int64_t ldx, bool x_vec_ok, int64_t L, int maxseg,
                       double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
@@ -183,13 +183,9 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32)
     const int64_t I = cc.I;
     cursor_next(cc, n, b1, BN);
     if (cc.I != I) {  // the piece of band I is complete: fold it as wz2_gemv_kernel does
-      const int64_t g_lo = (I * BN) / L, g_hi = ((I + 1) * BN - 1) / L;
-      if (g_lo == g_hi) {
-        wz2_finish<LIFT, 1>(hi, lo, lane, 4 * I, M, 0, 1, 4 * BM, ws, y, ldy, state, decay, red32);
-      } else {
-        wz2_finish<LIFT, 1>(hi, lo, lane, 4 * ((I * maxseg + (g - g_lo)) * 1), M, 0, 2, 0, ws, y, ldy, state, decay,
-                            red32);
-      }
+      const int64_t g_lo = div64(I * BN, L), g_hi = div64((I + 1) * BN - 1, L);
+      band_finish<LIFT ? 1 : 2, 1>(hi, lo, lane, 4 * I, M, g_lo == g_hi ? nullptr : ws + (I * maxseg + (g - g_lo)) * 4,
+                                   y, ldy, state, decay, red32);
 #pragma unroll
       for (int i = 0; i < 4; ++i) hi[i][0] = lo[i][0] = 0.f;
     }

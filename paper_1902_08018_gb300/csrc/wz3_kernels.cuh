@@ -192,12 +192,9 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
         wz3_accumulate<R>(V, s, xt, ldt, 32 * q + lane, hi, lo);
       }
     }
-    const int64_t g_lo = (I * RB) / L, g_hi = ((I + 1) * RB - 1) / L;
-    if (g_lo == g_hi)
-      band_finish<1, R>(hi, lo, lane, 4 * I, M, 0, 1, 4 * BM, ws, y, ldy, state, decay, false);
-    else
-      band_finish<1, R>(hi, lo, lane, 4 * ((I * maxseg + (g - g_lo)) * R), M, 0, 2, 0, ws, y, ldy, state, decay,
-                        false);
+    const int64_t g_lo = div64(I * RB, L), g_hi = div64((I + 1) * RB - 1, L);
+    band_finish<1, R>(hi, lo, lane, 4 * I, M, g_lo == g_hi ? nullptr : ws + (I * maxseg + (g - g_lo)) * R * 4, y, ldy,
+                      state, decay, false);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -216,8 +213,8 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
 // The chain of a row takes scalar FMAs (their operands need no doubling into
 // pairs; a packed instruction takes two issue cycles of the FMA pipe anyway), the
 // TwoSum packed ones on rows 2h and 2h + 1.
-// The 32 sums of a band (r, i) are folded over the lanes by warp_sum_pairs32,
-// lane 4 r + i ending with that of row i and column r: FP64 butterflies cost
+// The 32 sums of a band (r, i) are folded over the lanes as pairs
+// (fold.cuh), lane 4 r + i ending with that of row i and column r: FP64 butterflies cost
 // 2600 cycles of GB300's FP64 pipe per band piece.
 // 8192^2 at 1e-7 (0.18 GB, one pass of 8 columns): 269 us and 12 us of segment
 // epilogue with warp ranges and FP64 folds, 105 us and 4 us this way, at 56 % of
@@ -272,32 +269,6 @@ __device__ __forceinline__ void wz3_prefetch_run(const uint8_t* __restrict__ are
 
 __device__ __forceinline__ int64_t wz3_groups(int64_t BM) { return (BM + 7) / 8; }
 
-// The lane's total z of (r, i), lane = 4 r + i, mixed with 2G over the rows
-// (lanes 4 r .. 4 r + 3): y of row i.
-__device__ __forceinline__ double wz3_mix_rows(double z, int lane) {
-  const int q = lane & ~3, i = lane & 3;
-  const double z0 = __shfl_sync(0xffffffffu, z, q), z1 = __shfl_sync(0xffffffffu, z, q + 1),
-               z2 = __shfl_sync(0xffffffffu, z, q + 2), z3 = __shfl_sync(0xffffffffu, z, q + 3);
-  double t = 2.0 * z0;
-  t = i < 2 ? t - z1 : t + z1;
-  t = i & 1 ? t + z2 : t - z2;
-  if (i >= 2) t = i == 2 ? t - z3 : t + z3;
-  return t * 0.125;
-}
-
-// y (and the state, column by column) of one band from its 32 totals.
-__device__ __forceinline__ void wz3_write_band8(double t, int lane, int64_t I, int64_t M, double* __restrict__ y,
-                                                int64_t ldy, double* __restrict__ state, double decay) {
-  const int64_t row = 4 * I + (lane & 3);
-  if (row < M) y[(int64_t)(lane >> 2) * ldy + row] = t;
-  if (state) {
-    double s = lane < 4 && row < M ? state[row] : 0.0;
-#pragma unroll
-    for (int r = 0; r < 8; ++r) s = decay * s + __shfl_sync(0xffffffffu, t, 4 * r + (lane & 3));
-    if (lane < 4 && row < M) state[row] = s;
-  }
-}
-
 static __global__ void __launch_bounds__(kWarpsPerCta * 32, 2)
     wz3_gemv8_kernel(const uint64_t* __restrict__ index, const uint8_t* __restrict__ area, int64_t M, int64_t BM,
                      int BN, int RB, const float* __restrict__ xt, int64_t L, int maxseg, double* __restrict__ ws,
@@ -342,12 +313,11 @@ static __global__ void __launch_bounds__(kWarpsPerCta * 32, 2)
         h[4 * r + 2 * k] = a.x, h[4 * r + 2 * k + 1] = a.y;
         l[4 * r + 2 * k] = b.x, l[4 * r + 2 * k + 1] = b.y;
       }
-    const double t = wz3_mix_rows(warp_sum_pairs32(h, l, lane), lane);
-    const int64_t c_lo = (G * RB) / L, c_hi = ((G + 1) * RB - 1) / L;
-    if (c_lo == c_hi)
-      wz3_write_band8(t, lane, I, M, y, ldy, state, decay);
-    else
-      ws[(I * maxseg + (blockIdx.x - c_lo)) * 32 + lane] = t;
+    double z[1];
+    fold_lanes<32, 32, false, true>(h, l, lane, z);
+    const int64_t c_lo = div64(G * RB, L), c_hi = div64((G + 1) * RB - 1, L);
+    band_write<1, 8, 32>(z, lane, 4 * I, M, c_lo == c_hi ? nullptr : ws + (I * maxseg + (blockIdx.x - c_lo)) * 32, y,
+                         ldy, state, decay, true);
   }
 }
 
@@ -362,8 +332,8 @@ static __global__ void __launch_bounds__(256)
   const int64_t G = b / RB, I = 8 * G + (threadIdx.x >> 5);
   if (b >= wz3_groups(BM) * RB || b % RB == 0 || (c - 1) * L > G * RB || I >= BM) return;
   const int64_t c_lo = (G * RB) / L, c_hi = ((G + 1) * RB - 1) / L;
-  const double t = seq_sum_strided(ws + I * maxseg * 32 + lane, c_hi - c_lo + 1, 32);
-  wz3_write_band8(t, lane, I, M, y, ldy, state, decay);
+  double z[1] = {seq_sum_strided(ws + I * maxseg * 32 + lane, c_hi - c_lo + 1, 32)};
+  band_write<0, 8, 32>(z, lane, 4 * I, M, nullptr, y, ldy, state, decay, true);
 }
 
 // Decode: thread per block, the exact definition -- T = (2G) V (2G)^T in

@@ -1,0 +1,44 @@
+"""Folding a band's sums over the lanes: totals past FP32's range and near its
+lower end, where the long bands' fold (beyond FP64) has to hold what FP64 held.
+
+Constant rows make every product the same power of two, so lane sums, totals
+and y are exact: y must equal the FP64 product exactly (lift: 2G mixing and the
+scaling are exact too)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need CUDA")
+    import paper_1902_08018_gb300 as W
+
+    W.library()
+    return W, torch
+
+
+@pytest.mark.parametrize("fmt,rate", [(1, 16), (5, 8), (5, 16), (6, 16), (8, 0)])
+@pytest.mark.parametrize("exp", [112, 0, -80])
+@pytest.mark.parametrize("R", [1, 8])
+def test_totals_beyond_fp32(env, orc, fmt, rate, exp, R):
+    W, torch = env
+    M, N = 9, 1 << 16  # 16384 blocks per band: the FP64 default; totals of 2^(16 + exp) times 1 or 2
+    A = np.full((M, N), 2.0**exp)
+    A[4] = -A[4]
+    blob = W.whff_compress_accuracy(A, 0.0) if fmt == 8 else W.whff_compress(A, fmt, rate)
+    Ahat = orc.wz3_decode(blob.tobytes())[0] if fmt == 8 else orc.decode(blob.tobytes())
+    assert (Ahat == A).all()
+    X = np.full((R, N), 1.0, dtype=np.float32) * np.array([2.0**(r % 2) for r in range(R)], dtype=np.float32)[:, None]
+    with W.whff_create(blob, max_rhs=R) as h:
+        if R > 1 and fmt in (5, 6):
+            h.crossover = 33  # CUDA cores
+        y = torch.zeros((R, M), dtype=torch.float64, device="cuda")
+        h.step(torch.from_numpy(X).cuda(), y)
+        torch.cuda.synchronize()
+        got = y.cpu().numpy()
+    assert (got == X.astype(np.float64) @ A.T).all()
