@@ -20,6 +20,12 @@ static int mma_set_smem(int bytes) {
   return 0;
 }
 
+// CTAs that take `ranges` item ranges, kMmaRanges each.
+template <int RATE>
+static unsigned mma_grid(int ranges) {
+  return (unsigned)((ranges + dev::kMmaRanges<RATE> - 1) / dev::kMmaRanges<RATE>);
+}
+
 template <int RATE, bool LIFT, int NR>
 static int mma_one(const MmaStep& a, cudaStream_t st) {
   using S = dev::MmaSmem<RATE, NR>;
@@ -27,11 +33,11 @@ static int mma_one(const MmaStep& a, cudaStream_t st) {
   if (mma_set_smem<RATE, LIFT, NR, false>(smem)) return -1;
   const int nstages = (int)((a.BN + dev::kMmaStageBlocks - 1) / dev::kMmaStageBlocks);
   const int tiles = (int)((a.BM + dev::kMmaBands - 1) / dev::kMmaBands);
-  const dev::MmaMember mem{a.stream, a.btiles, a.ws, a.BM, a.BN, 0, nstages, tiles, a.R, a.maxseg};
+  const dev::MmaMember mem{a.stream, a.btiles, a.ws, a.BM, a.BN, 0, nstages, tiles, a.R, a.maxseg, a.map, a.paired, a.band0};
   const dev::MmaPass pass{a.x, a.y, a.btiles, a.ws, a.ldx, a.ldy, a.N, a.M, 0, 0, 0, nstages, tiles, a.R, a.maxseg};
   const int64_t bthreads = (int64_t)nstages * dev::kMmaStageBlocks * NR;
   dev::wz2_mma_btiles<LIFT, NR><<<(unsigned)((bthreads + 255) / 256), 256, 0, st>>>(pass, nullptr, 1, bthreads);
-  dev::wz2_mma_kernel<RATE, LIFT, NR, false><<<(unsigned)a.ctas, dev::kMmaThreads, smem, st>>>(
+  dev::wz2_mma_kernel<RATE, LIFT, NR, false><<<mma_grid<RATE>(a.ctas), dev::kMmaDecodeThreads, smem, st>>>(
       mem, nullptr, 1, (int64_t)tiles * nstages, a.L, a.status, a.spin);
   const int64_t fin_threads = (int64_t)tiles * a.R * 32;
   dev::wz2_mma_finish<LIFT><<<(unsigned)((fin_threads + 255) / 256), 256, 0, st>>>(pass, nullptr, 1, fin_threads,
@@ -60,7 +66,7 @@ static int mma_batch_one(const MmaBatchStep& a, cudaStream_t st) {
   const dev::MmaPass p0{};
   dev::wz2_mma_btiles<LIFT, NR><<<(unsigned)((a.bt_threads + 255) / 256), 256, 0, st>>>(p0, a.passes, a.nmem,
                                                                                        a.bt_threads);
-  dev::wz2_mma_kernel<RATE, LIFT, NR, true><<<(unsigned)a.ctas, dev::kMmaThreads, smem, st>>>(m0, a.members, a.nmem,
+  dev::wz2_mma_kernel<RATE, LIFT, NR, true><<<mma_grid<RATE>(a.ctas), dev::kMmaDecodeThreads, smem, st>>>(m0, a.members, a.nmem,
                                                                                             a.total, a.L, a.status,
                                                                                             a.spin);
   dev::wz2_mma_finish<LIFT><<<(unsigned)((a.fin_threads + 255) / 256), 256, 0, st>>>(p0, a.passes, a.nmem,
@@ -100,32 +106,19 @@ int mma_launch(const MmaStep& a, cudaStream_t st) {
   }
 }
 
-// Resident CTAs per SM from the kernel's registers, shared memory and TMEM
-// columns (the occupancy API under-reports this kernel); a persistent grid
-// sized from a value that is too high is still correct, only slower.
+// Item ranges per SM of a pass (0 if the kernel cannot run here): one resident
+// CTA takes them one after another.
 template <int RATE, bool LIFT, int NR>
 static int mma_occ_one() {
   using S = dev::MmaSmem<RATE, NR>;
-  auto kern = dev::wz2_mma_kernel<RATE, LIFT, NR, true>;  // the larger of the two (registers, table)
-  const int smem = S::kBytes + kMaxMembers * (int)sizeof(dev::MmaMember);
   cudaFuncAttributes fa;
-  int dev = 0, smem_sm = 0, regs_sm = 0, reserved = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
-          cudaSuccess ||
-      cudaFuncGetAttributes(&fa, kern) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess) {
+  if (mma_set_smem<RATE, LIFT, NR, true>(S::kBytes + kMaxMembers * (int)sizeof(dev::MmaMember)) ||
+      cudaFuncGetAttributes(&fa, dev::wz2_mma_kernel<RATE, LIFT, NR, true>) != cudaSuccess ||
+      fa.maxThreadsPerBlock < dev::kMmaDecodeThreads) {
     cudaGetLastError();
     return 0;
   }
-  const int warps = dev::kMmaThreads / 32;
-  const int regs_warp = (fa.numRegs * 32 + 255) / 256 * 256;
-  const int by_regs = regs_sm / (regs_warp * warps);
-  const int by_smem = smem_sm / (smem + (int)fa.sharedSizeBytes + reserved);
-  const int by_tmem = 512 / (int)dev::mma_tmem_cols<NR>();
-  return std::min(std::min(by_regs, by_smem), by_tmem);
+  return dev::kMmaRanges<RATE>;
 }
 
 template <int RATE>

@@ -22,19 +22,32 @@
 // and drained into TwoSum FP32 registers, so FP32 rounding never sees long
 // sums.
 //
-// CTA = 8 warps = 256 threads, persistent: the grid splits the sequence of
-// (tile, stage) items -- tile = 32 bands = 128 coefficient rows, stage = 16
-// blocks of K -- into equal contiguous ranges.  Two stages are in flight:
-// while the tensor cores multiply stage k (A and B tiles of buffer k % 2),
-// the threads decode stage k+1 into the other A tile and drain the other TMEM
-// accumulator when stage k-1 closed its group; the words of stage k+2 are already
-// being loaded, and one thread brings the prebuilt B tile of stage k+1 in with
-// a bulk copy (cp.async.bulk) tracked by an mbarrier.  A tile row m holds
-// coefficient row a of band b as m = 32a + b, which makes every warp's tile
-// stores bank-conflict free.  At the end of a tile piece the FP32 sums go to
-// the workspace as one FP64 segment partial; wz2_mma_finish adds a band's
-// segments in order and mixes with 2G, wz2_mma_state applies the state.
+// Tiles are 32 bands = 128 coefficient rows, stages 16 blocks of K.  The sequence
+// of (tile, stage) items is split into equal contiguous ranges; one CTA per SM is
+// resident and takes its ranges' stages through three rings with a role each:
+//  * copies: the stage's B tile (bulk copy) and its compressed words (tiled copy)
+//    into shared memory, five or six stages ahead;
+//  * decode: twelve warps in quartets, a quartet a stage; a thread turns a block
+//    into its BF16 pieces and stores them straight to TMEM, where A is read from:
+//    the 16x256b store gives lane l the row l / 4 and four values of K, so a
+//    block's four rows land at TMEM lanes 8a + band % 8 of its bands' quarter;
+//  * issue: one elected lane starts the stage's MMAs (A from TMEM, B from shared
+//    memory) and commits them to the stage's and the group's barriers;
+//  * drain: eight warps add a finished group's three accumulators into TwoSum
+//    registers; a range's sums go to the workspace as one FP64 segment partial.
+// wz2_mma_finish adds a band's segments in order and mixes with 2G, wz2_mma_state
+// applies the state.
+// A in shared memory cost 32 KB of stores and as many of operand reads per stage,
+// and the register-fed words a barrier of the whole CTA per stage; measured per
+// stage's MMAs (N = 96 and 64), A from TMEM takes 324 clocks, from shared memory
+// 426 (N = 48 and 32: 175 and 349).  WZ2-lift 16, 12288^2, 32 columns: 131 us
+// before, 79 us now (pass 156 -> 102 us); rate 12 batches of 1024..8192 at 16 and
+// 32 columns: 67 + 54 -> 44 + 40 us.  The same MMAs in the same groups: the results
+// are the same bits.  What bounds it now is the issuing warp's turn-around per
+// stage (about 1200 clocks of waits, issue and commits), not the tensor pipe (27 %
+// busy) nor HBM.
 #pragma once
+#include <cuda.h>
 #include <cuda_bf16.h>
 
 #include <cstdint>
@@ -113,18 +126,26 @@ __host__ __device__ constexpr uint32_t mma_tmem_cols() {
   return 6 * NR <= 32 ? 32u : 6 * NR <= 64 ? 64u : 6 * NR <= 128 ? 128u : 256u;
 }
 
-// Shared memory: A and B tiles of two stages, then 4 mbarriers, the TMEM slot,
-// flags and thread 0's B-copy cursor; the member table follows kBytes.
+// Shared memory of wz2_mma_kernel: a ring of kNB B tiles and of as many stages'
+// compressed words, the barriers, the TMEM
+// slot and the abort flag; the member table follows kBytes.
 template <int RATE, int NR>
 struct MmaSmem {
-  static constexpr int kATile = 128 * 16 * 2;  // one piece, one K step
-  static constexpr int kA = MmaPieces<RATE>::kA * kMmaKSteps * kATile;
+  static constexpr int kNA = MmaPieces<RATE>::kA == 3 ? 3 : 4;  // A buffers in TMEM
   static constexpr int kB = MmaBTile<NR>::kB;
-  static constexpr int kBars = 2 * (kA + kB);
-  static constexpr int kBytes = kBars + 80;  // 4 mbarriers, TMEM slot, flags, cursors
+  static constexpr int kNB = RATE >= 20 ? 5 : 6;
+  static constexpr int kBB = 2 * RATE;  // bytes of a block
+  static constexpr int kRowBytes = kMmaStageBlocks * kBB;  // a band's words, rows back to back as the tiled copy writes them
+  static constexpr int kWords = kMmaBands * (kRowBytes + 16);  // 16 bytes more per row, see the copies
+  static constexpr int kBars = kNB * (kB + kWords);
+  static constexpr int kBytes = kBars + 256;
 };
 
-
+// Ranges that a CTA of wz2_mma_kernel takes one after another.  The ranges, and
+// the accumulator groups that end with them, are those of a grid of two CTAs per
+// SM (one where A takes three pieces).
+template <int RATE>
+constexpr int kMmaRanges = MmaPieces<RATE>::kA == 3 ? 1 : 2;
 
 // Eight columns of the three accumulators at ta, ta + stride, ta + 2 stride,
 // summed big + (small + smaller): one wait for the three loads, tied to their
@@ -276,299 +297,395 @@ __device__ __forceinline__ void split_pair(float2 v, uint32_t (&d)[PA]) {
   }
 }
 
+// Warps of the kernel: one issues the MMAs, three bring the compressed words and
+// the B tiles in, kMmaQuartets x 4 decode, 8 drain.
+constexpr int kMmaIssueWarp = 0, kMmaCopyWarp = 1, kMmaDecodeWarp = 4;
+constexpr int kMmaCopyThreads = 32 * (kMmaDecodeWarp - kMmaCopyWarp);
+constexpr int kMmaQuartets = 3;
+constexpr int kMmaDrainWarp = kMmaDecodeWarp + 4 * kMmaQuartets;
+constexpr int kMmaDecodeThreads = 32 * (kMmaDrainWarp + 8);
+
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
+  return p != 0;
+}
+
+// `bytes` (0 to 16) bytes global -> shared without a register, zeros for the rest
+// of 16; both addresses 16-byte aligned.
+__device__ __forceinline__ void cp_async_zfill(uint32_t dst, const void* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
+// Four 32-bit columns to TMEM by the warp's lanes, 16 lanes of the warp's
+// quarter from taddr on: r0, r1 go to row lane / 4, columns 2 (lane % 4) and + 1;
+// r2, r3 to row 8 + lane / 4.
+__device__ __forceinline__ void tmem_store_16x256(uint32_t taddr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+  asm volatile("tcgen05.st.sync.aligned.16x256b.x1.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(taddr), "r"(r0), "r"(r1), "r"(r2),
+               "r"(r3)
+               : "memory");
+}
+
 // Persistent grid over the item sequence of one or more passes (members):
 // member k owns items [item_begin, item_begin + tiles S), item = item_begin +
-// tile S + stage; CTA g takes items [g L, g L + L).  ws[((tile * maxseg + seg)
-// * R + r) * 128 + m] of a member receives the FP64 partial of tile row m
-// (= 32a + band) for the CTA's segment seg = g - (item_begin + tile S) / L.
+// tile S + stage; range v is items [v L, v L + L), and CTA g takes the
+// kMmaRanges ranges from kMmaRanges g on.  ws[((tile * maxseg + seg) * R + r) *
+// 128 + m] of a member receives the FP64 partial of coefficient row a of band b
+// of the tile, m = 32a + b, for the range's segment seg = v - (item_begin + tile
+// S) / L.  Accumulator groups end with a range, so a result does not depend on
+// how the ranges are dealt to the CTAs.
 // `single` is the only member when table is null (one matrix); otherwise the
 // nmem members of the table (a batch) are copied to shared memory.
 template <int RATE, bool LIFT, int NR, bool TABLE>
-__global__ void __launch_bounds__(kMmaThreads, MmaPieces<RATE>::kA == 3 ? 1 : 2)  // 3 A pieces: 120 KB of tiles
+__global__ void __launch_bounds__(kMmaDecodeThreads, 1)
     wz2_mma_kernel(MmaMember single, const MmaMember* __restrict__ table, int nmem, int64_t total, int64_t L,
                    int* __restrict__ status, uint32_t spin) {
   using SM = MmaSmem<RATE, NR>;
-  constexpr int PA = MmaPieces<RATE>::kA;
+  constexpr int PA = MmaPieces<RATE>::kA, NB = SM::kNB, NA = SM::kNA, NQ = kMmaQuartets;
   constexpr int NW = Wz2Layout<RATE>::kWords;
-  constexpr int HALF = NR / 2;  // TMEM columns drained by each of the two warps on a lane quarter
-  constexpr uint32_t kCols = mma_tmem_cols<NR>();  // two groups of three accumulators
+  constexpr int HALF = NR / 2;  // columns drained by each of the two warps on a lane quarter
+  constexpr uint32_t kACols = 8 * kMmaKSteps * PA;  // TMEM columns of a stage's A pieces
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t s_base = smem_addr(smem);
-  const uint32_t mma_bar = s_base + SM::kBars;  // two mbarriers: MMAs of buffer 0, 1 done
-  const uint32_t b_bar = mma_bar + 16;          // two mbarriers: B tile of buffer 0, 1 landed
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + SM::kBars + 32);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + SM::kBars + 36);
-  int64_t* last_commit = reinterpret_cast<int64_t*>(smem + SM::kBars + 48);  // last stage whose MMAs were committed
-  int64_t* last_copy = reinterpret_cast<int64_t*>(smem + SM::kBars + 56);    // last stage whose B copy was started
-  MmaMember* tab = reinterpret_cast<MmaMember*>(smem + SM::kBytes);          // the members
+  const uint32_t b_full = s_base + SM::kBars;  // NB: the B tile in the slot has landed
+  const uint32_t w_full = b_full + 8 * NB;     // NB: so have its compressed words (every copying thread's)
+  const uint32_t done = w_full + 8 * NB;       // NB: the MMAs of the stage in the slot are done
+  const uint32_t a_full = done + 8 * NB;       // NA: the stage's A pieces are in the buffer (4 arrivals)
+  const uint32_t gfull = a_full + 8 * NA;      // 2: the accumulator group is complete
+  const uint32_t gfree = gfull + 16;           // 2: the accumulator group has been drained (8 arrivals)
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + SM::kBars + 8 * (3 * NB + NA + 4));
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
+  MmaMember* tab = reinterpret_cast<MmaMember*>(smem + SM::kBytes);  // the members
 
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int64_t it0 = (int64_t)blockIdx.x * L;
-  const int64_t n = max((int64_t)0, min(total, it0 + L) - it0);
+  // broadcast, so that the compiler knows the roles to be warp-uniform
+  const int t = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, t >> 5, 0), lane = t & 31;
+  const int64_t it0 = (int64_t)blockIdx.x * kMmaRanges<RATE> * L;
+  const int n = (int)max((int64_t)0, min(total, it0 + kMmaRanges<RATE> * L) - it0);  // stages of this CTA
+  const int len = (int)L;
   if constexpr (TABLE)
-    for (int i = t; i < nmem; i += kMmaThreads) tab[i] = table[i];
+    for (int i = t; i < nmem; i += kMmaDecodeThreads) tab[i] = table[i];
   // member m (TABLE: of the batch's table; else the one matrix)
   auto mb = [&](int m) -> const MmaMember& {
     if constexpr (TABLE) return tab[m];
     return single;
   };
-
   if (t == 0) {
-    mbar_init(mma_bar, 1);
-    mbar_init(mma_bar + 8, 1);
-    mbar_init(b_bar, 1);
-    mbar_init(b_bar + 8, 1);
+    for (int i = 0; i < NB; ++i)
+      mbar_init(b_full + 8 * i, 1), mbar_init(w_full + 8 * i, kMmaCopyThreads), mbar_init(done + 8 * i, 1);
+    for (int i = 0; i < NA; ++i) mbar_init(a_full + 8 * i, 4);
+    for (int i = 0; i < 2; ++i) mbar_init(gfull + 8 * i, 1), mbar_init(gfree + 8 * i, 8);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     *abort_flag = 0;
-    *last_commit = *last_copy = -1;
   }
-  if (warp == 0) {  // TMEM: six accumulators of NR fp32 columns
+  if (warp == kMmaIssueWarp) {  // all of TMEM: two groups of three accumulators, then the A buffers
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_addr(tslot)),
-                 "r"(kCols));
+                 "r"(512u));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  const uint32_t tmem = *tslot;
-
-  // decode assignment: band 8(warp%4) + lane%8 of the tile, blocks jl and jl+4
-  // of the stage, jl = 8(warp/4) + lane/8
-  const int band_l = 8 * (warp & 3) + (lane & 7);
-  const int jl0 = 8 * (warp >> 2) + (lane >> 3);
-  // drain assignment: tile row 32(warp%4) + lane, accumulator columns HALF(warp/4)..
-  const int m_row = 32 * (warp & 3) + lane;
-  const int c0 = HALF * (warp >> 2);
-
-  // Cursors (member, tile, stage) of the next item to fetch, to copy B for
-  // and to issue; they advance in item order, so the loop has no divisions.
-  int mem0 = 0;
-  if constexpr (TABLE)
-    while (mem0 + 1 < nmem && tab[mem0 + 1].item_begin <= it0) ++mem0;
-  const int tile0 = (int)((it0 - mb(mem0).item_begin) / mb(mem0).S);
-  const int st0 = (int)(it0 - mb(mem0).item_begin - (int64_t)tile0 * mb(mem0).S);
-  int f_m = mem0, f_tile = tile0, f_st = st0;  // fetch
-  int m_m = mem0, m_tile = tile0, m_st = st0;  // issue
-  // the B-copy cursor (member, tile, stage) is thread 0's alone: it lives in
-  // shared memory, not in every thread's registers
-  int* b_cur = reinterpret_cast<int*>(smem + SM::kBars + 64);
-  if (t == 0) b_cur[0] = mem0, b_cur[1] = tile0, b_cur[2] = st0;
-  auto advance = [&](int& m, int& tile, int& st) {
-    if (++st == mb(m).S) {
-      st = 0, ++tile;
-      if constexpr (TABLE)
-        if (tile == tab[m].tiles) tile = 0, ++m;
-    }
-  };
-
-  uint32_t w[2][2][NW];  // compressed words of two stages (ring), 2 blocks each
-  constexpr int64_t kBlockBytes = 4 * NW;
-  // this thread's first block of the next fetch: band 32 f_tile + band_l, block 16 f_st + jl0
-  bool f_band_ok = false;
-  const uint8_t* f_ptr = nullptr;
-  auto fetch_at = [&]() {
-    const int64_t band = 32 * (int64_t)f_tile + band_l;
-    f_band_ok = band < mb(f_m).BM;
-    f_ptr = mb(f_m).stream + (band * mb(f_m).BN + 16 * (int64_t)f_st + jl0) * kBlockBytes;
-  };
-  if (n > 0) fetch_at();
-  auto fetch = [&](int slot) {
-    const int64_t J = 16 * (int64_t)f_st + jl0;
-    const int64_t BN = mb(f_m).BN;
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      if (f_band_ok && J + 4 * u < BN) {
-        wz2_load<RATE>(f_ptr, 4 * u, w[slot][u]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < NW; ++i) w[slot][u][i] = 0u;  // a zero block: E = 0, scale 0
-      }
-    }
-    const int m_before = f_m, t_before = f_tile;
-    advance(f_m, f_tile, f_st);
-    if (f_m != m_before || f_tile != t_before) {
-      if (f_m < nmem) fetch_at();
-    } else {
-      f_ptr += 16 * kBlockBytes;
-    }
-  };
-  auto b_copy = [&](int64_t k) {  // thread 0: B tile of stage k into buffer k % 2
-    const int buf = (int)(k & 1);
-    int bm = b_cur[0], bt = b_cur[1], bs = b_cur[2];
-    bulk_copy_g2s(s_base + 2 * SM::kA + buf * SM::kB, mb(bm).btiles + (int64_t)bs * SM::kB, (uint32_t)SM::kB,
-                  b_bar + 8 * buf);
-    advance(bm, bt, bs);
-    b_cur[0] = bm, b_cur[1] = bt, b_cur[2] = bs;
-    *last_copy = k;
-  };
-  auto fail = [&]() {  // a wait ran out: the CTA stops at its next barrier
+  const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, *tslot, 0);
+  static_assert(6 * NR + NA * (int)kACols <= 512, "accumulators and A buffers fit TMEM");
+  auto a_cols = [&](uint32_t k) { return tmem + (uint32_t)(6 * NR) + k % NA * kACols; };  // of stage k
+  auto fail = [&]() {  // a wait ran out: every other wait gives up
     atomicExch(status, WHFF_ETIMEOUT);
     *abort_flag = 1;
   };
-
-  float hi[HALF], lo[HALF];
-#pragma unroll
-  for (int r = 0; r < HALF; ++r) hi[r] = lo[r] = 0.f;
-  int cur_m = mem0, cur_tile = tile0;  // member and tile of the sums in hi/lo
-  auto flush = [&]() {
-    const MmaMember& me = mb(cur_m);
-    const int64_t seg = (int64_t)blockIdx.x - (me.item_begin + (int64_t)cur_tile * me.S) / L;
-    double* dst = me.ws + (((int64_t)cur_tile * me.maxseg + seg) * me.R) * 128 + m_row;
-#pragma unroll
-    for (int r = 0; r < HALF; ++r) {
-      if (c0 + r < me.R) dst[(int64_t)(c0 + r) * 128] = (double)hi[r] + (double)lo[r];
-      hi[r] = lo[r] = 0.f;
-    }
-  };
-  // drain accumulator group `acc` (its three accumulators, added), which holds
-  // a group of stages of tile `tile` of member `mem`
-  auto drain = [&](int acc, int mem, int tile) {
-    if (mem != cur_m || tile != cur_tile) {
-      flush();
-      cur_m = mem;
-      cur_tile = tile;
-    }
-    const uint32_t ta = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(3 * acc * NR + c0);
-#pragma unroll
-    for (int h = 0; h < HALF; h += 8) {
-      float v[8];
-      tmem_load_sum8(ta + h, NR, v);
-#pragma unroll
-      for (int r = 0; r < 8; r += 2) {  // TwoSum on packed pairs of columns (the same bits per half)
-        float2 H = make_float2(hi[h + r], hi[h + r + 1]), Lo = make_float2(lo[h + r], lo[h + r + 1]);
-        two_sum_acc2(H, Lo, make_float2(v[r], v[r + 1]));
-        hi[h + r] = H.x, hi[h + r + 1] = H.y, lo[h + r] = Lo.x, lo[h + r + 1] = Lo.y;
-      }
-    }
+  // a whole warp waits; false if the wait ran out (reported) or the CTA gave up
+  auto warp_wait = [&](uint32_t bar, uint32_t parity) {
+    const int r = mbar_wait_or_abort(bar, parity, spin, abort_flag);
+    const bool ran_out = __any_sync(0xFFFFFFFFu, r == 0), ok = __all_sync(0xFFFFFFFFu, r > 0);
+    if (ran_out && lane == 0) fail();
+    return ok;
   };
 
-  const uint64_t a_desc0 = smem_desc(s_base, 128, 256);
-  const uint64_t b_desc0 = smem_desc(s_base + 2 * SM::kA, 128, 256);
-  bool ok = true;  // this thread's waits all ended in time
-  // accumulator groups: up to kMmaDrainStages consecutive stages of one tile
-  // share a TMEM accumulator pair (alternating 0, 1); a group is drained after
-  // its last stage's MMAs complete
-  int gpos = 0, gacc = 0;
-  bool p_ends = false;  // stage k-1 closed its group ...
-  int p_acc = 0, p_m = mem0, p_tile = tile0;  // ... in accumulator pair p_acc, of member p_m's tile p_tile
+  // Cursor (member, tile, stage): advances in item order, so the loops have no divisions.
+  int c_m = 0;
+  if constexpr (TABLE)
+    while (c_m + 1 < nmem && tab[c_m + 1].item_begin <= it0) ++c_m;
+  int c_tile = 0, c_st = 0;
   if (n > 0) {
-    fetch(0);
-    if (t == 0) b_copy(0);
+    const MmaMember& me = mb(c_m);
+    c_tile = (int)((it0 - me.item_begin) / me.S);
+    c_st = (int)(it0 - me.item_begin - (int64_t)c_tile * me.S);
   }
-  if (n > 1) fetch(1);
-
-  // one stage; `buf` is a literal at every call, so the ring stays in registers
-  auto stage = [&](const int buf, const int64_t k) -> bool {
-    uint8_t* As = smem + buf * SM::kA;
-    // ---- A tile: this thread's 2 blocks
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int jl = jl0 + 4 * u;
-      float2 P[4][2];
-      mma_block_pairs<RATE, LIFT>(w[buf][u], P);
-      const int kstep = jl >> 2, kk = (jl & 3) * 4;
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        uint32_t d0[PA], d1[PA];
-        split_pair<PA>(P[a][0], d0);
-        split_pair<PA>(P[a][1], d1);
-        const uint32_t off = tile_off(32 * a + band_l, kk);
-#pragma unroll
-        for (int p = 0; p < PA; ++p)
-          *reinterpret_cast<uint2*>(As + (p * kMmaKSteps + kstep) * SM::kATile + off) = make_uint2(d0[p], d1[p]);
-      }
+  auto advance = [&]() {
+    if (++c_st == mb(c_m).S) {
+      c_st = 0, ++c_tile;
+      if constexpr (TABLE)
+        if (c_tile == tab[c_m].tiles) c_tile = 0, ++c_m;
     }
-    // this ring slot is free: the words of stage k+2 are on their way from here
-    // on, through the barrier, the MMA issue and the drain
-    if (k + 2 < n) fetch(buf);
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // generic writes -> tensor-core reads
-    if (!__syncthreads_and(ok ? 1 : 0)) return false;
-    // group bookkeeping of stage k (the same in every thread)
-    const bool init = gpos == 0;
-    const int acc = gacc;
-    const int tile_k = m_tile, mem_k = m_m;
-    const bool ends = ++gpos == kMmaDrainStages || m_st == mb(m_m).S - 1 || k == n - 1;
-    if (ends) gpos = 0, gacc ^= 1;
-    advance(m_m, m_tile, m_st);
-    if (t == 0) {
-      if (!mbar_wait(b_bar + 8 * buf, (uint32_t)((k >> 1) & 1), spin)) {
-        ok = false;
-        fail();
+  };
+  // Whether the item at the cursor, with range_left items of its range to go
+  // and stage k of this CTA, closes its accumulator group at position gpos.
+  auto closes = [&](int gpos, int range_left, int k) {
+    return gpos + 1 == kMmaDrainStages || c_st == mb(c_m).S - 1 || range_left == 1 || k == n - 1;
+  };
+
+  // every role's end: nothing more goes to TMEM or is read from it
+  auto leave = [&]() {
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+  };
+  if (warp >= kMmaDecodeWarp && warp < kMmaDrainWarp) {
+    // ---- decode: quartet q takes stages q, q + NQ, ...; warp w of it bands 8w .. 8w + 7
+    // of the tile, lane l band l / 4 of those and the blocks l % 4 of the four K steps.
+    const int q = (warp - kMmaDecodeWarp) >> 2, quarter = warp & 3, cb = lane & 3;
+    const int band_l = 8 * quarter + (lane >> 2);
+    for (int i = 0; i < q && i < n; ++i) advance();
+    for (int k = q; k < n; k += NQ) {
+      const MmaMember& me = mb(c_m);
+      // the lane's first block in the slot (see the copies)
+      const uint8_t* staged = smem + NB * SM::kB + (uint32_t)k % NB * SM::kWords + cb * SM::kBB;
+      if (me.paired) {
+        const int odd = ((int)me.band0 + band_l) & 1;
+        staged += (odd * (kMmaBands / 2) + (band_l >> 1)) * (SM::kRowBytes + 16) + 8 * odd;
+      } else if (me.map) {
+        staged += band_l * SM::kRowBytes;
       } else {
+        const uint32_t blk = (32 * (uint32_t)c_tile + band_l) * (uint32_t)me.BN + 16 * (uint32_t)c_st;
+        staged += band_l * (SM::kRowBytes + 16) +
+                  (((uint32_t)reinterpret_cast<uintptr_t>(me.stream) + blk * SM::kBB) & 8u);
+      }
+      if (k + NQ < n) {
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) advance();
+      }
+      if (!warp_wait(w_full + 8 * ((uint32_t)k % NB), (uint32_t)k / NB & 1u)) break;  // the words are here
+      if (k >= NA) {  // the A buffer is free once the MMAs of the stage NA before are done
+        const uint32_t p = (uint32_t)(k - NA);
+        if (!warp_wait(done + 8 * (p % NB), p / NB & 1u)) break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+      const uint32_t a_row = a_cols((uint32_t)k) + ((uint32_t)(32 * quarter) << 16);
+#pragma unroll
+      for (int u = 0; u < kMmaKSteps; ++u) {
+        uint32_t w[NW];
+        wz2_lds<RATE>(staged + 4 * u * SM::kBB, w);  // zeros past the matrix: a zero block
+        float2 P[4][2];
+        mma_block_pairs<RATE, LIFT>(w, P);
+        uint32_t d[4][2][PA];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) split_pair<PA>(P[a][h], d[a][h]);
+        __syncwarp();
+#pragma unroll
+        for (int p = 0; p < PA; ++p) {
+          const uint32_t col = a_row + (uint32_t)(8 * (p * kMmaKSteps + u));
+          tmem_store_16x256(col, d[0][0][p], d[0][1][p], d[1][0][p], d[1][1][p]);
+          tmem_store_16x256(col + (16u << 16), d[2][0][p], d[2][1][p], d[3][0][p], d[3][1][p]);
+        }
+      }
+      asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(a_full + 8 * ((uint32_t)k % NA));
+    }
+    asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+    leave();
+  } else if (warp >= kMmaDrainWarp) {
+    // ---- drain: TMEM lane 32 quarter + lane holds coefficient row a = lane / 8 of band
+    // 8 quarter + lane % 8.  A group's three accumulators are added and enter TwoSum sums.
+    const int quarter = warp & 3, m_row = 32 * (lane >> 3) + 8 * quarter + (lane & 7);
+    const int c0 = HALF * ((warp - kMmaDrainWarp) >> 2);
+    const uint32_t rows = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)c0;
+    float hi[HALF], lo[HALF];
+#pragma unroll
+    for (int r = 0; r < HALF; ++r) hi[r] = lo[r] = 0.f;
+    int cur_m = c_m, cur_tile = c_tile;  // member and tile of the sums
+    int v = (int)blockIdx.x * kMmaRanges<RATE>, left = len;  // the range, and its items from here on
+    auto flush = [&](int range) {
+      const MmaMember& me = mb(cur_m);
+      const int64_t seg = range - (me.item_begin + (int64_t)cur_tile * me.S) / L;
+      double* dst = me.ws + (((int64_t)cur_tile * me.maxseg + seg) * me.R) * 128 + m_row;
+#pragma unroll
+      for (int r = 0; r < HALF; ++r) {
+        if (c0 + r < me.R) dst[(int64_t)(c0 + r) * 128] = widen(hi[r]) + widen(lo[r]);
+        hi[r] = lo[r] = 0.f;
+      }
+    };
+    int gpos = 0, acc = 0;
+    uint32_t parity = 0;
+    bool open = false, alive = true;
+    for (int k = 0; k < n; ++k) {
+      const int m = c_m, tile = c_tile;
+      const bool ends = closes(gpos, left, k);
+      gpos = ends ? 0 : gpos + 1;
+      advance();
+      if (ends) {
+        if (!warp_wait(gfull + 8 * acc, parity)) {
+          alive = false;
+          break;
+        }
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        const uint64_t ad0 = a_desc0 + (uint64_t)((buf * SM::kA) >> 4);
-        const uint64_t bd0 = b_desc0 + (uint64_t)((buf * SM::kB) >> 4);
-        const uint32_t d0 = tmem + (uint32_t)(3 * acc * NR);
-        // A_p [B_0 .. B_{2-p}] into accumulators p..2; A_0 of the first K step
-        // of a group starts all three
+        if (open && (m != cur_m || tile != cur_tile)) flush(v);
+        cur_m = m, cur_tile = tile, open = true;
+        const uint32_t ta = rows + (uint32_t)(3 * acc * NR);
 #pragma unroll
-        for (int ks = 0; ks < kMmaKSteps; ++ks) {
+        for (int h = 0; h < HALF; h += 8) {
+          float x[8];
+          tmem_load_sum8(ta + h, NR, x);
 #pragma unroll
-          for (int pa = 0; pa < PA; ++pa) {
-            const uint64_t ad = ad0 + (uint64_t)(((pa * kMmaKSteps + ks) * SM::kATile) >> 4);
-            const uint64_t bd = bd0 + (uint64_t)((3 * ks * MmaBTile<NR>::kBTile) >> 4);
-            const uint32_t accumulate = (init && ks == 0 && pa == 0) ? 0u : 1u;
-            asm volatile(
-                "{\n\t.reg .pred p;\n\t"
-                "setp.ne.b32 p, %4, 0;\n\t"
-                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d0 + (uint32_t)(pa * NR)),
-                "l"(ad), "l"(bd), "r"(mma_idesc((3 - pa) * NR)), "r"(accumulate));
+          for (int r = 0; r < 8; r += 2) {  // TwoSum on packed pairs of columns (the same bits per half)
+            float2 H = make_float2(hi[h + r], hi[h + r + 1]), Lo = make_float2(lo[h + r], lo[h + r + 1]);
+            two_sum_acc2(H, Lo, make_float2(x[r], x[r + 1]));
+            hi[h + r] = H.x, hi[h + r + 1] = H.y, lo[h + r] = Lo.x, lo[h + r + 1] = Lo.y;
           }
         }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                         mma_bar + 8 * buf)
-                     : "memory");
-        *last_commit = k;
-      }
-    }
-    if (k >= 1) {  // stage k-1 (other buffer): wait for its MMAs; drain its group if it closed one
-      const bool done =
-          __all_sync(0xFFFFFFFFu, mbar_wait(mma_bar + 8 * (buf ^ 1), (uint32_t)(((k - 1) >> 1) & 1), spin));
-      if (!done) {
-        if (ok && lane == 0) fail();
-        ok = false;
-      } else {
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        if (t == 0 && ok && k + 1 < n) b_copy(k + 1);  // its B tile buffer is free now
-        if (p_ends) drain(p_acc, p_m, p_tile);
         asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(gfree + 8 * acc);
+        parity ^= (uint32_t)acc;
+        acc ^= 1;
       }
-    } else if (t == 0 && ok && k + 1 < n) {
-      b_copy(k + 1);
+      if (--left == 0) {
+        flush(v);
+        open = false, left = len, ++v;
+      }
     }
-    p_ends = ends;
-    p_acc = acc;
-    p_m = mem_k;
-    p_tile = tile_k;
-    return true;
-  };
-
-  bool alive = true;
-  for (int64_t k = 0; k < n && alive; k += 2) {
-    alive = stage(0, k);
-    if (alive && k + 1 < n) alive = stage(1, k + 1);
-  }
-  if (alive && n > 0) alive = __syncthreads_and(ok ? 1 : 0) != 0;
-  if (alive && n > 0) {  // the last stage, which always closes its group
-    const int buf = (int)((n - 1) & 1);
-    if (__all_sync(0xFFFFFFFFu, mbar_wait(mma_bar + 8 * buf, (uint32_t)(((n - 1) >> 1) & 1), spin))) {
+    if (alive && open) flush(v);
+    leave();
+  } else {
+    if (warp == kMmaIssueWarp) {
+      // ---- issue.  The whole warp walks the stages, so that everything the MMAs take is
+      // warp-uniform; lanes 0-2 wait for a stage's three barriers side by side (a wait costs
+      // about 250 clocks even when its phase is over), one elected lane issues.
+      int last_commit = -1, gpos = 0, acc = 0, buf = 0, slot = 0, left = len;
+      uint32_t phase = 0, a_phase = 0, g_phase = 1;  // g_phase: the groups are free at first
+      const uint64_t b_desc0 = smem_desc(s_base, 128, 256);
+#pragma unroll 1
+      for (int k = 0; k < n; ++k) {
+        const bool init = gpos == 0, ends = closes(gpos, left, k);
+        const uint32_t bar = lane == 0 ? b_full + 8 * slot : lane == 1 ? a_full + 8 * buf : gfree + 8 * acc;
+        const uint32_t par = lane == 0 ? phase : lane == 1 ? a_phase : g_phase;
+        int r = 1;
+        if (lane < (init ? 3 : 2)) r = mbar_wait_or_abort(bar, par, spin, abort_flag);
+        if (__any_sync(0xFFFFFFFFu, r <= 0)) {
+          if (r == 0) fail();
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        if (elect_one()) {
+          // A_p [B_0 .. B_{2-p}] into accumulators p..2; A_0 of the first K step of
+          // a group starts all three
+          const uint64_t bd0 = b_desc0 + (uint64_t)((slot * SM::kB) >> 4);
+          const uint32_t d0 = tmem + (uint32_t)(3 * acc * NR), a0 = a_cols((uint32_t)buf);
+#pragma unroll
+          for (int ks = 0; ks < kMmaKSteps; ++ks) {
+#pragma unroll
+            for (int pa = 0; pa < PA; ++pa) {
+              const uint32_t ad = a0 + (uint32_t)(8 * (pa * kMmaKSteps + ks));
+              const uint64_t bd = bd0 + (uint64_t)((3 * ks * MmaBTile<NR>::kBTile) >> 4);
+              const uint32_t accumulate = (init && ks == 0 && pa == 0) ? 0u : 1u;
+              asm volatile(
+                  "{\n\t.reg .pred p;\n\t"
+                  "setp.ne.b32 p, %4, 0;\n\t"
+                  "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d0 + (uint32_t)(pa * NR)),
+                  "r"(ad), "l"(bd), "r"(mma_idesc((3 - pa) * NR)), "r"(accumulate));
+            }
+          }
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(done +
+                                                                                                          8 * slot)
+                       : "memory");
+          if (ends)
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                             gfull + 8 * acc)
+                         : "memory");
+        }
+        __syncwarp();
+        last_commit = k;
+        if (ends) {
+          g_phase ^= (uint32_t)acc;
+          acc ^= 1;
+        }
+        gpos = ends ? 0 : gpos + 1;
+        advance();
+        if (--left == 0) left = len;
+        if (++buf == NA) buf = 0, a_phase ^= 1;
+        if (++slot == NB) slot = 0, phase ^= 1;
+      }
+      __syncwarp();
+      leave();
+      if (lane == 0 && *abort_flag && last_commit >= 0)  // MMAs in flight: a second bounded chance
+        (void)mbar_wait(done + 8 * (last_commit % NB), (uint32_t)((last_commit / NB) & 1));
+      __syncwarp();
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      drain(p_acc, p_m, p_tile);
-      flush();
-    } else if (lane == 0) {
-      fail();
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512u));
+    } else {
+      // ---- copies, NB stages ahead: the B tile, and the compressed words of the stage's 32
+      // bands with zeros where the matrix ends.  One tiled copy; at rates 12 and 20 with an odd
+      // number of blocks per band (rows 8 bytes off 16) two, of the even and the odd bands, the
+      // odd rows starting 8 bytes into theirs; from host memory aligned 16-byte pieces (a row
+      // may start 8 bytes into the first one).  A slot is refilled once its MMAs are done.
+      constexpr bool kShift = SM::kBB % 16 != 0;
+      constexpr int kRow = (kMmaStageBlocks * SM::kBB + (kShift ? 8 : 0) + 15) / 16;  // pieces of a band
+      // a warp takes one row (two of 16 pieces) at a time, every third
+      constexpr int kLanes = kRow <= 16 ? 16 : 32, kStep = (32 / kLanes) * (kMmaCopyThreads / 32);
+      const int r0 = (warp - kMmaCopyWarp) * (32 / kLanes) + lane / kLanes, c0 = lane % kLanes;
+      int issued = 0, slot = 0;
+      uint32_t phase = 1;  // the slots are free at first
+      for (; issued < n; ++issued) {
+        if (!warp_wait(done + 8 * slot, phase)) break;
+        const MmaMember& me = mb(c_m);
+        const uint32_t words = s_base + NB * SM::kB + slot * SM::kWords, w_bar = w_full + 8 * slot;
+        const bool tiled = me.map != nullptr;
+        if (warp == kMmaCopyWarp && elect_one()) {
+          bulk_copy_g2s(s_base + slot * SM::kB, me.btiles + (int64_t)c_st * SM::kB, (uint32_t)SM::kB, b_full + 8 * slot);
+          if (tiled) {
+            const int x = c_st * kMmaStageBlocks * NW, g = (int)(me.band0 + kMmaBands * (int64_t)c_tile);
+            if (me.paired) {  // odd and even bands, a map each
+              constexpr uint32_t kHalf = kMmaBands / 2 * (SM::kRowBytes + 16);
+              mbar_expect_tx_only(w_bar, 2 * kHalf);
+              tma_load_2d(words + (g & 1) * kHalf, static_cast<const uint8_t*>(me.map) + (g & 1) * 128, x, g >> 1, w_bar);
+              tma_load_2d(words + (~g & 1) * kHalf, static_cast<const uint8_t*>(me.map) + (~g & 1) * 128, x, (g + 1) >> 1,
+                          w_bar);
+            } else {
+              mbar_expect_tx_only(w_bar, (uint32_t)(kMmaBands * SM::kRowBytes));
+              tma_load_2d(words, me.map, x, g, w_bar);
+            }
+          }
+        }
+        __syncwarp();
+        if (tiled) {  // the copy engine brings the words
+          mbar_arrive(w_bar);
+          advance();
+          if (++slot == NB) slot = 0, phase ^= 1;
+          continue;
+        }
+        const int bands = (int)min((int64_t)kMmaBands, me.BM - kMmaBands * (int64_t)c_tile);
+        const int row_bytes = (int)min((int64_t)kMmaStageBlocks, me.BN - kMmaStageBlocks * (int64_t)c_st) * SM::kBB;
+        const uint8_t* src =
+            me.stream + (kMmaBands * (int64_t)c_tile * me.BN + kMmaStageBlocks * (int64_t)c_st) * SM::kBB;
+        const int64_t band_bytes = me.BN * SM::kBB;
+        const uint8_t* row = src + r0 * band_bytes + c0 * 16;
+        uint32_t dst = words + r0 * (SM::kRowBytes + 16) + c0 * 16;
+#pragma unroll
+        for (int i = 0; i < (kMmaBands + kStep - 1) / kStep; ++i) {
+          const int r = r0 + i * kStep;
+          const int shift = kShift ? (int)(reinterpret_cast<uintptr_t>(row) & 8u) : 0;
+#pragma unroll
+          for (int c = 0; c < kRow; c += kLanes) {
+            const int bytes = r < bands ? max(0, min(16, row_bytes + shift - 16 * (c0 + c))) : 0;
+            if (r < kMmaBands && c0 + c < kRow)
+              cp_async_zfill(dst + 16 * c, bytes ? row - shift + 16 * c : me.btiles, bytes);
+          }
+          row += kStep * band_bytes;
+          dst += kStep * (SM::kRowBytes + 16);
+        }
+        asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(w_bar) : "memory");
+        advance();
+        if (++slot == NB) slot = 0, phase ^= 1;
+      }
+      __syncwarp();
+      asm volatile("cp.async.wait_all;\n" ::: "memory");
+      leave();
+      if (warp == kMmaCopyWarp && lane == 0 && *abort_flag)  // the B tiles in flight land before the CTA goes
+        for (int k = issued > NB ? issued - NB : 0; k < issued; ++k)
+          (void)mbar_wait(b_full + 8 * (k % NB), (uint32_t)((k / NB) & 1));
     }
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  if (t == 0 && *abort_flag) {  // give the MMAs and the copy in flight a second bounded chance
-    const int64_t c = *last_commit, b = *last_copy;
-    if (c >= 0) (void)mbar_wait(mma_bar + 8 * (int)(c & 1), (uint32_t)((c >> 1) & 1));
-    if (b >= 0) (void)mbar_wait(b_bar + 8 * (int)(b & 1), (uint32_t)((b >> 1) & 1));
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols));
   }
 }
 
@@ -576,6 +693,8 @@ __global__ void __launch_bounds__(kMmaThreads, MmaPieces<RATE>::kA == 3 ? 1 : 2)
 // y (2G mix and 2^-3 with the lift, 2^3 without).  Thread per (pass, tile,
 // column, band of the tile), the band fastest, so a warp reads 32 consecutive
 // partials of one row and writes 32 consecutive 4-row groups of y.
+// Its few FP64 additions are 16 clocks a warp each; powers of two go through the
+// exponent instead.
 template <bool LIFT>
 __global__ void wz2_mma_finish(MmaPass single, const MmaPass* __restrict__ table, int n, int64_t threads, int64_t L) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -595,13 +714,13 @@ __global__ void wz2_mma_finish(MmaPass single, const MmaPass* __restrict__ table
     z[a] = seq_sum_strided(ps.ws + ((tile * ps.maxseg) * ps.R + r) * 128 + 32 * a + bl, nseg, (int64_t)ps.R * 128);
   double yy[4];
   if (LIFT) {
-    const double a = 2.0 * z[0];
-    yy[0] = (a - z[1] - z[2]) * 0.125;
-    yy[1] = (a - z[1] + z[2]) * 0.125;
-    yy[2] = (a + z[1] - z[2] - z[3]) * 0.125;
-    yy[3] = (a + z[1] + z[2] + z[3]) * 0.125;
+    const double a = times_pow2(z[0], 1), m = a - z[1], p = a + z[1];
+    yy[0] = times_pow2(m - z[2], -3);
+    yy[1] = times_pow2(m + z[2], -3);
+    yy[2] = times_pow2(p - z[2] - z[3], -3);
+    yy[3] = times_pow2(p + z[2] + z[3], -3);
   } else {
-    for (int i = 0; i < 4; ++i) yy[i] = z[i] * 8.0;
+    for (int i = 0; i < 4; ++i) yy[i] = times_pow2(z[i], 3);
   }
   for (int i = 0; i < 4; ++i)
     if (4 * I + i < ps.M) ps.y[(int64_t)r * ps.ldy + 4 * I + i] = yy[i];

@@ -149,7 +149,7 @@ int scaled_mma_occupancy(int fmt, bool tma) {
 
 namespace whff {
 
-int scaled_tma_map(void* out, const void* payload, int64_t M, int64_t ld, int fmt) {
+static PFN_cuTensorMapEncodeTiled_v12000 tma_encoder() {
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   if (!encode) {
     cudaDriverEntryPointQueryResult q;
@@ -158,10 +158,38 @@ int scaled_tma_map(void* out, const void* payload, int64_t M, int64_t ld, int fm
             cudaSuccess ||
         q != cudaDriverEntryPointSuccess || !fn) {
       cudaGetLastError();
-      return -1;
+      return nullptr;
     }
     encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   }
+  return encode;
+}
+
+int wz2_tma_map(void* out, const void* stream, int64_t BM, int64_t BN, int rate) {
+  const auto encode = tma_encoder();
+  const cuuint64_t words = (cuuint64_t)rate / 2, inner = (cuuint64_t)BN * words;
+  if (!encode || inner >= (1ull << 31) - 2 || BM >= (1ll << 31)) return 0;
+  const int maps = inner % 4 ? 2 : 1;
+  for (int k = 0; k < maps; ++k) {
+    const cuuint64_t rows = maps == 1 ? (cuuint64_t)BM : (cuuint64_t)(BM + 1 - k) / 2;
+    const cuuint64_t dims[2] = {inner + 2 * k, rows ? rows : 1};
+    const cuuint64_t strides[1] = {inner * 4 * maps};
+    const cuuint32_t box[2] = {(cuuint32_t)(16 * words + (maps == 2 ? 4 : 0)), (cuuint32_t)(32 / maps)};
+    const cuuint32_t estr[2] = {1, 1};
+    // no odd band: an empty map is not encodable, and its one row is never wanted below BM
+    const uint8_t* base = static_cast<const uint8_t*>(stream) + (k && rows ? inner * 4 - 8 : 0);
+    if (encode(reinterpret_cast<CUtensorMap*>(static_cast<uint8_t*>(out) + 128 * k), CU_TENSOR_MAP_DATA_TYPE_UINT32, 2,
+               const_cast<uint8_t*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return 0;
+  }
+  return maps;
+}
+
+int scaled_tma_map(void* out, const void* payload, int64_t M, int64_t ld, int fmt) {
+  const auto encode = tma_encoder();
+  if (!encode) return -1;
   const cuuint64_t dims[2] = {(cuuint64_t)ld, (cuuint64_t)M};
   const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};  // bytes between rows (a multiple of 16: ld % 16 == 0)
   const cuuint32_t box[2] = {64, 128};                  // 128 bytes x 128 rows: one stage

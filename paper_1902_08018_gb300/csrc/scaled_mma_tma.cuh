@@ -44,29 +44,6 @@ struct TmaSmem {
   static constexpr int kBytes = kBars + (2 * kNS + 4) * 8 + 64;
 };
 
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
-}
-
-// 2-D tiled TMA load of the box at (x, y) (x: column, a multiple of 64 BF16 =
-// 128 bytes; y: row) into shared memory (1024-byte aligned for the 128-byte
-// swizzle); completes bytes on bar.
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n" ::"r"(
-          dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
-
-// 1-D bulk copy whose bytes the caller has already announced on bar.
-__device__ __forceinline__ void bulk_g2s_tx(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst), "l"(src),
-      "r"(bytes), "r"(bar)
-      : "memory");
-}
-
 // Shared-memory descriptor of a K-major SWIZZLE_128B operand: 8-row x 128-byte
 // atoms 1024 bytes apart along M (stride byte offset), the leading byte offset
 // unused (1), descriptor version 1 (bit 46), layout type 2 = 128-byte swizzle
@@ -76,17 +53,6 @@ __device__ __forceinline__ void bulk_g2s_tx(uint32_t dst, const void* src, uint3
 __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
   return (uint64_t)((addr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) |
          (2ull << 61);
-}
-
-// Bounded wait that also gives up when the CTA's abort flag is raised:
-// 1 done, 0 timed out, -1 aborted elsewhere.
-__device__ __forceinline__ int mbar_wait_or_abort(uint32_t bar, uint32_t parity, uint32_t limit,
-                                                  const volatile int* abort_flag) {
-  for (uint32_t it = 0; it < limit; ++it) {
-    if (mbar_try_wait(bar, parity)) return 1;
-    if (*abort_flag) return -1;
-  }
-  return 0;
 }
 
 // Same items, segments and workspace layout as scaled_mma_kernel<BF16, NR>;

@@ -63,17 +63,19 @@ struct whff_handle {
   int mma_ctas = 0;
   int mma_maxseg = 1;
   int mma_min_rhs = 4;          // passes of at least this many columns use tcgen05 (whff_set_crossover, whff_tune)
-  int mma_occ = 0;              // resident tensor-core CTAs per SM
+  int mma_occ = 0;              // tensor-core item ranges per SM
   size_t ws_mma_cap = 0;        // bytes of d_ws_mma
   const float* d_scales = nullptr;  // scaled formats: the tile scales after the payload
   int64_t slice_rows = 0;       // > 0: whff_step runs as consecutive slits of this many rows
   alignas(64) unsigned char tmap[128] = {};  // BF16: TMA map of the stored matrix (tensor-core passes)
   bool has_tmap = false;
+  int map_count = 0;            // 2: the even and the odd bands (rows 8 bytes off 16)
+  uint8_t* d_map = nullptr;     // WZ2: TMA map of the stored blocks, after the B tiles (tensor-core passes)
   int64_t tma_row0 = 0;         // first row of a row view within the map's matrix
   const uint64_t* wz3_index = nullptr;  // fixed accuracy: the run index and the block area (device)
   const uint8_t* wz3_area = nullptr;
   int64_t wz3_RB = 0;           // runs per band
-  int64_t band0 = 0;            // fixed accuracy: first band of a row view
+  int64_t band0 = 0;            // WZ2, fixed accuracy: first band of a row view
   int64_t wz3_L8 = 0;           // fixed accuracy, 8 columns: (group of 8 bands, run) units per CTA
   int64_t wz3_ctas8 = 0;
   int wz3_maxseg8 = 1;          // most CTAs sharing one group
@@ -581,6 +583,17 @@ int create_impl(const BlobInfo& info, const uint8_t* src, int max_rhs, unsigned 
   // the same results for BF16, the same accuracy bar for FP16)
   if ((info.fmt == WHFF_FMT_BF16 || info.fmt == WHFF_FMT_FP16) && h->d_ws_mma && !h->h_stream)
     h->has_tmap = scaled_tma_map(h->tmap, h->d_stream, info.M, scaled_ld(info.N), info.fmt) == 0;
+  // WZ2 tensor-core passes bring device-resident blocks in by TMA, host-resident
+  // ones in 16-byte pieces: the same words, so the same results
+  alignas(64) unsigned char map[256];
+  static_assert(sizeof(map) <= kColexpBytes, "after the B tiles, where FP16 passes keep their exponents");
+  if (wz2 && h->d_ws_mma && !h->h_stream && (h->map_count = wz2_tma_map(map, h->d_stream, h->BM, h->BN, info.rate))) {
+    h->d_map = h->d_btiles + h->btile_bytes;
+    if (cudaMemcpy(h->d_map, map, sizeof(map), cudaMemcpyHostToDevice) != cudaSuccess) {
+      set_error(std::string("whff_create: tensor map upload failed: ") + cudaGetErrorString(cudaGetLastError()));
+      return fail(WHFF_ECUDA);
+    }
+  }
   *out = h;
   return WHFF_OK;
 }
@@ -611,7 +624,7 @@ int launch_mma(const whff_handle* h, const float* x, int R, int64_t ldx, double*
   if (is_blocked(h->info.fmt)) {
     MmaStep a{h->info.rate, h->info.fmt == WHFF_FMT_FIXED_LIFT, h->d_stream, h->info.M, h->info.N, h->BM, h->BN,
               x, ldx, R, h->mma_L, h->mma_ctas, h->mma_maxseg, h->d_ws_mma, h->d_btiles, y, ldy, state, decay,
-              h->d_status, h->wait_polls};
+              h->d_status, h->wait_polls, h->d_map, h->map_count == 2, h->band0};
     e = mma_launch(a, st);
   } else {
     ScaledMmaStep a{h->info.fmt, h->d_stream, h->d_scales, h->info.M, h->info.N, scaled_ld(h->info.N),
@@ -684,6 +697,7 @@ int step_view(const whff_handle* h, int64_t row0, int64_t nrows, const float* x,
   if (is_blocked(fmt)) {
     v.BM = ceil_div(nrows, 4);
     v.d_stream = h->d_stream + (uint64_t)(row0 / 4) * (uint64_t)h->BN * (uint64_t)(2 * h->info.rate);
+    v.band0 = h->band0 + row0 / 4;
   } else if (is_wz3(fmt)) {  // the same index and blocks, from band row0 / 4 on
     v.BM = ceil_div(nrows, 4);
     v.band0 = h->band0 + row0 / 4;
@@ -1543,6 +1557,9 @@ extern "C" int whff_batch_create(whff_handle* const* hs, const int* R, int count
       m.S = (int)ceil_div(h->BN, 16);
       m.tiles = (int)ceil_div(h->BM, 32);
       m.R = rp;
+      m.map = h->d_map;
+      m.paired = h->map_count == 2;
+      m.band0 = h->band0;
       m.item_begin = items;
       items += (int64_t)m.tiles * m.S;
     }

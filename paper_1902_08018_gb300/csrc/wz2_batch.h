@@ -43,6 +43,9 @@ struct MmaMember {
   int64_t BM, BN;         // block grid
   int64_t item_begin;
   int S, tiles, R, maxseg;  // stages per tile, tiles, columns of the pass, segments per tile
+  const void* map;          // CUtensorMap (device memory) of the whole stored matrix, or null
+  int paired;               // two maps: the even and the odd bands
+  int64_t band0;            // first band of this matrix (a row view) in the map
 };
 
 // The vectors of one tensor-core pass (rewritten every step): B tiles are

@@ -103,6 +103,9 @@ struct MmaStep {
   double decay;
   int* status;
   uint32_t spin;   // polls of an in-loop mbarrier wait before it gives up (kWaitPolls)
+  const void* map; // CUtensorMap in device memory of the whole stored matrix, or null
+  int paired;      // two maps, 128 bytes apart: the even and the odd bands
+  int64_t band0;   // first band of this pass in it (row views)
 };
 int mma_launch(const MmaStep& a, cudaStream_t st);
 
@@ -123,7 +126,7 @@ struct MmaBatchStep {
 };
 int mma_batch_launch(const MmaBatchStep& a, cudaStream_t st);
 int mma_max_members();  // most members of one batched launch
-// resident CTAs per SM of the tensor-core kernel at this rate for R <= nr (0 on error)
+// item ranges per SM of the tensor-core kernel at this rate for R <= nr (0 on error)
 int mma_occupancy(int rate, bool lift, int nr);
 int scaled_occupancy(int fmt, bool groups8);  // resident CTAs per SM of the R = 1 kernel
 
@@ -153,6 +156,11 @@ struct ScaledMmaStep {
   int* colexp;       // FP16 with tmap: 32 ints of scratch for the per-column exponents of x
 };
 int scaled_mma_launch(const ScaledMmaStep& a, cudaStream_t st);
+// Host: encode the TMA map of a WZ2 stream (BM bands of BN blocks, box one stage:
+// 32 bands x 16 blocks), or, where its rows are 8 bytes off 16, the maps of the
+// even and of the odd bands (box 16 bands, 16 bytes more per row; the odd rows
+// start 8 bytes in).  out: 256 bytes.  Returns the number of maps, 0 if none.
+int wz2_tma_map(void* out, const void* stream, int64_t BM, int64_t BN, int rate);
 // Host: encode the TMA map of a BF16 or FP16 (fmt 3) payload (M x ld
 // elements, row-major, box 64 x 128, 128-byte swizzle) into out (a
 // CUtensorMap, 128 bytes, 64-byte aligned); 0 on success.

@@ -93,6 +93,25 @@ __device__ __forceinline__ void wz2_load(const uint8_t* __restrict__ base, int64
   }
 }
 
+// Words of a block in shared memory (8-byte aligned at rates 12 and 20, else 16).
+template <int RATE>
+__device__ __forceinline__ void wz2_lds(const uint8_t* p, uint32_t (&w)[Wz2Layout<RATE>::kWords]) {
+  constexpr int NW = Wz2Layout<RATE>::kWords;
+  if constexpr (NW % 4 == 0) {
+#pragma unroll
+    for (int i = 0; i < NW / 4; ++i) {
+      const uint4 v = *reinterpret_cast<const uint4*>(p + 16 * i);
+      w[4 * i] = v.x, w[4 * i + 1] = v.y, w[4 * i + 2] = v.z, w[4 * i + 3] = v.w;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < NW / 2; ++i) {
+      const uint2 v = *reinterpret_cast<const uint2*>(p + 8 * i);
+      w[2 * i] = v.x, w[2 * i + 1] = v.y;
+    }
+  }
+}
+
 // Field k of a block, already times the block scale s = 2^e: the field is
 // OR-ed into the mantissa of 2^(e+23) (creg = its exponent bits) and
 // 2^e (2^23 + 2^(W-1)) (bias) is subtracted -- both exact, so this is

@@ -43,25 +43,6 @@ struct Wz2Stream {
   static constexpr int kSmemBytes = kWarpsPerCta * (kRingBytes + 8 * kNS);
 };
 
-// Words of lane block `b` of a slot (8-byte aligned in shared memory).
-template <int RATE>
-__device__ __forceinline__ void wz2_lds(const uint8_t* p, uint32_t (&w)[Wz2Layout<RATE>::kWords]) {
-  constexpr int NW = Wz2Layout<RATE>::kWords;
-  if constexpr (Wz2Stream<RATE>::kBB % 16 == 0) {
-#pragma unroll
-    for (int i = 0; i < NW / 4; ++i) {
-      const uint4 v = *reinterpret_cast<const uint4*>(p + 16 * i);
-      w[4 * i] = v.x, w[4 * i + 1] = v.y, w[4 * i + 2] = v.z, w[4 * i + 3] = v.w;
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < NW / 2; ++i) {
-      const uint2 v = *reinterpret_cast<const uint2*>(p + 8 * i);
-      w[2 * i] = v.x, w[2 * i + 1] = v.y;
-    }
-  }
-}
-
 // The warp's position in its sequence of stages: band I, blocks [J, Jend) of
 // the band still to stream (Jend = the end of the range's piece of band I).
 struct StageCursor {
