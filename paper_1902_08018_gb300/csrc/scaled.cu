@@ -10,11 +10,11 @@ static void scaled_one(const ScaledStep& a, cudaStream_t st) {
   if (a.groups8)
     dev::scaled_range_kernel<FMT, R, 8><<<(unsigned)a.ctas, dev::kWarpsPerCta * 32, 0, st>>>(
         a.payload, a.scales, a.M, a.N, a.ld, a.TN, a.x, a.ldx, a.x_vec_ok, a.L, a.maxseg, a.ws, a.y, a.ldy, a.state,
-        a.decay, a.red32);
+        a.decay, a.red32, a.seen);
   else
     dev::scaled_range_kernel<FMT, R, 32><<<(unsigned)a.ctas, dev::kWarpsPerCta * 32, 0, st>>>(
         a.payload, a.scales, a.M, a.N, a.ld, a.TN, a.x, a.ldx, a.x_vec_ok, a.L, a.maxseg, a.ws, a.y, a.ldy, a.state,
-        a.decay, a.red32);
+        a.decay, a.red32, a.seen);
 }
 
 template <int FMT>
@@ -30,21 +30,13 @@ static int scaled_fmt(const ScaledStep& a, cudaStream_t st) {
 }
 
 int scaled_launch(const ScaledStep& a, cudaStream_t st) {
-  int e;
   switch (a.fmt) {
-    case 2: e = scaled_fmt<2>(a, st); break;
-    case 3: e = scaled_fmt<3>(a, st); break;
-    case 4: e = scaled_fmt<4>(a, st); break;
-    case 7: e = scaled_fmt<7>(a, st); break;
+    case 2: return scaled_fmt<2>(a, st);
+    case 3: return scaled_fmt<3>(a, st);
+    case 4: return scaled_fmt<4>(a, st);
+    case 7: return scaled_fmt<7>(a, st);
     default: return -1;
   }
-  if (e) return e;
-  if (a.maxseg > 1) {  // shared bands: the chunks of a band are the "blocks" of the segment epilogue
-    const int V = scaled_vec(a.fmt);
-    dev::wz2_segment_epilogue<<<(unsigned)((dev::segment_epilogue_threads(a.M, a.ld / V, a.L) + 255) / 256), 256, 0, st>>>(a.ws, a.M, a.ld / V, a.L, a.maxseg,
-                                                                            a.R, a.y, a.ldy, a.state, a.decay);
-  }
-  return 0;
 }
 
 template <int FMT>

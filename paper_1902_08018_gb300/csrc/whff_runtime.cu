@@ -38,6 +38,7 @@ struct whff_handle {
   uint8_t* h_stream = nullptr;  // host-resident handles: the pinned, mapped host copy behind d_stream
   double* d_ws = nullptr;       // split-K partials: ksplit x max_rhs x Mpad
   size_t ws_bytes = 0;
+  int* d_seen = nullptr;        // per band: segments of the running pass written so far, zero between passes
   int* d_status = nullptr;      // device-side error word
   float* d_x = nullptr;         // staging for whff_step_host
   double* d_y = nullptr;
@@ -257,7 +258,7 @@ int launch_wz2(const whff_handle* h, const float* x, int R, int64_t ldx, bool ve
                       reinterpret_cast<uintptr_t>(h->d_stream) % (h->info.rate % 8 == 0 ? 16 : 8) == 0;
   Wz2Step a{h->d_stream, h->info.M, h->info.N, h->BM, h->BN, x, ldx, vec, h->range_len, h->maxseg, h->d_ws,
             y, ldy, state, decay, h->range_ctas, R == 1 ? h->unroll : 2, h->info.fmt == WHFF_FMT_FIXED_LIFT, R,
-            h->red32, h->groups8, h->d_xt, staged, h->d_status};
+            h->red32, h->groups8, h->d_xt, staged, h->d_status, h->d_seen};
   int e;
   switch (h->info.rate) {
     case 8: e = wz2_launch<8>(a, st); break;
@@ -301,7 +302,7 @@ int launch_scaled(const whff_handle* h, const float* x, int R, int64_t ldx, bool
   const auto& b = h->info;
   const int64_t ld = scaled_ld(b.N);
   ScaledStep a{b.fmt, h->d_stream, h->d_scales, b.M, b.N, ld, ceil_div(b.N, kScaleTile), x, ldx, vec,
-               h->range_len, h->maxseg, h->d_ws, y, ldy, state, decay, h->range_ctas, R, h->red32, h->groups8};
+               h->range_len, h->maxseg, h->d_ws, y, ldy, state, decay, h->range_ctas, R, h->red32, h->groups8, h->d_seen};
   if (scaled_launch(a, st)) {
     set_error("whff_step: scaled formats take R 1, 2, 4 or 8 per pass");
     return WHFF_EINVAL;
@@ -331,7 +332,7 @@ int launch_pass(const whff_handle* h, const float* x, int R, int64_t ldx, double
       const bool wide = R == 8;
       Wz3Step a{h->wz3_index, h->wz3_area, h->band0, h->info.M, h->info.N, h->BM, h->BN, h->wz3_RB, x, ldx,
                 h->d_xt, R, wide ? h->wz3_L8 : h->range_len, wide ? h->wz3_maxseg8 : h->maxseg,
-                wide ? h->wz3_ctas8 : h->range_ctas, h->d_ws, y, ldy, state, decay};
+                wide ? h->wz3_ctas8 : h->range_ctas, h->d_ws, y, ldy, state, decay, h->d_seen};
       e = wz3_launch(a, st) ? WHFF_EINVAL : WHFF_OK;
       if (e) set_error("whff_step: fixed-accuracy passes take 1 or 8 right-hand sides");
       break;
@@ -557,6 +558,7 @@ int create_impl(const BlobInfo& info, const uint8_t* src, int max_rhs, unsigned 
   if (((info.fmt == WHFF_FMT_FIXED_LIFT || is_wz3(info.fmt)) && cudaMalloc(&h->d_xt, xt_bytes(h)) != cudaSuccess) ||
       (h->ws_bytes && cudaMalloc(&h->d_ws, h->ws_bytes) != cudaSuccess) ||
       cudaMalloc(&h->d_status, sizeof(int)) != cudaSuccess ||
+      cudaMalloc(&h->d_seen, (size_t)h->BM * sizeof(int)) != cudaSuccess ||
       cudaMalloc(&h->d_x, (size_t)info.N * (size_t)max_rhs * sizeof(float)) != cudaSuccess ||
       cudaMalloc(&h->d_y, (size_t)info.M * (size_t)max_rhs * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
@@ -564,6 +566,7 @@ int create_impl(const BlobInfo& info, const uint8_t* src, int max_rhs, unsigned 
     return fail(WHFF_ENOMEM);
   }
   if (cudaMemsetAsync(h->d_status, 0, sizeof(int), st) != cudaSuccess ||
+      cudaMemsetAsync(h->d_seen, 0, (size_t)h->BM * sizeof(int), st) != cudaSuccess ||
       (!h->h_stream && src &&
        cudaMemcpyAsync(h->d_stream, src, info.stream_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess) ||
       cudaStreamSynchronize(st) != cudaSuccess) {
@@ -610,7 +613,7 @@ extern "C" int whff_info(const whff_handle* h, int* fmt, int* rate, int64_t* M, 
   if (M) *M = h->info.M;
   if (N) *N = h->info.N;
   if (device_bytes)
-    *device_bytes = (h->h_stream ? 0 : h->info.stream_bytes) + h->ws_bytes + h->ws_mma_bytes + sizeof(int) +
+    *device_bytes = (h->h_stream ? 0 : h->info.stream_bytes) + h->ws_bytes + h->ws_mma_bytes + sizeof(int) + (size_t)h->BM * sizeof(int) +
                     (size_t)h->info.N * h->max_rhs * 4 + (size_t)h->info.M * h->max_rhs * 8 +
                     (h->d_xt ? xt_bytes(h) : 0);
   return WHFF_OK;
@@ -651,7 +654,7 @@ extern "C" int whff_plan(const whff_handle* h, int* ksplit, int* launches) {
   }
   if (ksplit) *ksplit = h->ksplit;
   if (launches)
-    *launches = ((h->ksplit > 1 || h->maxseg > 1) ? 2 : 1) +
+    *launches = (h->ksplit > 1 || (h->maxseg > 1 && h->bulk) ? 2 : 1) +
                 (h->info.fmt == WHFF_FMT_FIXED_LIFT || is_wz3(h->info.fmt) ? 1 : 0);
   return WHFF_OK;
 }
@@ -1150,6 +1153,7 @@ extern "C" void whff_destroy(whff_handle* h) {
   cudaFree(h->d_btiles);
   cudaFree(h->d_xt);
   cudaFree(h->d_status);
+  cudaFree(h->d_seen);
   cudaFree(h->d_x);
   cudaFree(h->d_y);
   cudaGetLastError();

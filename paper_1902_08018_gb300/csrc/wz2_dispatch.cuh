@@ -11,7 +11,7 @@ template <int RATE, bool LIFT, int R, int U, int GL = 32>
 static void wz2_launch_one(const Wz2Step& a, cudaStream_t st) {
   dev::wz2_gemv_kernel<RATE, LIFT, R, U, GL><<<(unsigned)a.ctas, dev::kWarpsPerCta * 32, 0, st>>>(
       a.stream, a.M, a.N, a.BM, a.BN, a.x, a.ldx, a.x_vec_ok, a.L, a.maxseg, a.ws, a.y, a.ldy, a.state, a.decay,
-      a.red32);
+      a.red32, a.seen);
 }
 
 template <int RATE, bool LIFT>
@@ -35,6 +35,9 @@ static int wz2_launch_lift(const Wz2Step& a, cudaStream_t st) {
     dev::wz2_stream_kernel<RATE, LIFT><<<(unsigned)a.ctas, dev::kWarpsPerCta * 32, dev::Wz2Stream<RATE>::kSmemBytes,
                                          st>>>(a.stream, a.M, a.N, a.BM, a.BN, a.x, a.ldx, a.x_vec_ok, a.L, a.maxseg,
                                                a.ws, a.y, a.ldy, a.state, a.decay, a.red32, a.status);
+    if (a.maxseg > 1)
+      dev::wz2_segment_epilogue<<<(unsigned)((dev::segment_epilogue_threads(a.M, a.BN, a.L) + 255) / 256), 256, 0, st>>>(
+          a.ws, a.M, a.BN, a.L, a.maxseg, a.R, a.y, a.ldy, a.state, a.decay);
   } else if (a.groups8) {  // short bands: four 8-lane groups per warp, two blocks in flight per lane
     switch (a.R) {
       case 1: wz2_launch_one<RATE, LIFT, 1, 2, 8>(a, st); break;
@@ -54,9 +57,6 @@ static int wz2_launch_lift(const Wz2Step& a, cudaStream_t st) {
     case 8: wz2_launch_one<RATE, LIFT, 8, 2>(a, st); break;
     default: return -1;
   }
-  if (a.maxseg > 1)
-    dev::wz2_segment_epilogue<<<(unsigned)((dev::segment_epilogue_threads(a.M, a.BN, a.L) + 255) / 256), 256, 0, st>>>(a.ws, a.M, a.BN, a.L, a.maxseg, a.R,
-                                                                            a.y, a.ldy, a.state, a.decay);
   return 0;
 }
 

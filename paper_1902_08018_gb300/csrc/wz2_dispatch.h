@@ -35,6 +35,7 @@ struct Wz2Step {
   float* xt;       // lift: scratch for (2G)^T x, 4 BN floats per right-hand side (8 columns)
   bool staged;     // R = 1: stream each warp's range through shared memory by bulk copies
   int* status;     // device status word (bounded waits of the staged kernel)
+  int* seen;       // per band: segments of the pass written so far (zero between passes)
 };
 
 // Bytes a handle's device stream allocation carries past the stream, so that
@@ -80,6 +81,7 @@ struct ScaledStep {
   int R;
   bool red32;
   bool groups8;  // four 8-lane groups per warp, one band each (short bands)
+  int* seen;     // per band: segments written so far
 };
 int scaled_launch(const ScaledStep& a, cudaStream_t st);  // scaled.cu
 
@@ -170,8 +172,8 @@ int scaled_mma_occupancy(int fmt, bool tma);
 
 // Fixed-accuracy (WZ3) pass: (2G)^T x, then persistent ranges (R = 1: a warp's,
 // of L runs of the pass's bands in band-major order; R = 8: a CTA's, of L
-// (group of 8 bands, run) units), then (maxseg > 1) the epilogue for bands
-// shared by several ranges.  band0 is the first band of a
+// (group of 8 bands, run) units); the last range of a shared band adds its
+// segments.  band0 is the first band of a
 // row view within the matrix (its index is the matrix's).
 struct Wz3Step {
   const uint64_t* index;  // the matrix's run index (BM_total x RB)
@@ -190,6 +192,7 @@ struct Wz3Step {
   int64_t ldy;
   double* state;
   double decay;
+  int* seen;      // per band: segments written so far
 };
 int wz3_launch(const Wz3Step& a, cudaStream_t st);
 int wz3_occupancy();  // resident CTAs per SM of the R = 1 kernel (0 on error)

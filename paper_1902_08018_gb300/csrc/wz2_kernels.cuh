@@ -407,13 +407,74 @@ static __global__ void wz2_xt_kernel(const float* __restrict__ x, int64_t ldx, i
   *reinterpret_cast<float4*>(xt + (int64_t)r * ldt + 4 * J) = make_float4(2.f * (a + b), b - a, d - c, xv[3] - xv[2]);
 }
 
+// The segments [0, nseg) of shared band I added up into y, then the state update.
+// The whole warp calls it: 8 lanes per row of the band, lane j adds segments j,
+// j + 8, ... in order, then a fixed xor tree over the eight (the same order every
+// time, so the result is deterministic; with one or two segments it is the plain
+// sum).  A slit of a long matrix has dozens of segments per band: eight lanes keep
+// their loads in flight together.  The partials come from other SMs: not from L1.
+__device__ __forceinline__ void sum_segments(const double* __restrict__ ws, int64_t I, int64_t M, int nseg, int maxseg,
+                                             int R, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
+                                             double decay, bool valid) {
+  const int lane = threadIdx.x & 31, i = lane >> 3, j = lane & 7;
+  const int64_t row = 4 * I + i;
+  valid = valid && row < M;
+  double s = (valid && state) ? state[row] : 0.0;
+  for (int r = 0; r < R; ++r) {
+    double t = 0.0;
+    if (valid)
+      for (int seg = j; seg < nseg; seg += 8) t += __ldcg(ws + ((I * maxseg + seg) * R + r) * 4 + i);
+#pragma unroll
+    for (int o = 4; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (valid && j == 0) {
+      y[(int64_t)r * ldy + row] = t;
+      s = decay * s + t;
+    }
+  }
+  if (valid && j == 0 && state) state[row] = s;
+}
+
+// After a warp has written its segment of shared band I: the warp that brings the
+// band's last of nseg segments adds them up (the order of the sum is the segments',
+// whoever does it), and leaves the band's counter at zero for the next pass.  A
+// kernel of its own for these few sums cost 4 us of launch and latency per pass.
+__device__ __forceinline__ void finish_shared_band(int* __restrict__ seen, const double* __restrict__ ws, int64_t I,
+                                                   int64_t M, int nseg, int maxseg, int R, double* __restrict__ y,
+                                                   int64_t ldy, double* __restrict__ state, double decay) {
+  __threadfence();
+  __syncwarp();
+  int last = 0;
+  if ((threadIdx.x & 31) == 0) {
+    last = atomicAdd(seen + I, 1) == nseg - 1;
+    if (last) seen[I] = 0;
+  }
+  last = __shfl_sync(0xffffffffu, last, 0);
+  if (!last) return;
+  __threadfence();
+  sum_segments(ws, I, M, nseg, maxseg, R, y, ldy, state, decay, true);
+}
+
+// The same for the four lane groups of a warp, each with a piece of a band of its own.
+template <int GL>
+__device__ __forceinline__ void finish_shared_groups(int* __restrict__ seen, const double* __restrict__ ws, int64_t I,
+                                                     int64_t M, int nseg, bool shared, int maxseg, int R,
+                                                     double* __restrict__ y, int64_t ldy, double* __restrict__ state,
+                                                     double decay) {
+  if (!__any_sync(0xffffffffu, shared)) return;
+#pragma unroll 1
+  for (int g = 0; g < 32; g += GL) {
+    if (!__shfl_sync(0xffffffffu, (int)shared, g)) continue;
+    finish_shared_band(seen, ws, __shfl_sync(0xffffffffu, I, g), M, __shfl_sync(0xffffffffu, nseg, g), maxseg, R, y,
+                       ldy, state, decay);
+  }
+}
+
 // Persistent kernel with exact balance: the G warps of the grid split the
 // band-major sequence of all BM*BN blocks into G contiguous ranges of L
 // blocks.  A range covers pieces of one to a few 4-row bands; for every piece
 // the lanes' sums are folded and either y (and the state) is written
 // directly, when the band lies inside one range, or the piece's partial goes
-// to ws[band][segment] for wz2_segment_epilogue, which adds a band's segments
-// in order.  GL = 32: the warp takes one piece at a time; GL = 8: four lane
+// to ws[band][segment], and the band's last warp adds its segments in order.  GL = 32: the warp takes one piece at a time; GL = 8: four lane
 // groups take the next four pieces at once (short bands, where a warp per
 // band would spend its time folding).  With the lift, x is the transformed
 // vector of wz2_xt_kernel (4 BN floats per right-hand side).
@@ -421,7 +482,7 @@ template <int RATE, bool LIFT, int R, int UNROLL, int GL>
 __device__ __forceinline__ void wz2_gemv_body(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM,
                                               int64_t BN, const float* __restrict__ x, int64_t ldx, bool x_vec_ok,
                                               int64_t L, int maxseg, double* __restrict__ ws, double* __restrict__ y,
-                                              int64_t ldy, double* __restrict__ state, double decay, bool red32) {
+                                              int64_t ldy, double* __restrict__ state, double decay, bool red32, int* __restrict__ seen) {
   constexpr int64_t kBlockBytes = 4 * Wz2Layout<RATE>::kWords;
   constexpr int NG = 32 / GL;  // pieces taken at once
   const int lane = threadIdx.x & 31;
@@ -445,8 +506,10 @@ __device__ __forceinline__ void wz2_gemv_body(const uint8_t* __restrict__ stream
       // a band inside one range is finished here, a shared one leaves a segment:
       // ws[(band * maxseg + seg) * R + r][i]
       const int64_t g_lo = div64(I * BN, L), g_hi = div64((I + 1) * BN - 1, L);
-      band_finish<LIFT ? 1 : 2, R>(hi, lo, lane, 4 * I, M, g_lo == g_hi ? nullptr : ws + (I * maxseg + (g - g_lo)) * R * 4,
-                                   y, ldy, state, decay, red32);
+      const bool shared = g_lo != g_hi;
+      band_finish<LIFT ? 1 : 2, R>(hi, lo, lane, 4 * I, M, shared ? ws + (I * maxseg + (g - g_lo)) * R * 4 : nullptr, y,
+                                   ldy, state, decay, red32);
+      if (shared) finish_shared_band(seen, ws, I, M, (int)(g_hi - g_lo + 1), maxseg, R, y, ldy, state, decay);
       b0 = piece_end;
     } else {  // lane group lane / GL takes the piece of band b0 / BN + lane / GL
       const int64_t I0 = div64(b0, BN), I = I0 + lane / GL;
@@ -457,9 +520,10 @@ __device__ __forceinline__ void wz2_gemv_body(const uint8_t* __restrict__ stream
                                                    pe - I * BN, gl, x, ldx, N, x_fast, x_vec_ok, hi, lo);
       // one call for all groups (the folds shuffle across the whole warp)
       const int64_t g_lo = div64(I * BN, L), g_hi = div64((I + 1) * BN - 1, L);
-      band_finish<LIFT ? 1 : 2, R, GL>(hi, lo, gl, 4 * I, M,
-                                       g_lo == g_hi ? nullptr : ws + (I * maxseg + (g - g_lo)) * R * 4, y, ldy, state,
-                                       decay, red32, active);
+      const bool shared = active && g_lo != g_hi;
+      band_finish<LIFT ? 1 : 2, R, GL>(hi, lo, gl, 4 * I, M, shared ? ws + (I * maxseg + (g - g_lo)) * R * 4 : nullptr, y,
+                                       ldy, state, decay, red32, active);
+      finish_shared_groups<GL>(seen, ws, I, M, (int)(g_hi - g_lo + 1), shared, maxseg, R, y, ldy, state, decay);
       b0 = min(b1, (I0 + NG) * BN);
     }
   }
@@ -480,9 +544,9 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? wz2_ctas_per_sm<RA
     wz2_gemv_kernel(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM, int64_t BN,
                     const float* __restrict__ x, int64_t ldx, bool x_vec_ok, int64_t L, int maxseg,
                     double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
-                    double decay, bool red32) {
+                    double decay, bool red32, int* __restrict__ seen) {
   wz2_gemv_body<RATE, LIFT, R, UNROLL, GL>(stream, M, N, BM, BN, x, ldx, x_vec_ok, L, maxseg, ws, y, ldy, state,
-                                           decay, red32);
+                                           decay, red32, seen);
 }
 
 // sum_{k < n} p[k * stride], added in k order; the loads of eight terms are
@@ -503,16 +567,11 @@ __device__ __forceinline__ double seq_sum_strided(const double* __restrict__ p, 
   return t;
 }
 
-// Sum the segments of bands shared by several warp ranges, then the state
-// update (bands inside one range were finished by the kernel).  The shared
-// bands are exactly those with a range boundary b = g L strictly inside them
-// (b not a multiple of BN); each is taken by the warp of its first such
-// boundary, so the launch has a warp per boundary (segment_epilogue_threads),
-// not a thread per row.  In that warp, 8 lanes per row of the band: lane j
-// adds segments j, j + 8, ... in order, then a fixed xor tree over the eight
-// (the same order every time, so the result is deterministic; with one or two
-// segments it is the plain sum).  A slit of a long matrix has dozens of
-// segments per band: eight lanes keep their loads in flight together.
+// The sums of shared bands as a launch of their own (the bulk-staged kernel, whose
+// warps may give up): the shared bands are exactly those with a range boundary
+// b = g L strictly inside them (b not a multiple of BN); each is taken by the warp
+// of its first such boundary, so the launch has a warp per boundary
+// (segment_epilogue_threads), not a thread per row.
 __host__ __device__ inline int64_t segment_epilogue_threads(int64_t M, int64_t BN, int64_t L) {
   const int64_t total = ((M + 3) / 4) * BN, ranges = (total + L - 1) / L;
   return ranges > 1 ? 32 * (ranges - 1) : 0;
@@ -523,27 +582,12 @@ static __global__ void wz2_segment_epilogue(const double* __restrict__ ws, int64
                                             double* __restrict__ state, double decay) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t g = 1 + (q >> 5);  // the boundary of this warp (warp-uniform)
-  const int i = (int)((q & 31) >> 3), j = (int)(q & 7);
   const int64_t b = g * L, total = ((M + 3) / 4) * BN;
   const int64_t I = div64(b, BN);
   // a boundary inside band I, and the first one there (the previous one is not inside I)
   const bool mine = b < total && b != I * BN && (g - 1) * L <= I * BN;
-  const int64_t row = 4 * I + i;
-  const bool valid = mine && row < M;
   const int64_t g_lo = div64(I * BN, L), g_hi = div64((I + 1) * BN - 1, L);
-  double s = (valid && state) ? state[row] : 0.0;
-  for (int r = 0; r < R; ++r) {
-    double t = 0.0;
-    if (valid)
-      for (int64_t seg = j; seg <= g_hi - g_lo; seg += 8) t += ws[((I * maxseg + seg) * R + r) * 4 + i];
-#pragma unroll
-    for (int o = 4; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (valid && j == 0) {
-      y[(int64_t)r * ldy + row] = t;
-      s = decay * s + t;
-    }
-  }
-  if (valid && j == 0 && state) state[row] = s;
+  sum_segments(ws, I, M, (int)(g_hi - g_lo + 1), maxseg, R, y, ldy, state, decay, mine);
 }
 
 // ------------------------------------------------------------- batched launch

@@ -12,19 +12,13 @@ int wz3_launch(const Wz3Step& a, cudaStream_t st) {
   if (a.R == 8) {
     dev::wz3_xt8_kernel<<<(unsigned)a.RB, 256, 0, st>>>(a.x, a.ldx, a.N, a.RB, a.xt);
     dev::wz3_gemv8_kernel<<<(unsigned)a.ctas, threads, 0, st>>>(index, a.area, a.M, a.BM, (int)a.BN, (int)a.RB, a.xt,
-                                                                a.L, a.maxseg, a.ws, a.y, a.ldy, a.state, a.decay);
-    if (a.maxseg > 1)
-      dev::wz3_epilogue8_kernel<<<(unsigned)(a.ctas - 1), 256, 0, st>>>(a.ws, a.M, a.BM, a.RB, a.L, a.maxseg, a.y,
-                                                                        a.ldy, a.state, a.decay);
+                                                                a.L, a.maxseg, a.ws, a.y, a.ldy, a.state, a.decay, a.seen);
     return 0;
   }
   const int64_t ldt = 4 * a.BN;
   dev::wz2_xt_kernel<<<(unsigned)((a.BN + 255) / 256), 256, 0, st>>>(a.x, a.ldx, a.N, 1, a.BN, a.xt, ldt);
   dev::wz3_gemv_kernel<1><<<(unsigned)a.ctas, threads, 0, st>>>(index, a.area, a.M, a.BM, (int)a.BN, (int)a.RB, a.xt,
-                                                                ldt, a.L, a.maxseg, a.ws, a.y, a.ldy, a.state, a.decay);
-  if (a.maxseg > 1)  // units per band: runs
-    dev::wz2_segment_epilogue<<<(unsigned)((dev::segment_epilogue_threads(a.M, a.RB, a.L) + 255) / 256), 256, 0, st>>>(
-        a.ws, a.M, a.RB, a.L, a.maxseg, a.R, a.y, a.ldy, a.state, a.decay);
+                                                                ldt, a.L, a.maxseg, a.ws, a.y, a.ldy, a.state, a.decay, a.seen);
   return 0;
 }
 

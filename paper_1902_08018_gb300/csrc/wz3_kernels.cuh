@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
     wz3_gemv_kernel(const uint64_t* __restrict__ index, const uint8_t* __restrict__ area, int64_t M, int64_t BM,
                     int BN, int RB, const float* __restrict__ xt, int64_t ldt, int64_t L, int maxseg,
                     double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
-                    double decay) {
+                    double decay, int* __restrict__ seen) {
   const int lane = threadIdx.x & 31;
   const int64_t g = (int64_t)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
   const int64_t total = BM * RB;
@@ -193,8 +193,10 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
       }
     }
     const int64_t g_lo = div64(I * RB, L), g_hi = div64((I + 1) * RB - 1, L);
-    band_finish<1, R>(hi, lo, lane, 4 * I, M, g_lo == g_hi ? nullptr : ws + (I * maxseg + (g - g_lo)) * R * 4, y, ldy,
-                      state, decay, false);
+    const bool shared = g_lo != g_hi;
+    band_finish<1, R>(hi, lo, lane, 4 * I, M, shared ? ws + (I * maxseg + (g - g_lo)) * R * 4 : nullptr, y, ldy, state,
+                      decay, false);
+    if (shared) finish_shared_band(seen, ws, I, M, (int)(g_hi - g_lo + 1), maxseg, R, y, ldy, state, decay);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -272,7 +274,7 @@ __device__ __forceinline__ int64_t wz3_groups(int64_t BM) { return (BM + 7) / 8;
 static __global__ void __launch_bounds__(kWarpsPerCta * 32, 2)
     wz3_gemv8_kernel(const uint64_t* __restrict__ index, const uint8_t* __restrict__ area, int64_t M, int64_t BM,
                      int BN, int RB, const float* __restrict__ xt, int64_t L, int maxseg, double* __restrict__ ws,
-                     double* __restrict__ y, int64_t ldy, double* __restrict__ state, double decay) {
+                     double* __restrict__ y, int64_t ldy, double* __restrict__ state, double decay, int* __restrict__ seen) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t u0 = (int64_t)blockIdx.x * L, u1 = min(wz3_groups(BM) * RB, u0 + L);
   for (int64_t ub = u0; ub < u1;) {  // the range's piece of group G: runs [q0, q1) of each of its bands
@@ -316,24 +318,11 @@ static __global__ void __launch_bounds__(kWarpsPerCta * 32, 2)
     double z[1];
     fold_lanes<32, 32, false, true>(h, l, lane, z);
     const int64_t c_lo = div64(G * RB, L), c_hi = div64((G + 1) * RB - 1, L);
-    band_write<1, 8, 32>(z, lane, 4 * I, M, c_lo == c_hi ? nullptr : ws + (I * maxseg + (blockIdx.x - c_lo)) * 32, y,
-                         ldy, state, decay, true);
+    const bool shared = c_lo != c_hi;
+    band_write<1, 8, 32>(z, lane, 4 * I, M, shared ? ws + (I * maxseg + (blockIdx.x - c_lo)) * 32 : nullptr, y, ldy,
+                         state, decay, true);
+    if (shared) finish_shared_band(seen, ws, I, M, (int)(c_hi - c_lo + 1), maxseg, 8, y, ldy, state, decay);
   }
-}
-
-// The bands of groups shared by several CTAs: their segments added in order.
-// A warp per (range boundary, band of the group it cuts); the first boundary
-// inside a group does the work.
-static __global__ void __launch_bounds__(256)
-    wz3_epilogue8_kernel(const double* __restrict__ ws, int64_t M, int64_t BM, int64_t RB, int64_t L, int maxseg,
-                         double* __restrict__ y, int64_t ldy, double* __restrict__ state, double decay) {
-  const int lane = threadIdx.x & 31;
-  const int64_t c = 1 + (int64_t)blockIdx.x, b = c * L;
-  const int64_t G = b / RB, I = 8 * G + (threadIdx.x >> 5);
-  if (b >= wz3_groups(BM) * RB || b % RB == 0 || (c - 1) * L > G * RB || I >= BM) return;
-  const int64_t c_lo = (G * RB) / L, c_hi = ((G + 1) * RB - 1) / L;
-  double z[1] = {seq_sum_strided(ws + I * maxseg * 32 + lane, c_hi - c_lo + 1, 32)};
-  band_write<0, 8, 32>(z, lane, 4 * I, M, nullptr, y, ldy, state, decay, true);
 }
 
 // Decode: thread per block, the exact definition -- T = (2G) V (2G)^T in

@@ -42,3 +42,33 @@ def test_totals_beyond_fp32(env, orc, fmt, rate, exp, R):
         torch.cuda.synchronize()
         got = y.cpu().numpy()
     assert (got == X.astype(np.float64) @ A.T).all()
+
+
+@pytest.mark.parametrize("fmt,rate", [(5, 8), (5, 16), (6, 24), (2, 0), (4, 0), (7, 0), (8, 0)])
+@pytest.mark.parametrize("M,N", [(30, 40000), (700, 3001), (5000, 378)])
+def test_shared_bands_pass_after_pass(env, fmt, rate, M, N):
+    """A band's last segment adds them all up and leaves its counter at zero: whole
+    steps, row views and other column counts on one handle repeat bit for bit."""
+    W, torch = env
+    A = np.random.default_rng(M + fmt).standard_normal((M, N))
+    blob = W.whff_compress_accuracy(A, 1e-4) if fmt == 8 else W.whff_compress(A, fmt, rate or 16)
+    x = torch.from_numpy(np.random.default_rng(N).standard_normal((8, N)).astype(np.float32)).cuda()
+    with W.whff_create(blob, max_rhs=8) as h:
+        if fmt in (2, 4, 5, 6):
+            h.crossover = 33  # CUDA cores
+        rows = min(M, 256)
+        first = None
+        for _ in range(3):
+            out = []
+            for R in (1, 8, 2):
+                y = torch.zeros((R, M), dtype=torch.float64, device="cuda")
+                h.step(x[:R], y)
+                v = torch.zeros((R, rows), dtype=torch.float64, device="cuda")
+                h.step_rows(0, rows, x[:R], v)
+                out += [y, v]
+            torch.cuda.synchronize()
+            if first is None:
+                first = out
+                for y, v in zip(out[::2], out[1::2]):  # two partitions of the same sums
+                    assert (y[:, :rows] - v).norm() <= 1e-6 * v.norm()
+            assert all(torch.equal(a, b) for a, b in zip(first, out))
