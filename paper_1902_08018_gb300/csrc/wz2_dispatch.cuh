@@ -7,9 +7,9 @@
 
 namespace whff {
 
-template <int RATE, bool LIFT, int R, int U, int GL = 32>
+template <int RATE, bool LIFT, int R, int U, int GL = 32, bool PRE = LIFT>
 static void wz2_launch_one(const Wz2Step& a, cudaStream_t st) {
-  dev::wz2_gemv_kernel<RATE, LIFT, R, U, GL><<<(unsigned)a.ctas, dev::kWarpsPerCta * 32, 0, st>>>(
+  dev::wz2_gemv_kernel<RATE, LIFT, R, U, GL, PRE><<<(unsigned)a.ctas, dev::kWarpsPerCta * 32, 0, st>>>(
       a.stream, a.M, a.N, a.BM, a.BN, a.x, a.ldx, a.x_vec_ok, a.L, a.maxseg, a.ws, a.y, a.ldy, a.state, a.decay,
       a.red32, a.seen);
 }
@@ -63,6 +63,14 @@ static int wz2_launch_lift(const Wz2Step& a, cudaStream_t st) {
 template <int RATE>
 int wz2_launch(const Wz2Step& a, cudaStream_t st) {
   if (!a.lift) return wz2_launch_lift<RATE, false>(a, st);
+  // One column of a small matrix: the kernel transforms x block by block, which
+  // costs less than a launch of its own (see kWz2FuseBlocks); the same operations,
+  // so the same bits.
+  if (a.R == 1 && !a.staged && (a.groups8 || a.unroll == 2) && a.BM * a.BN <= kWz2FuseBlocks) {
+    if (a.groups8) wz2_launch_one<RATE, true, 1, 2, 8, false>(a, st);
+    else wz2_launch_one<RATE, true, 1, 2, 32, false>(a, st);
+    return 0;
+  }
   // the lift: transform x once per pass, then the kernels read (2G)^T x as their x
   const int64_t ldt = 4 * a.BN, n = (int64_t)a.R * a.BN;
   dev::wz2_xt_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a.x, a.ldx, a.N, a.R, a.BN, a.xt, ldt);

@@ -13,6 +13,12 @@ namespace whff {
 // and records WHFF_ETIMEOUT: about a second of try_wait.
 constexpr uint32_t kWaitPolls = 1u << 22;
 
+// Blocks up to which a one-column pass of the lift transforms x in its kernel: a
+// launch of its own costs 2 to 4 us (4096^2 at rate 16 20.9 us with it, 17.7
+// without; 16384^2 97.5 and 94.2, at rate 8 83.6 and 83.1), seven more additions
+// per block about 2 % of a long pass (32768^2: 6383 GB/s with them, 6519 without).
+constexpr int64_t kWz2FuseBlocks = (int64_t)1 << 25;
+
 struct Wz2Step {
   const uint8_t* stream;
   int64_t M, N, BM, BN;

@@ -476,9 +476,10 @@ __device__ __forceinline__ void finish_shared_groups(int* __restrict__ seen, con
 // directly, when the band lies inside one range, or the piece's partial goes
 // to ws[band][segment], and the band's last warp adds its segments in order.  GL = 32: the warp takes one piece at a time; GL = 8: four lane
 // groups take the next four pieces at once (short bands, where a warp per
-// band would spend its time folding).  With the lift, x is the transformed
-// vector of wz2_xt_kernel (4 BN floats per right-hand side).
-template <int RATE, bool LIFT, int R, int UNROLL, int GL>
+// band would spend its time folding).  PRE: x is the transformed vector of
+// wz2_xt_kernel (4 BN floats per right-hand side); otherwise, with the lift, every
+// block transforms its own four values.
+template <int RATE, bool LIFT, int R, int UNROLL, int GL, bool PRE>
 __device__ __forceinline__ void wz2_gemv_body(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM,
                                               int64_t BN, const float* __restrict__ x, int64_t ldx, bool x_vec_ok,
                                               int64_t L, int maxseg, double* __restrict__ ws, double* __restrict__ y,
@@ -501,7 +502,7 @@ __device__ __forceinline__ void wz2_gemv_body(const uint8_t* __restrict__ stream
     if constexpr (GL == 32) {  // the warp takes the piece starting at b0
       const int64_t I = div64(b0, BN);
       const int64_t piece_end = min(b1, (I + 1) * BN);
-      wz2_piece<RATE, LIFT, R, UNROLL, 32, LIFT>(stream + (uint64_t)(I * BN) * kBlockBytes, b0 - I * BN,
+      wz2_piece<RATE, LIFT, R, UNROLL, 32, PRE>(stream + (uint64_t)(I * BN) * kBlockBytes, b0 - I * BN,
                                                  piece_end - I * BN, lane, x, ldx, N, x_fast, x_vec_ok, hi, lo);
       // a band inside one range is finished here, a shared one leaves a segment:
       // ws[(band * maxseg + seg) * R + r][i]
@@ -516,7 +517,7 @@ __device__ __forceinline__ void wz2_gemv_body(const uint8_t* __restrict__ stream
       const int64_t pb = max(b0, I * BN), pe = min(b1, (I + 1) * BN);
       const bool active = pb < pe;
       if (active)
-        wz2_piece<RATE, LIFT, R, UNROLL, GL, LIFT>(stream + (uint64_t)(I * BN) * kBlockBytes, pb - I * BN,
+        wz2_piece<RATE, LIFT, R, UNROLL, GL, PRE>(stream + (uint64_t)(I * BN) * kBlockBytes, pb - I * BN,
                                                    pe - I * BN, gl, x, ldx, N, x_fast, x_vec_ok, hi, lo);
       // one call for all groups (the folds shuffle across the whole warp)
       const int64_t g_lo = div64(I * BN, L), g_hi = div64((I + 1) * BN - 1, L);
@@ -539,13 +540,13 @@ __host__ __device__ constexpr int wz2_ctas_per_sm(int unroll) {
   return unroll == 8 ? (RATE <= 8 ? 3 : RATE <= 20 ? 2 : 1) : unroll == 4 ? (RATE <= 16 ? 3 : 2) : RATE <= 16 ? 4 : 3;
 }
 
-template <int RATE, bool LIFT, int R, int UNROLL, int GL>
+template <int RATE, bool LIFT, int R, int UNROLL, int GL, bool PRE = LIFT>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? wz2_ctas_per_sm<RATE>(UNROLL) : 1)
     wz2_gemv_kernel(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM, int64_t BN,
                     const float* __restrict__ x, int64_t ldx, bool x_vec_ok, int64_t L, int maxseg,
                     double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
                     double decay, bool red32, int* __restrict__ seen) {
-  wz2_gemv_body<RATE, LIFT, R, UNROLL, GL>(stream, M, N, BM, BN, x, ldx, x_vec_ok, L, maxseg, ws, y, ldy, state,
+  wz2_gemv_body<RATE, LIFT, R, UNROLL, GL, PRE>(stream, M, N, BM, BN, x, ldx, x_vec_ok, L, maxseg, ws, y, ldy, state,
                                            decay, red32, seen);
 }
 

@@ -72,3 +72,18 @@ def test_shared_bands_pass_after_pass(env, fmt, rate, M, N):
                 for y, v in zip(out[::2], out[1::2]):  # two partitions of the same sums
                     assert (y[:, :rows] - v).norm() <= 1e-6 * v.norm()
             assert all(torch.equal(a, b) for a, b in zip(first, out))
+
+
+@pytest.mark.parametrize("M,N", [(257, 516), (1000, 1027)])
+@pytest.mark.parametrize("rate", [8, 16])
+def test_x_of_any_alignment(env, M, N, rate):
+    """The one-column kernel that transforms x itself: x at an odd address, same bits."""
+    W, torch = env
+    A = np.random.default_rng(rate + N).standard_normal((M, N))
+    buf = torch.from_numpy(np.random.default_rng(N).standard_normal(N + 1).astype(np.float32)).cuda()
+    with W.whff_create(W.whff_compress(A, 5, rate), max_rhs=1) as h:
+        y = torch.zeros((2, M), dtype=torch.float64, device="cuda")
+        h.step(buf[1:], y[0])
+        h.step(buf[1:].clone(), y[1])
+        torch.cuda.synchronize()
+    assert torch.equal(y[0], y[1])
