@@ -4,6 +4,7 @@
 #include <cudaTypedefs.h>
 
 #include "scaled_mma.cuh"
+#include "scaled_mma_fp8.cuh"
 #include "scaled_mma_tma.cuh"
 #include "wz2_dispatch.h"
 
@@ -28,13 +29,30 @@ static int scaled_tma_attr() {
   return 0;
 }
 
+// The FP8 kernel's shared-memory attribute, set once per width.
+template <int NR>
+static int fp8_attr() {
+  static int done = 0;
+  if (!done) {
+    if (cudaFuncSetAttribute(dev::fp8_mma_kernel<NR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             dev::Fp8Smem<NR>::kBytes) != cudaSuccess) {
+      cudaGetLastError();
+      return -1;
+    }
+    done = 1;
+  }
+  return 0;
+}
+
 template <int FMT, int NR>
 static int scaled_mma_one(const ScaledMmaStep& a, cudaStream_t st) {
   using S = dev::ScaledMmaSmem<FMT, NR>;
   auto kern = dev::scaled_mma_kernel<FMT, NR>;
   constexpr bool kF16 = FMT == 3;
   const bool tma = (FMT == 2 || FMT == 3) && a.tmap != nullptr;
-  if (tma ? scaled_tma_attr<NR, kF16>() != 0
+  const bool fp8 = FMT == 4 && a.tmap != nullptr;
+  if (fp8 ? fp8_attr<NR>() != 0
+      : tma ? scaled_tma_attr<NR, kF16>() != 0
           : (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes) != cudaSuccess ||
              cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                   cudaSharedmemCarveoutMaxShared) != cudaSuccess)) {
@@ -52,7 +70,12 @@ static int scaled_mma_one(const ScaledMmaStep& a, cudaStream_t st) {
   } else {
     dev::wz2_mma_btiles<false, NR><<<(unsigned)((bthreads + 255) / 256), 256, 0, st>>>(pass, nullptr, 1, bthreads);
   }
-  if (tma) {
+  if (fp8) {
+    dev::fp8_mma_kernel<NR><<<(unsigned)((a.ctas + dev::kFp8Ranges - 1) / dev::kFp8Ranges), dev::kMmaDecodeThreads,
+                              dev::Fp8Smem<NR>::kBytes, st>>>(*static_cast<const CUtensorMap*>(a.tmap), a.row0, a.scales,
+                                                              a.TN, a.btiles, a.ws, nstages, a.R, a.maxseg,
+                                                              (int64_t)tiles * nstages, a.L, a.status, a.spin);
+  } else if (tma) {
     dev::scaled_mma_tma_kernel<NR, kF16><<<(unsigned)a.ctas, dev::kTmaThreads, dev::TmaSmem<NR>::kBytes, st>>>(
         *static_cast<const CUtensorMap*>(a.tmap), a.row0, a.scales, a.TN, a.btiles, a.ws, nstages, a.R, a.maxseg,
         (int64_t)tiles * nstages, a.L, a.status, a.spin);
@@ -190,15 +213,18 @@ int wz2_tma_map(void* out, const void* stream, int64_t BM, int64_t BN, int rate)
 int scaled_tma_map(void* out, const void* payload, int64_t M, int64_t ld, int fmt) {
   const auto encode = tma_encoder();
   if (!encode) return -1;
+  const bool fp8 = fmt == 4;
   const cuuint64_t dims[2] = {(cuuint64_t)ld, (cuuint64_t)M};
-  const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};  // bytes between rows (a multiple of 16: ld % 16 == 0)
-  const cuuint32_t box[2] = {64, 128};                  // 128 bytes x 128 rows: one stage
+  const cuuint64_t strides[1] = {(cuuint64_t)ld * (fp8 ? 1 : 2)};  // bytes between rows (ld % 16 == 0)
+  const cuuint32_t box[2] = {64, 128};                             // one stage: 64 columns x 128 rows
   const cuuint32_t estr[2] = {1, 1};
   const CUresult r = encode(static_cast<CUtensorMap*>(out),
-                            fmt == 3 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
-                            const_cast<void*>(payload), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                            fp8        ? CU_TENSOR_MAP_DATA_TYPE_UINT8
+                            : fmt == 3 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
+                                       : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
+                            2, const_cast<void*>(payload), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                            fp8 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? 0 : -1;
 }
 

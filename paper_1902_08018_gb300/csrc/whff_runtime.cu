@@ -581,10 +581,10 @@ int create_impl(const BlobInfo& info, const uint8_t* src, int max_rhs, unsigned 
     h->d_scales = reinterpret_cast<const float*>(h->d_stream + (uint64_t)info.M * (uint64_t)scaled_ld(info.N) *
                                                                    (uint64_t)elem_bytes(info.fmt));
   }
-  // BF16 and FP16 tensor-core passes take their A tiles by TMA from device
+  // BF16, FP16 and FP8 tensor-core passes take their A tiles by TMA from device
   // memory (if the map cannot be encoded the register-fed kernel runs instead:
-  // the same results for BF16, the same accuracy bar for FP16)
-  if ((info.fmt == WHFF_FMT_BF16 || info.fmt == WHFF_FMT_FP16) && h->d_ws_mma && !h->h_stream)
+  // the same results for BF16 and FP8, the same accuracy bar for FP16)
+  if (scaled16 && h->d_ws_mma && !h->h_stream)
     h->has_tmap = scaled_tma_map(h->tmap, h->d_stream, info.M, scaled_ld(info.N), info.fmt) == 0;
   // WZ2 tensor-core passes bring device-resident blocks in by TMA, host-resident
   // ones in 16-byte pieces: the same words, so the same results

@@ -54,3 +54,29 @@ def test_copies_agree(env, orc, fmt, rate, M, N, row0, nrows, R):
     for r in range(R):
         for got, want in ((out[0][0][r], ref[r]), (out[0][1][r], ref[r, row0:row0 + nrows])):
             assert np.linalg.norm(got - want) <= TOL * np.linalg.norm(want)
+
+
+# (M, N): one row and less than a 16-byte piece; an odd last stage; a last row past a tile; many
+# stages a tile; more tiles than item ranges
+@pytest.mark.parametrize("M,N", [(1, 5), (127, 65), (129, 700), (300, 9001), (40000, 100)])
+@pytest.mark.parametrize("R", [5, 20, 32])
+def test_fp8_copies_agree(env, orc, M, N, R):
+    """FP8 by tiled copies (device memory) and through registers (host memory): the same bits."""
+    W, torch = env
+    rng = np.random.default_rng(M + N)
+    A = rng.standard_normal((M, N)) * np.exp(rng.uniform(-3, 3, size=(M, 1)))
+    blob = W.whff_compress(A, 4, 0)
+    X = rng.standard_normal((R, N)).astype(np.float32)
+    out = []
+    for host in (False, True):
+        with W.whff_create(blob, max_rhs=32, host_resident=host) as h:
+            x = torch.from_numpy(X).cuda()
+            y = torch.zeros((R, M), dtype=torch.float64, device="cuda")
+            h.step(x, y)
+            torch.cuda.synchronize()
+            assert h.sync_status() == 0
+            out.append(y.cpu().numpy())
+    assert (out[0] == out[1]).all()
+    ref = X.astype(np.float64) @ orc.decode(blob.tobytes()).T
+    for r in range(R):
+        assert np.linalg.norm(out[0][r] - ref[r]) <= TOL * np.linalg.norm(ref[r])
