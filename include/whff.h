@@ -184,8 +184,9 @@ int whff_info(const whff_handle* h, int* fmt, int* rate, int64_t* M, int64_t* N,
 /* Launch plan of a resident matrix: *ksplit = column splits per 4-row band
  * (1 for matrices with enough rows to fill the GPU), *launches = kernel
  * launches of one CUDA-core whff_step pass: the fused kernel, the epilogue of
- * split-K (or of shared bands, bulk-staged) if any, and for FIXED_LIFT and FIXED_ACC the
- * (2G)^T x transform of x that the fused kernel reads. */
+ * split-K (or of shared bands, bulk-staged) if any, and the (2G)^T x transform of x
+ * where the fused kernel reads it: FIXED_ACC, and FIXED_LIFT unless the kernel
+ * transforms x itself (two blocks in flight, up to 2^24 blocks at rate 8, else 2^25). */
 int whff_plan(const whff_handle* h, int* ksplit, int* launches);
 
 /* One control step (Sec. 2.1 / Sec. 4.4): y[:,r] = Ahat * x[:,r] for r < R,

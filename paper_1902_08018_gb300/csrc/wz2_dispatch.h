@@ -13,11 +13,14 @@ namespace whff {
 // and records WHFF_ETIMEOUT: about a second of try_wait.
 constexpr uint32_t kWaitPolls = 1u << 22;
 
-// Blocks up to which a one-column pass of the lift transforms x in its kernel: a
-// launch of its own costs 2 to 4 us (4096^2 at rate 16 20.9 us with it, 17.7
-// without; 16384^2 97.5 and 94.2, at rate 8 83.6 and 83.1), seven more additions
-// per block about 2 % of a long pass (32768^2: 6383 GB/s with them, 6519 without).
-constexpr int64_t kWz2FuseBlocks = (int64_t)1 << 25;
+// Blocks up to which a one-column pass of the lift transforms x in its kernel: that
+// saves a launch and costs seven additions per block.  Transform launched / fused, us:
+//   4096^2 (2^20 blocks), rate 16: 20.9 / 17.7
+//   16384^2 (2^24), rates 8 12 16 20 24: 83.3 86.8 97.4 114.7 129.1 / 82.6 84.3 94.0 111.5 124.9
+//   20480^2: 121.0 127.0 144.2 170.2 194.2 / 122.0 123.5 139.9 168.2 189.4
+//   32768^2 (2^26): 277.1 290.4 334.5 410.5 467.6 / 286.7 292.7 332.1 410.0 463.2
+// Rate 8, bound by decode instructions, loses from 20480^2 on; rate 12 at 32768^2.
+constexpr int64_t wz2_fuse_blocks(int rate) { return (int64_t)1 << (rate == 8 ? 24 : 25); }
 
 struct Wz2Step {
   const uint8_t* stream;
