@@ -321,13 +321,13 @@ __global__ void __launch_bounds__(kWz1Threads)
   using Smem = Wz1Smem<NW32, kWz1Threads>;
   __shared__ __align__(16) Smem sm;
   static_assert(sizeof(Smem) >= (kWz1Threads / 32) * 512 * 8, "turns the rows round: 4 x 128 doubles a warp");
-  wz1_smem_init(sm);
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool live = b < nblocks;
   int64_t I = 0, J = 0;
   unit_of(live ? b : nblocks - 1, BN, I, J);
   uint32_t w[NW32];
   load_block<NW32>(stream, live ? b : nblocks - 1, w);
+  wz1_smem_init(sm);  // while the words are on their way
   int32_t q[16];
   int emax;
   const bool nz = decode_block(w, sm, q, emax);

@@ -88,7 +88,7 @@ constexpr TestTable make_test_table() {
   }
   return t;
 }
-static __device__ const TestTable kTestTable = make_test_table();
+alignas(16) static __device__ const TestTable kTestTable = make_test_table();
 
 // Shared memory of a block of TH threads decoding NW32-word blocks: per thread a
 // column of stream words (two zero words follow) and one of 16 plane pairs
@@ -97,13 +97,17 @@ template <int NW32, int TH>
 struct Wz1Smem {
   uint32_t words[(NW32 + 2) * TH];
   uint32_t planes[16 * TH];
-  uint32_t table[kTestEntries];
+  alignas(16) uint32_t table[kTestEntries];
 };
 
-// Once per block, before the first decode; ends with a barrier.
+// Once per block, before the first decode; ends with a barrier.  16 bytes at a
+// time, and a caller with one block a thread asks for its words first: a small
+// matrix is bound by these latencies.
 template <int NW32, int TH>
 __device__ __forceinline__ void wz1_smem_init(Wz1Smem<NW32, TH>& sm) {
-  for (int i = threadIdx.x; i < kTestEntries; i += TH) sm.table[i] = kTestTable.e[i];
+  static_assert(kTestEntries % 4 == 0, "whole 16-byte pieces");
+  for (int i = threadIdx.x; i < kTestEntries / 4; i += TH)
+    reinterpret_cast<uint4*>(sm.table)[i] = reinterpret_cast<const uint4*>(kTestTable.e)[i];
   sm.words[NW32 * TH + threadIdx.x] = sm.words[(NW32 + 1) * TH + threadIdx.x] = 0u;
   __syncthreads();
 }
