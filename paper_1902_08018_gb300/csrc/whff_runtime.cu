@@ -1268,7 +1268,7 @@ extern "C" int whff_tune(whff_handle* h, int iters, void* stream, double* best_m
   const int orig_u = h->unroll, orig_c = h->ctas_per_sm;
   const int orig_f = (h->red32 ? WHFF_FOLD_FP32_PAIRS : 0) | (h->groups8 ? WHFF_FOLD_LANE_GROUPS : 0) |
                      (h->bulk ? WHFF_CONFIG_BULK : 0);
-  double best = 1e30;
+  double best = 1e30, fastest = 1e30;  // of the shape taken, of all
   int bu = orig_u, bc = 1 << 20, bf = orig_f;
   int err = WHFF_OK;
   const bool lift = h->info.fmt == WHFF_FMT_FIXED_LIFT;
@@ -1292,9 +1292,14 @@ extern "C" int whff_tune(whff_handle* h, int iters, void* stream, double* best_m
     if (err) break;
     float ms = 0.f;
     cudaEventElapsedTime(&ms, e0, e1);
-    // within the timing's noise of each other (1.5 %), the shape with fewer CTAs
-    if (c < bc ? ms / iters < 1.015 * best : c > bc ? 1.015 * ms / iters < best : ms / iters < best) {
-      best = ms / iters;
+    // Within the events' noise of the fastest so far, the shape with fewer CTAs: 0.5 us,
+    // and 1.5 % on short passes.  A share alone gave long passes away: 32768^2 at rate
+    // 16 took a shape of 339 us where another has 335.
+    const double t = ms / iters, tie = std::min(0.015 * fastest, 0.0005);
+    const bool take = c < bc ? t < fastest + tie : c > bc ? t < fastest - tie : t < best;
+    fastest = std::min(fastest, t);
+    if (take) {
+      best = t;
       bu = u;
       bc = c;
       bf = f;
