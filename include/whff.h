@@ -186,7 +186,7 @@ int whff_info(const whff_handle* h, int* fmt, int* rate, int64_t* M, int64_t* N,
  * launches of one CUDA-core whff_step pass: the fused kernel, the epilogue of
  * split-K (or of shared bands, bulk-staged) if any, and the (2G)^T x transform of x
  * where the fused kernel reads it: FIXED_ACC, and FIXED_LIFT unless the kernel
- * transforms x itself (two blocks in flight, up to 2^24 blocks at rate 8, else 2^25). */
+ * transforms x itself (two blocks in flight, up to 2^24 blocks at rate 8, 2^25 at 12, else 2^26). */
 int whff_plan(const whff_handle* h, int* ksplit, int* launches);
 
 /* One control step (Sec. 2.1 / Sec. 4.4): y[:,r] = Ahat * x[:,r] for r < R,

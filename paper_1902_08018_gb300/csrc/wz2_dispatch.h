@@ -19,8 +19,9 @@ constexpr uint32_t kWaitPolls = 1u << 22;
 //   16384^2 (2^24), rates 8 12 16 20 24: 83.3 86.8 97.4 114.7 129.1 / 82.6 84.3 94.0 111.5 124.9
 //   20480^2: 121.0 127.0 144.2 170.2 194.2 / 122.0 123.5 139.9 168.2 189.4
 //   32768^2 (2^26): 277.1 290.4 334.5 410.5 467.6 / 286.7 292.7 332.1 410.0 463.2
-// Rate 8, bound by decode instructions, loses from 20480^2 on; rate 12 at 32768^2.
-constexpr int64_t wz2_fuse_blocks(int rate) { return (int64_t)1 << (rate == 8 ? 24 : 25); }
+// Rate 8, bound by decode instructions, loses from 20480^2 on; rate 12 at 32768^2;
+// the others gain up to there, the longest measured.
+constexpr int64_t wz2_fuse_blocks(int rate) { return (int64_t)1 << (rate == 8 ? 24 : rate == 12 ? 25 : 26); }
 
 struct Wz2Step {
   const uint8_t* stream;
