@@ -348,8 +348,8 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
   constexpr uint32_t kACols = 8 * kMmaKSteps * PA;  // TMEM columns of a stage's A pieces
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t s_base = smem_addr(smem);
-  const uint32_t b_full = s_base + SM::kBars;  // NB: the B tile in the slot has landed
-  const uint32_t w_full = b_full + 8 * NB;     // NB: so have its compressed words (every copying thread's)
+  const uint32_t b_full = s_base + SM::kBars;  // NB: the B tile in the slot has landed, and the words of a tiled copy
+  const uint32_t w_full = b_full + 8 * NB;     // NB: so have the words copied in pieces (every copying thread's)
   const uint32_t done = w_full + 8 * NB;       // NB: the MMAs of the stage in the slot are done
   const uint32_t a_full = done + 8 * NB;       // NA: the stage's A pieces are in the buffer (4 arrivals)
   const uint32_t gfull = a_full + 8 * NA;      // 2: the accumulator group is complete
@@ -437,12 +437,13 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
     for (int i = 0; i < q && i < n; ++i) advance();
     for (int k = q; k < n; k += NQ) {
       const MmaMember& me = mb(c_m);
+      const bool tiled = me.map != nullptr;
       // the lane's first block in the slot (see the copies)
       const uint8_t* staged = smem + NB * SM::kB + (uint32_t)k % NB * SM::kWords + cb * SM::kBB;
       if (me.paired) {
         const int odd = ((int)me.band0 + band_l) & 1;
         staged += (odd * (kMmaBands / 2) + (band_l >> 1)) * (SM::kRowBytes + 16) + 8 * odd;
-      } else if (me.map) {
+      } else if (tiled) {
         staged += band_l * SM::kRowBytes;
       } else {
         const uint32_t blk = (32 * (uint32_t)c_tile + band_l) * (uint32_t)me.BN + 16 * (uint32_t)c_st;
@@ -453,7 +454,8 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
 #pragma unroll
         for (int i = 0; i < NQ; ++i) advance();
       }
-      if (!warp_wait(w_full + 8 * ((uint32_t)k % NB), (uint32_t)k / NB & 1u)) break;  // the words are here
+      // the words are here
+      if (!warp_wait((tiled ? b_full : w_full) + 8 * ((uint32_t)k % NB), (uint32_t)k / NB & 1u)) break;
       if (k >= NA) {  // the A buffer is free once the MMAs of the stage NA before are done
         const uint32_t p = (uint32_t)(k - NA);
         if (!warp_wait(done + 8 * (p % NB), p / NB & 1u)) break;
@@ -553,7 +555,7 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
       // ---- issue.  The whole warp walks the stages, so that everything the MMAs take is
       // warp-uniform; lanes 0-2 wait for a stage's three barriers side by side (a wait costs
       // about 250 clocks even when its phase is over), one elected lane issues.
-      int last_commit = -1, gpos = 0, acc = 0, buf = 0, slot = 0, left = len;
+      int last_commit = -1, groups = 0, gpos = 0, acc = 0, buf = 0, slot = 0, left = len;
       uint32_t phase = 0, a_phase = 0, g_phase = 1;  // g_phase: the groups are free at first
       const uint64_t b_desc0 = smem_desc(s_base, 128, 256);
 #pragma unroll 1
@@ -600,6 +602,7 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
         if (ends) {
           g_phase ^= (uint32_t)acc;
           acc ^= 1;
+          ++groups;
         }
         gpos = ends ? 0 : gpos + 1;
         advance();
@@ -609,8 +612,10 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
       }
       __syncwarp();
       leave();
-      if (lane == 0 && *abort_flag && last_commit >= 0)  // MMAs in flight: a second bounded chance
-        (void)mbar_wait(done + 8 * (last_commit % NB), (uint32_t)((last_commit / NB) & 1));
+      if (lane == 0 && *abort_flag) {  // MMAs and their commits in flight: a second bounded chance
+        if (last_commit >= 0) (void)mbar_wait(done + 8 * (last_commit % NB), (uint32_t)((last_commit / NB) & 1));
+        if (groups) (void)mbar_wait(gfull + 8 * ((groups - 1) & 1), (uint32_t)(((groups - 1) >> 1) & 1));
+      }
       __syncwarp();
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512u));
@@ -620,6 +625,8 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
       // number of blocks per band (rows 8 bytes off 16) two, of the even and the odd bands, the
       // odd rows starting 8 bytes into theirs; from host memory aligned 16-byte pieces (a row
       // may start 8 bytes into the first one).  A slot is refilled once its MMAs are done.
+      // What the copy engine brings completes on b_full alone, which one arrival closes: this
+      // warp can then wait for all of it at the end, whoever has given up before.
       constexpr bool kShift = SM::kBB % 16 != 0;
       constexpr int kRow = (kMmaStageBlocks * SM::kBB + (kShift ? 8 : 0) + 15) / 16;  // pieces of a band
       // a warp takes one row (two of 16 pieces) at a time, every third
@@ -630,26 +637,26 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
       for (; issued < n; ++issued) {
         if (!warp_wait(done + 8 * slot, phase)) break;
         const MmaMember& me = mb(c_m);
-        const uint32_t words = s_base + NB * SM::kB + slot * SM::kWords, w_bar = w_full + 8 * slot;
+        const uint32_t words = s_base + NB * SM::kB + slot * SM::kWords;
+        const uint32_t b_bar = b_full + 8 * slot, w_bar = w_full + 8 * slot;
         const bool tiled = me.map != nullptr;
         if (warp == kMmaCopyWarp && elect_one()) {
-          bulk_copy_g2s(s_base + slot * SM::kB, me.btiles + (int64_t)c_st * SM::kB, (uint32_t)SM::kB, b_full + 8 * slot);
+          constexpr uint32_t kHalf = kMmaBands / 2 * (SM::kRowBytes + 16);  // paired: odd and even bands, a map each
+          if (tiled) mbar_expect_tx_only(b_bar, me.paired ? 2 * kHalf : (uint32_t)(kMmaBands * SM::kRowBytes));
+          bulk_copy_g2s(s_base + slot * SM::kB, me.btiles + (int64_t)c_st * SM::kB, (uint32_t)SM::kB, b_bar);
           if (tiled) {
             const int x = c_st * kMmaStageBlocks * NW, g = (int)(me.band0 + kMmaBands * (int64_t)c_tile);
-            if (me.paired) {  // odd and even bands, a map each
-              constexpr uint32_t kHalf = kMmaBands / 2 * (SM::kRowBytes + 16);
-              mbar_expect_tx_only(w_bar, 2 * kHalf);
-              tma_load_2d(words + (g & 1) * kHalf, static_cast<const uint8_t*>(me.map) + (g & 1) * 128, x, g >> 1, w_bar);
+            if (me.paired) {
+              tma_load_2d(words + (g & 1) * kHalf, static_cast<const uint8_t*>(me.map) + (g & 1) * 128, x, g >> 1, b_bar);
               tma_load_2d(words + (~g & 1) * kHalf, static_cast<const uint8_t*>(me.map) + (~g & 1) * 128, x, (g + 1) >> 1,
-                          w_bar);
+                          b_bar);
             } else {
-              mbar_expect_tx_only(w_bar, (uint32_t)(kMmaBands * SM::kRowBytes));
-              tma_load_2d(words, me.map, x, g, w_bar);
+              tma_load_2d(words, me.map, x, g, b_bar);
             }
           }
         }
         __syncwarp();
-        if (tiled) {  // the copy engine brings the words
+        if (tiled) {  // nothing to copy in pieces: the phase turns all the same
           mbar_arrive(w_bar);
           advance();
           if (++slot == NB) slot = 0, phase ^= 1;
@@ -682,7 +689,7 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
       __syncwarp();
       asm volatile("cp.async.wait_all;\n" ::: "memory");
       leave();
-      if (warp == kMmaCopyWarp && lane == 0 && *abort_flag)  // the B tiles in flight land before the CTA goes
+      if (warp == kMmaCopyWarp && lane == 0 && *abort_flag)  // the engine's copies in flight land before the CTA goes
         for (int k = issued > NB ? issued - NB : 0; k < issued; ++k)
           (void)mbar_wait(b_full + 8 * (k % NB), (uint32_t)((k / NB) & 1));
     }

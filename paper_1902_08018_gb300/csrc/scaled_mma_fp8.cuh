@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
       // ---- issue.  The whole warp walks the stages, so that everything the MMAs take is
       // warp-uniform; lanes 0-2 wait for a stage's three barriers side by side (a wait costs
       // about 250 clocks even when its phase is over), one elected lane issues.
-      int last_commit = -1, gpos = 0, acc = 0, buf = 0, slot = 0, left = len;
+      int last_commit = -1, groups = 0, gpos = 0, acc = 0, buf = 0, slot = 0, left = len;
       uint32_t phase = 0, a_phase = 0, g_phase = 1;  // g_phase: the groups are free at first
       const uint64_t b_desc0 = smem_desc(s_base, 128, 256);
 #pragma unroll 1
@@ -249,6 +249,7 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
         if (ends) {
           g_phase ^= (uint32_t)acc;
           acc ^= 1;
+          ++groups;
         }
         gpos = ends ? 0 : gpos + 1;
         advance();
@@ -258,8 +259,10 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
       }
       __syncwarp();
       leave();
-      if (lane == 0 && *abort_flag && last_commit >= 0)  // MMAs in flight: a second bounded chance
-        (void)mbar_wait(done + 8 * (last_commit % NB), (uint32_t)((last_commit / NB) & 1));
+      if (lane == 0 && *abort_flag) {  // MMAs and their commits in flight: a second bounded chance
+        if (last_commit >= 0) (void)mbar_wait(done + 8 * (last_commit % NB), (uint32_t)((last_commit / NB) & 1));
+        if (groups) (void)mbar_wait(gfull + 8 * ((groups - 1) & 1), (uint32_t)(((groups - 1) >> 1) & 1));
+      }
       __syncwarp();
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512u));
