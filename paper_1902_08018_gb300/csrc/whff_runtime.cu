@@ -565,8 +565,16 @@ int create_impl(const BlobInfo& info, const uint8_t* src, int max_rhs, unsigned 
     set_error("whff_create: cudaMalloc of the workspace failed");
     return fail(WHFF_ENOMEM);
   }
+  // WZ2 tensor-core passes bring device-resident blocks in by TMA, host-resident
+  // ones in 16-byte pieces: the same words, so the same results
+  alignas(64) unsigned char map[256];
+  static_assert(sizeof(map) <= kColexpBytes, "after the B tiles, where FP16 passes keep their exponents");
+  if (wz2 && h->d_ws_mma && !h->h_stream) h->map_count = wz2_tma_map(map, h->d_stream, h->BM, h->BN, info.rate);
+  if (h->map_count) h->d_map = h->d_btiles + h->btile_bytes;
+  // everything on st, and complete before any other stream can use the handle
   if (cudaMemsetAsync(h->d_status, 0, sizeof(int), st) != cudaSuccess ||
       cudaMemsetAsync(h->d_seen, 0, (size_t)h->BM * sizeof(int), st) != cudaSuccess ||
+      (h->d_map && cudaMemcpyAsync(h->d_map, map, sizeof(map), cudaMemcpyHostToDevice, st) != cudaSuccess) ||
       (!h->h_stream && src &&
        cudaMemcpyAsync(h->d_stream, src, info.stream_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess) ||
       cudaStreamSynchronize(st) != cudaSuccess) {
@@ -586,17 +594,6 @@ int create_impl(const BlobInfo& info, const uint8_t* src, int max_rhs, unsigned 
   // the same results for BF16 and FP8, the same accuracy bar for FP16)
   if (scaled16 && h->d_ws_mma && !h->h_stream)
     h->has_tmap = scaled_tma_map(h->tmap, h->d_stream, info.M, scaled_ld(info.N), info.fmt) == 0;
-  // WZ2 tensor-core passes bring device-resident blocks in by TMA, host-resident
-  // ones in 16-byte pieces: the same words, so the same results
-  alignas(64) unsigned char map[256];
-  static_assert(sizeof(map) <= kColexpBytes, "after the B tiles, where FP16 passes keep their exponents");
-  if (wz2 && h->d_ws_mma && !h->h_stream && (h->map_count = wz2_tma_map(map, h->d_stream, h->BM, h->BN, info.rate))) {
-    h->d_map = h->d_btiles + h->btile_bytes;
-    if (cudaMemcpy(h->d_map, map, sizeof(map), cudaMemcpyHostToDevice) != cudaSuccess) {
-      set_error(std::string("whff_create: tensor map upload failed: ") + cudaGetErrorString(cudaGetLastError()));
-      return fail(WHFF_ECUDA);
-    }
-  }
   *out = h;
   return WHFF_OK;
 }
