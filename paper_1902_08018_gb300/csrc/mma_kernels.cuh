@@ -634,9 +634,15 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
       const int r0 = (warp - kMmaCopyWarp) * (32 / kLanes) + lane / kLanes, c0 = lane % kLanes;
       int issued = 0, slot = 0;
       uint32_t phase = 1;  // the slots are free at first
+      const void* acquired = nullptr;  // the map that this CTA may use
       for (; issued < n; ++issued) {
         if (!warp_wait(done + 8 * slot, phase)) break;
         const MmaMember& me = mb(c_m);
+        if (me.map && me.map != acquired && warp == kMmaCopyWarp) {
+          acquired = me.map;
+          tensormap_acquire(me.map);
+          if (me.paired) tensormap_acquire(static_cast<const uint8_t*>(me.map) + 128);
+        }
         const uint32_t words = s_base + NB * SM::kB + slot * SM::kWords;
         const uint32_t b_bar = b_full + 8 * slot, w_bar = w_full + 8 * slot;
         const bool tiled = me.map != nullptr;
