@@ -10,36 +10,15 @@
 
 namespace whff {
 
-// The TMA-fed kernel (BF16, or FP16 with F16): its shared-memory attribute,
-// set once per width and type.
-template <int NR, bool F16>
-static int scaled_tma_attr() {
-  static int done = 0;
-  if (!done) {
-    auto kern = dev::scaled_mma_tma_kernel<NR, F16>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dev::TmaSmem<NR>::kBytes) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
-            cudaSuccess) {
-      cudaGetLastError();
-      return -1;
-    }
-    done = 1;
-  }
-  return 0;
-}
-
-// The FP8 kernel's shared-memory attribute, set once per width.
-template <int NR>
-static int fp8_attr() {
-  static int done = 0;
-  if (!done) {
-    if (cudaFuncSetAttribute(dev::fp8_mma_kernel<NR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             dev::Fp8Smem<NR>::kBytes) != cudaSuccess) {
-      cudaGetLastError();
-      return -1;
-    }
-    done = 1;
+// Raise a kernel's dynamic shared-memory limit.  The limit belongs to the kernel on
+// one device (and context): every launch sets it, as one process may use several.
+template <class K>
+static int scaled_set_smem(K kern, int bytes) {
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
+      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
+          cudaSuccess) {
+    cudaGetLastError();
+    return -1;
   }
   return 0;
 }
@@ -51,14 +30,10 @@ static int scaled_mma_one(const ScaledMmaStep& a, cudaStream_t st) {
   constexpr bool kF16 = FMT == 3;
   const bool tma = (FMT == 2 || FMT == 3) && a.tmap != nullptr;
   const bool fp8 = FMT == 4 && a.tmap != nullptr;
-  if (fp8 ? fp8_attr<NR>() != 0
-      : tma ? scaled_tma_attr<NR, kF16>() != 0
-          : (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes) != cudaSuccess ||
-             cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  cudaSharedmemCarveoutMaxShared) != cudaSuccess)) {
-    cudaGetLastError();
+  if (fp8   ? scaled_set_smem(dev::fp8_mma_kernel<NR>, dev::Fp8Smem<NR>::kBytes)
+      : tma ? scaled_set_smem(dev::scaled_mma_tma_kernel<NR, kF16>, dev::TmaSmem<NR>::kBytes)
+            : scaled_set_smem(kern, S::kBytes))
     return -1;
-  }
   const int nstages = (int)((a.N + 63) / 64);
   const int tiles = (int)((a.M + 127) / 128);
   const dev::MmaPass pass{a.x, a.y, a.btiles, a.ws, a.ldx, a.ldy, a.N, a.M, 0, 0, 0, nstages, tiles, a.R, a.maxseg};
@@ -115,9 +90,7 @@ static int scaled_mma_occ_one() {
   auto kern = dev::scaled_mma_kernel<FMT, NR>;
   cudaFuncAttributes fa;
   int dev = 0, smem_sm = 0, regs_sm = 0, reserved = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes) != cudaSuccess ||
-      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
-          cudaSuccess ||
+  if (scaled_set_smem(kern, S::kBytes) ||
       cudaFuncGetAttributes(&fa, kern) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess ||
@@ -140,7 +113,7 @@ static int scaled_tma_occ_one() {
   auto kern = dev::scaled_mma_tma_kernel<NR, F16>;
   cudaFuncAttributes fa;
   int dev = 0, smem_sm = 0, regs_sm = 0, reserved = 0;
-  if (scaled_tma_attr<NR, F16>() || cudaFuncGetAttributes(&fa, kern) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
+  if (scaled_set_smem(kern, dev::TmaSmem<NR>::kBytes) || cudaFuncGetAttributes(&fa, kern) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess) {
