@@ -204,8 +204,11 @@ int whff_plan(const whff_handle* h, int* ksplit, int* launches);
  * per-lane sums in FP32 (compensated), cross-warp and cross-CTA sums and y in
  * FP64.  If state != NULL, afterwards for r = 0..R-1 in order:
  * state <- decay*state + y[:,r] (FP64).  x, y, state: device pointers.
- * Deterministic for a fixed (handle, R).  Errors: WHFF_EINVAL (R > max_rhs,
- * bad ld), WHFF_ECUDA. */
+ * Deterministic for a fixed (handle, R).  A handle takes one pass at a time:
+ * its passes, whether steps, row views or graph replays, share a workspace, so
+ * on several streams they must be ordered.  The results of passes that overlap
+ * are not defined; later passes are not affected.  Errors: WHFF_EINVAL
+ * (R > max_rhs, bad ld), WHFF_ECUDA. */
 int whff_step(whff_handle* h, const float* x, int R, int64_t ldx, double* y, int64_t ldy, double* state,
               double decay, void* stream);
 

@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, R > 1 ? 1 : FMT == 7 && GL 
     scaled_range_kernel(const uint8_t* __restrict__ payload, const float* __restrict__ scales, int64_t M, int64_t N,
                         int64_t ld, int64_t TN, const float* __restrict__ x, int64_t ldx, bool x_vec_ok, int64_t L,
                         int maxseg, double* __restrict__ ws, double* __restrict__ y, int64_t ldy,
-                        double* __restrict__ state, double decay, bool red32, int* __restrict__ seen) {
+                        double* __restrict__ state, double decay, bool red32, BandCount seen) {
   constexpr int V = ScaledTraits<FMT>::V;
   constexpr int NG = 32 / GL;  // pieces taken at once
   const int lane = threadIdx.x & 31;

@@ -436,17 +436,18 @@ __device__ __forceinline__ void sum_segments(const double* __restrict__ ws, int6
 
 // After a warp has written its segment of shared band I: the warp that brings the
 // band's last of nseg segments adds them up (the order of the sum is the segments',
-// whoever does it), and leaves the band's counter at zero for the next pass.  A
-// kernel of its own for these few sums cost 4 us of launch and latency per pass.
-__device__ __forceinline__ void finish_shared_band(int* __restrict__ seen, const double* __restrict__ ws, int64_t I,
+// whoever does it).  The count starts from the pass's own tag, which is above all that
+// an earlier pass left, so nothing that happened before can reach it.  A kernel of its
+// own for these few sums cost 4 us of launch and latency per pass.
+__device__ __forceinline__ void finish_shared_band(BandCount seen, const double* __restrict__ ws, int64_t I,
                                                    int64_t M, int nseg, int maxseg, int R, double* __restrict__ y,
                                                    int64_t ldy, double* __restrict__ state, double decay) {
   __threadfence();
   __syncwarp();
   int last = 0;
   if ((threadIdx.x & 31) == 0) {
-    last = atomicAdd(seen + I, 1) == nseg - 1;
-    if (last) seen[I] = 0;
+    (void)atomicMax(seen.count + I, seen.tag);
+    last = atomicAdd(seen.count + I, 1ull) == seen.tag + (unsigned)(nseg - 1);
   }
   last = __shfl_sync(0xffffffffu, last, 0);
   if (!last) return;
@@ -456,7 +457,7 @@ __device__ __forceinline__ void finish_shared_band(int* __restrict__ seen, const
 
 // The same for the four lane groups of a warp, each with a piece of a band of its own.
 template <int GL>
-__device__ __forceinline__ void finish_shared_groups(int* __restrict__ seen, const double* __restrict__ ws, int64_t I,
+__device__ __forceinline__ void finish_shared_groups(BandCount seen, const double* __restrict__ ws, int64_t I,
                                                      int64_t M, int nseg, bool shared, int maxseg, int R,
                                                      double* __restrict__ y, int64_t ldy, double* __restrict__ state,
                                                      double decay) {
@@ -483,7 +484,7 @@ template <int RATE, bool LIFT, int R, int UNROLL, int GL, bool PRE>
 __device__ __forceinline__ void wz2_gemv_body(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM,
                                               int64_t BN, const float* __restrict__ x, int64_t ldx, bool x_vec_ok,
                                               int64_t L, int maxseg, double* __restrict__ ws, double* __restrict__ y,
-                                              int64_t ldy, double* __restrict__ state, double decay, bool red32, int* __restrict__ seen) {
+                                              int64_t ldy, double* __restrict__ state, double decay, bool red32, BandCount seen) {
   constexpr int64_t kBlockBytes = 4 * Wz2Layout<RATE>::kWords;
   constexpr int NG = 32 / GL;  // pieces taken at once
   const int lane = threadIdx.x & 31;
@@ -545,7 +546,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? wz2_ctas_per_sm<RA
     wz2_gemv_kernel(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM, int64_t BN,
                     const float* __restrict__ x, int64_t ldx, bool x_vec_ok, int64_t L, int maxseg,
                     double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
-                    double decay, bool red32, int* __restrict__ seen) {
+                    double decay, bool red32, BandCount seen) {
   wz2_gemv_body<RATE, LIFT, R, UNROLL, GL, PRE>(stream, M, N, BM, BN, x, ldx, x_vec_ok, L, maxseg, ws, y, ldy, state,
                                            decay, red32, seen);
 }

@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
     wz3_gemv_kernel(const uint64_t* __restrict__ index, const uint8_t* __restrict__ area, int64_t M, int64_t BM,
                     int BN, int RB, const float* __restrict__ xt, int64_t ldt, int64_t L, int maxseg,
                     double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
-                    double decay, int* __restrict__ seen) {
+                    double decay, BandCount seen) {
   const int lane = threadIdx.x & 31;
   const int64_t g = (int64_t)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
   const int64_t total = BM * RB;
@@ -274,7 +274,7 @@ __device__ __forceinline__ int64_t wz3_groups(int64_t BM) { return (BM + 7) / 8;
 static __global__ void __launch_bounds__(kWarpsPerCta * 32, 2)
     wz3_gemv8_kernel(const uint64_t* __restrict__ index, const uint8_t* __restrict__ area, int64_t M, int64_t BM,
                      int BN, int RB, const float* __restrict__ xt, int64_t L, int maxseg, double* __restrict__ ws,
-                     double* __restrict__ y, int64_t ldy, double* __restrict__ state, double decay, int* __restrict__ seen) {
+                     double* __restrict__ y, int64_t ldy, double* __restrict__ state, double decay, BandCount seen) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t u0 = (int64_t)blockIdx.x * L, u1 = min(wz3_groups(BM) * RB, u0 + L);
   for (int64_t ub = u0; ub < u1;) {  // the range's piece of group G: runs [q0, q1) of each of its bands
