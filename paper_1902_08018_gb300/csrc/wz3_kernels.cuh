@@ -215,11 +215,12 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
 // The chain of a row takes scalar FMAs (their operands need no doubling into
 // pairs; a packed instruction takes two issue cycles of the FMA pipe anyway), the
 // TwoSum packed ones on rows 2h and 2h + 1.
-// The 32 sums of a band (r, i) are folded over the lanes as pairs
+// The 32 sums of a band (r, i) are folded over the lanes as triples
 // (fold.cuh), lane 4 r + i ending with that of row i and column r: FP64 butterflies cost
-// 2600 cycles of GB300's FP64 pipe per band piece.
+// 2600 cycles of GB300's FP64 pipe per band piece.  Pairs would take 3 us less of a
+// pass, and give up digits that FP64 kept.
 // 8192^2 at 1e-7 (0.18 GB, one pass of 8 columns): 269 us and 12 us of segment
-// epilogue with warp ranges and FP64 folds, 105 us and 4 us this way, at 56 % of
+// epilogue with warp ranges and FP64 folds, 117 us with all launches this way, at 56 % of
 // the issue slots; the FMA pipe (128 FMAs and 96 packed ones per 32 blocks, and
 // the moves between them) is what bounds it now, at 57 us of pipe time.
 
@@ -316,7 +317,7 @@ static __global__ void __launch_bounds__(kWarpsPerCta * 32, 2)
         l[4 * r + 2 * k] = b.x, l[4 * r + 2 * k + 1] = b.y;
       }
     double z[1];
-    fold_lanes<32, 32, false, true>(h, l, lane, z);
+    fold_lanes<32, 32, true>(h, l, lane, z);
     const int64_t c_lo = div64(G * RB, L), c_hi = div64((G + 1) * RB - 1, L);
     const bool shared = c_lo != c_hi;
     band_write<1, 8, 32>(z, lane, 4 * I, M, shared ? ws + (I * maxseg + (blockIdx.x - c_lo)) * 32 : nullptr, y, ldy,
