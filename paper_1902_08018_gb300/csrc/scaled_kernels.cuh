@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, R > 1 ? 1 : FMT == 7 && GL 
     scaled_range_kernel(const uint8_t* __restrict__ payload, const float* __restrict__ scales, int64_t M, int64_t N,
                         int64_t ld, int64_t TN, const float* __restrict__ x, int64_t ldx, bool x_vec_ok, int64_t L,
                         int maxseg, double* __restrict__ ws, double* __restrict__ y, int64_t ldy,
-                        double* __restrict__ state, double decay, bool red32, BandCount seen) {
+                        double* __restrict__ state, double decay, bool red32, unsigned* __restrict__ seen) {
   constexpr int V = ScaledTraits<FMT>::V;
   constexpr int NG = 32 / GL;  // pieces taken at once
   const int lane = threadIdx.x & 31;
@@ -179,7 +179,8 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, R > 1 ? 1 : FMT == 7 && GL 
       const bool shared = g_lo != g_hi;
       band_finish<0, R>(hi, lo, lane, 4 * I, M, shared ? ws + (I * maxseg + (g - g_lo)) * R * 4 : nullptr, y, ldy, state,
                         decay, red32);
-      if (shared) finish_shared_band(seen, ws, I, M, (int)(g_hi - g_lo + 1), maxseg, R, y, ldy, state, decay);
+      if (shared)
+        finish_shared_band(seen, ws, I, M, (int)(g - g_lo), (int)(g_hi - g_lo + 1), maxseg, R, y, ldy, state, decay);
       b0 = piece_end;
     } else {  // lane group lane / GL takes the piece of band b0 / CB + lane / GL
       const int64_t I0 = div64(b0, CB), I = I0 + lane / GL;
@@ -193,7 +194,8 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, R > 1 ? 1 : FMT == 7 && GL 
       const bool shared = active && g_lo != g_hi;
       band_finish<0, R, GL>(hi, lo, gl, 4 * I, M, shared ? ws + (I * maxseg + (g - g_lo)) * R * 4 : nullptr, y, ldy, state,
                             decay, red32, active);
-      finish_shared_groups<GL>(seen, ws, I, M, (int)(g_hi - g_lo + 1), shared, maxseg, R, y, ldy, state, decay);
+      finish_shared_groups<GL>(seen, ws, I, M, (int)(g - g_lo), (int)(g_hi - g_lo + 1), shared, maxseg, R, y, ldy, state,
+                               decay);
       b0 = min(b1, (I0 + NG) * CB);
     }
   }

@@ -3,7 +3,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -39,9 +38,7 @@ struct whff_handle {
   uint8_t* h_stream = nullptr;  // host-resident handles: the pinned, mapped host copy behind d_stream
   double* d_ws = nullptr;       // split-K partials: ksplit x max_rhs x Mpad
   size_t ws_bytes = 0;
-  unsigned long long* d_seen = nullptr;   // per band: tag and written segments of the latest pass (BandCount)
-  int64_t seen_bands = 0;
-  std::atomic<uint64_t>* passes = nullptr;  // passes that counted there so far (shared with row views)
+  unsigned* d_seen = nullptr;   // per band: counts the written segments of a pass (finish_shared_band)
   int* d_status = nullptr;      // device-side error word
   float* d_x = nullptr;         // staging for whff_step_host
   double* d_y = nullptr;
@@ -254,33 +251,14 @@ int launch_wz1(const whff_handle* h, const float* x, int R, int64_t ldx, bool ve
   }
 }
 
-// The band counters of a pass that shares bands.  A captured pass keeps one tag for all
-// its replays, so its counters are cleared by a node of their own (all of them: a row
-// view's graph is updated in place for other views).
-int band_count(const whff_handle* h, bool shared, cudaStream_t st, BandCount* out) {
-  *out = BandCount{h->d_seen, 0};
-  if (!shared) return WHFF_OK;
-  out->tag = (h->passes->fetch_add(1, std::memory_order_relaxed) + 1) << kBandCountBits;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {  // the legacy stream beside another one's capture
-    cudaGetLastError();
-    cap = cudaStreamCaptureStatusNone;
-  }
-  if (cap == cudaStreamCaptureStatusActive)
-    WHFF_CUDA_TRY(cudaMemsetAsync(h->d_seen, 0, (size_t)h->seen_bands * sizeof(*h->d_seen), st));
-  return WHFF_OK;
-}
-
 int launch_wz2(const whff_handle* h, const float* x, int R, int64_t ldx, bool vec, double* y, int64_t ldy,
                double* state, double decay, cudaStream_t st) {
   // the staged kernel needs a padded device stream aligned for its bulk copies
   const bool staged = h->bulk && R == 1 && !h->groups8 && !h->h_stream &&
                       reinterpret_cast<uintptr_t>(h->d_stream) % (h->info.rate % 8 == 0 ? 16 : 8) == 0;
-  BandCount seen;
-  if (const int be = band_count(h, h->maxseg > 1 && !staged, st, &seen)) return be;
   Wz2Step a{h->d_stream, h->info.M, h->info.N, h->BM, h->BN, x, ldx, vec, h->range_len, h->maxseg, h->d_ws,
             y, ldy, state, decay, h->range_ctas, R == 1 ? h->unroll : 2, h->info.fmt == WHFF_FMT_FIXED_LIFT, R,
-            h->red32, h->groups8, h->d_xt, staged, h->d_status, seen};
+            h->red32, h->groups8, h->d_xt, staged, h->d_status, h->d_seen};
   int e;
   switch (h->info.rate) {
     case 8: e = wz2_launch<8>(a, st); break;
@@ -323,10 +301,8 @@ int launch_scaled(const whff_handle* h, const float* x, int R, int64_t ldx, bool
                   double* state, double decay, cudaStream_t st) {
   const auto& b = h->info;
   const int64_t ld = scaled_ld(b.N);
-  BandCount seen;
-  if (const int be = band_count(h, h->maxseg > 1, st, &seen)) return be;
   ScaledStep a{b.fmt, h->d_stream, h->d_scales, b.M, b.N, ld, ceil_div(b.N, kScaleTile), x, ldx, vec,
-               h->range_len, h->maxseg, h->d_ws, y, ldy, state, decay, h->range_ctas, R, h->red32, h->groups8, seen};
+               h->range_len, h->maxseg, h->d_ws, y, ldy, state, decay, h->range_ctas, R, h->red32, h->groups8, h->d_seen};
   if (scaled_launch(a, st)) {
     set_error("whff_step: scaled formats take R 1, 2, 4 or 8 per pass");
     return WHFF_EINVAL;
@@ -354,11 +330,9 @@ int launch_pass(const whff_handle* h, const float* x, int R, int64_t ldx, double
       break;
     case WHFF_FMT_FIXED_ACC: {
       const bool wide = R == 8;
-      BandCount seen;
-      if ((e = band_count(h, (wide ? h->wz3_maxseg8 : h->maxseg) > 1, st, &seen))) break;
       Wz3Step a{h->wz3_index, h->wz3_area, h->band0, h->info.M, h->info.N, h->BM, h->BN, h->wz3_RB, x, ldx,
                 h->d_xt, R, wide ? h->wz3_L8 : h->range_len, wide ? h->wz3_maxseg8 : h->maxseg,
-                wide ? h->wz3_ctas8 : h->range_ctas, h->d_ws, y, ldy, state, decay, seen};
+                wide ? h->wz3_ctas8 : h->range_ctas, h->d_ws, y, ldy, state, decay, h->d_seen};
       e = wz3_launch(a, st) ? WHFF_EINVAL : WHFF_OK;
       if (e) set_error("whff_step: fixed-accuracy passes take 1 or 8 right-hand sides");
       break;
@@ -526,8 +500,6 @@ int create_impl(const BlobInfo& info, const uint8_t* src, int max_rhs, unsigned 
     }
   }
   choose_split(h);
-  h->seen_bands = h->BM;
-  h->passes = new std::atomic<uint64_t>(0);
   // short bands (tall matrices) fold their lanes in FP32 pairs, long ones in
   // triples; very short ones give each band a group of 8 lanes.  BN counts a
   // band's lane work units: 4-column blocks (WZ2) or 16-byte chunks (scaled).
@@ -586,7 +558,7 @@ int create_impl(const BlobInfo& info, const uint8_t* src, int max_rhs, unsigned 
   if (((info.fmt == WHFF_FMT_FIXED_LIFT || is_wz3(info.fmt)) && cudaMalloc(&h->d_xt, xt_bytes(h)) != cudaSuccess) ||
       (h->ws_bytes && cudaMalloc(&h->d_ws, h->ws_bytes) != cudaSuccess) ||
       cudaMalloc(&h->d_status, sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&h->d_seen, (size_t)h->seen_bands * sizeof(*h->d_seen)) != cudaSuccess ||
+      cudaMalloc(&h->d_seen, (size_t)h->BM * sizeof(unsigned)) != cudaSuccess ||
       cudaMalloc(&h->d_x, (size_t)info.N * (size_t)max_rhs * sizeof(float)) != cudaSuccess ||
       cudaMalloc(&h->d_y, (size_t)info.M * (size_t)max_rhs * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
@@ -601,7 +573,7 @@ int create_impl(const BlobInfo& info, const uint8_t* src, int max_rhs, unsigned 
   if (h->map_count) h->d_map = h->d_btiles + h->btile_bytes;
   // everything on st, and complete before any other stream can use the handle
   if (cudaMemsetAsync(h->d_status, 0, sizeof(int), st) != cudaSuccess ||
-      cudaMemsetAsync(h->d_seen, 0, (size_t)h->seen_bands * sizeof(*h->d_seen), st) != cudaSuccess ||
+      cudaMemsetAsync(h->d_seen, 0, (size_t)h->BM * sizeof(unsigned), st) != cudaSuccess ||
       (h->d_map && cudaMemcpyAsync(h->d_map, map, sizeof(map), cudaMemcpyHostToDevice, st) != cudaSuccess) ||
       (!h->h_stream && src &&
        cudaMemcpyAsync(h->d_stream, src, info.stream_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess) ||
@@ -639,7 +611,7 @@ extern "C" int whff_info(const whff_handle* h, int* fmt, int* rate, int64_t* M, 
   if (N) *N = h->info.N;
   if (device_bytes)
     *device_bytes = (h->h_stream ? 0 : h->info.stream_bytes) + h->ws_bytes + h->ws_mma_bytes + sizeof(int) +
-                    (size_t)h->seen_bands * sizeof(*h->d_seen) +
+                    (size_t)h->BM * sizeof(unsigned) +
                     (size_t)h->info.N * h->max_rhs * 4 + (size_t)h->info.M * h->max_rhs * 8 +
                     (h->d_xt ? xt_bytes(h) : 0);
   return WHFF_OK;
@@ -1187,7 +1159,6 @@ extern "C" void whff_destroy(whff_handle* h) {
   cudaFree(h->d_x);
   cudaFree(h->d_y);
   cudaGetLastError();
-  delete h->passes;
   delete h;
 }
 

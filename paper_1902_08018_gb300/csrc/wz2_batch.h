@@ -4,17 +4,6 @@
 #include <cstdint>
 
 namespace whff {
-
-// The segments of a pass's shared bands that have been written: count[I] is the tag of
-// the latest pass over band I plus its segments so far.  A tag is the pass's number in
-// its handle times 2^kBandCountBits; a pass counts up from its own tag, so that what
-// earlier passes left behind does not matter, be it that two of them overlapped.
-struct BandCount {
-  unsigned long long* count;
-  unsigned long long tag;
-};
-constexpr int kBandCountBits = 20;  // above the warps of any grid
-
 namespace dev {
 
 // One matrix of a batch: its compressed stream, vectors and place in the

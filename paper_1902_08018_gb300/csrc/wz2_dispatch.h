@@ -45,7 +45,7 @@ struct Wz2Step {
   float* xt;       // lift: scratch for (2G)^T x, 4 BN floats per right-hand side (8 columns)
   bool staged;     // R = 1: stream each warp's range through shared memory by bulk copies
   int* status;     // device status word (bounded waits of the staged kernel)
-  BandCount seen;  // segments of the pass written so far
+  unsigned* seen;  // per band: counts the segments of the pass (see finish_shared_band)
 };
 
 // Bytes a handle's device stream allocation carries past the stream, so that
@@ -91,7 +91,7 @@ struct ScaledStep {
   int R;
   bool red32;
   bool groups8;  // four 8-lane groups per warp, one band each (short bands)
-  BandCount seen;  // segments of the pass written so far
+  unsigned* seen;  // per band: counts the segments of the pass
 };
 int scaled_launch(const ScaledStep& a, cudaStream_t st);  // scaled.cu
 
@@ -202,7 +202,7 @@ struct Wz3Step {
   int64_t ldy;
   double* state;
   double decay;
-  BandCount seen;  // segments of the pass written so far
+  unsigned* seen;  // per band: counts the segments of the pass
 };
 int wz3_launch(const Wz3Step& a, cudaStream_t st);
 int wz3_occupancy();  // resident CTAs per SM of the R = 1 kernel (0 on error)

@@ -436,18 +436,23 @@ __device__ __forceinline__ void sum_segments(const double* __restrict__ ws, int6
 
 // After a warp has written its segment of shared band I: the warp that brings the
 // band's last of nseg segments adds them up (the order of the sum is the segments',
-// whoever does it).  The count starts from the pass's own tag, which is above all that
-// an earlier pass left, so nothing that happened before can reach it.  A kernel of its
-// own for these few sums cost 4 us of launch and latency per pass.
-__device__ __forceinline__ void finish_shared_band(BandCount seen, const double* __restrict__ ws, int64_t I,
-                                                   int64_t M, int nseg, int maxseg, int R, double* __restrict__ y,
+// whoever does it).  A kernel of its own for these few sums cost 4 us of launch and
+// latency per pass.
+// The band's counter is taken modulo 2^20, above the warps of any grid: a band's first
+// segment adds 2^20 - (nseg - 1), each other one 1, so that the count is 0 again when the
+// last has come and not before.  Every finished pass adds 0 whatever its segments, so
+// none can leave anything to the next one, even if two of them overlapped; a counter that
+// the last warp sets back is off for good after that.
+constexpr unsigned kSeenPeriod = 1u << 20;
+__device__ __forceinline__ void finish_shared_band(unsigned* __restrict__ seen, const double* __restrict__ ws, int64_t I,
+                                                   int64_t M, int seg, int nseg, int maxseg, int R, double* __restrict__ y,
                                                    int64_t ldy, double* __restrict__ state, double decay) {
   __threadfence();
   __syncwarp();
   int last = 0;
   if ((threadIdx.x & 31) == 0) {
-    (void)atomicMax(seen.count + I, seen.tag);
-    last = atomicAdd(seen.count + I, 1ull) == seen.tag + (unsigned)(nseg - 1);
+    const unsigned add = seg == 0 ? kSeenPeriod - (unsigned)(nseg - 1) : 1u;
+    last = (atomicAdd(seen + I, add) + add) % kSeenPeriod == 0;
   }
   last = __shfl_sync(0xffffffffu, last, 0);
   if (!last) return;
@@ -457,16 +462,16 @@ __device__ __forceinline__ void finish_shared_band(BandCount seen, const double*
 
 // The same for the four lane groups of a warp, each with a piece of a band of its own.
 template <int GL>
-__device__ __forceinline__ void finish_shared_groups(BandCount seen, const double* __restrict__ ws, int64_t I,
-                                                     int64_t M, int nseg, bool shared, int maxseg, int R,
+__device__ __forceinline__ void finish_shared_groups(unsigned* __restrict__ seen, const double* __restrict__ ws, int64_t I,
+                                                     int64_t M, int seg, int nseg, bool shared, int maxseg, int R,
                                                      double* __restrict__ y, int64_t ldy, double* __restrict__ state,
                                                      double decay) {
   if (!__any_sync(0xffffffffu, shared)) return;
 #pragma unroll 1
   for (int g = 0; g < 32; g += GL) {
     if (!__shfl_sync(0xffffffffu, (int)shared, g)) continue;
-    finish_shared_band(seen, ws, __shfl_sync(0xffffffffu, I, g), M, __shfl_sync(0xffffffffu, nseg, g), maxseg, R, y,
-                       ldy, state, decay);
+    finish_shared_band(seen, ws, __shfl_sync(0xffffffffu, I, g), M, __shfl_sync(0xffffffffu, seg, g),
+                       __shfl_sync(0xffffffffu, nseg, g), maxseg, R, y, ldy, state, decay);
   }
 }
 
@@ -484,7 +489,7 @@ template <int RATE, bool LIFT, int R, int UNROLL, int GL, bool PRE>
 __device__ __forceinline__ void wz2_gemv_body(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM,
                                               int64_t BN, const float* __restrict__ x, int64_t ldx, bool x_vec_ok,
                                               int64_t L, int maxseg, double* __restrict__ ws, double* __restrict__ y,
-                                              int64_t ldy, double* __restrict__ state, double decay, bool red32, BandCount seen) {
+                                              int64_t ldy, double* __restrict__ state, double decay, bool red32, unsigned* __restrict__ seen) {
   constexpr int64_t kBlockBytes = 4 * Wz2Layout<RATE>::kWords;
   constexpr int NG = 32 / GL;  // pieces taken at once
   const int lane = threadIdx.x & 31;
@@ -511,7 +516,8 @@ __device__ __forceinline__ void wz2_gemv_body(const uint8_t* __restrict__ stream
       const bool shared = g_lo != g_hi;
       band_finish<LIFT ? 1 : 2, R>(hi, lo, lane, 4 * I, M, shared ? ws + (I * maxseg + (g - g_lo)) * R * 4 : nullptr, y,
                                    ldy, state, decay, red32);
-      if (shared) finish_shared_band(seen, ws, I, M, (int)(g_hi - g_lo + 1), maxseg, R, y, ldy, state, decay);
+      if (shared)
+        finish_shared_band(seen, ws, I, M, (int)(g - g_lo), (int)(g_hi - g_lo + 1), maxseg, R, y, ldy, state, decay);
       b0 = piece_end;
     } else {  // lane group lane / GL takes the piece of band b0 / BN + lane / GL
       const int64_t I0 = div64(b0, BN), I = I0 + lane / GL;
@@ -525,7 +531,8 @@ __device__ __forceinline__ void wz2_gemv_body(const uint8_t* __restrict__ stream
       const bool shared = active && g_lo != g_hi;
       band_finish<LIFT ? 1 : 2, R, GL>(hi, lo, gl, 4 * I, M, shared ? ws + (I * maxseg + (g - g_lo)) * R * 4 : nullptr, y,
                                        ldy, state, decay, red32, active);
-      finish_shared_groups<GL>(seen, ws, I, M, (int)(g_hi - g_lo + 1), shared, maxseg, R, y, ldy, state, decay);
+      finish_shared_groups<GL>(seen, ws, I, M, (int)(g - g_lo), (int)(g_hi - g_lo + 1), shared, maxseg, R, y, ldy, state,
+                               decay);
       b0 = min(b1, (I0 + NG) * BN);
     }
   }
@@ -546,7 +553,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? wz2_ctas_per_sm<RA
     wz2_gemv_kernel(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM, int64_t BN,
                     const float* __restrict__ x, int64_t ldx, bool x_vec_ok, int64_t L, int maxseg,
                     double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
-                    double decay, bool red32, BandCount seen) {
+                    double decay, bool red32, unsigned* __restrict__ seen) {
   wz2_gemv_body<RATE, LIFT, R, UNROLL, GL, PRE>(stream, M, N, BM, BN, x, ldx, x_vec_ok, L, maxseg, ws, y, ldy, state,
                                            decay, red32, seen);
 }

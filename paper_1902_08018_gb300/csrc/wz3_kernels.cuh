@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
     wz3_gemv_kernel(const uint64_t* __restrict__ index, const uint8_t* __restrict__ area, int64_t M, int64_t BM,
                     int BN, int RB, const float* __restrict__ xt, int64_t ldt, int64_t L, int maxseg,
                     double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
-                    double decay, BandCount seen) {
+                    double decay, unsigned* __restrict__ seen) {
   const int lane = threadIdx.x & 31;
   const int64_t g = (int64_t)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
   const int64_t total = BM * RB;
@@ -196,7 +196,8 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
     const bool shared = g_lo != g_hi;
     band_finish<1, R>(hi, lo, lane, 4 * I, M, shared ? ws + (I * maxseg + (g - g_lo)) * R * 4 : nullptr, y, ldy, state,
                       decay, false);
-    if (shared) finish_shared_band(seen, ws, I, M, (int)(g_hi - g_lo + 1), maxseg, R, y, ldy, state, decay);
+    if (shared)
+      finish_shared_band(seen, ws, I, M, (int)(g - g_lo), (int)(g_hi - g_lo + 1), maxseg, R, y, ldy, state, decay);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -275,7 +276,7 @@ __device__ __forceinline__ int64_t wz3_groups(int64_t BM) { return (BM + 7) / 8;
 static __global__ void __launch_bounds__(kWarpsPerCta * 32, 2)
     wz3_gemv8_kernel(const uint64_t* __restrict__ index, const uint8_t* __restrict__ area, int64_t M, int64_t BM,
                      int BN, int RB, const float* __restrict__ xt, int64_t L, int maxseg, double* __restrict__ ws,
-                     double* __restrict__ y, int64_t ldy, double* __restrict__ state, double decay, BandCount seen) {
+                     double* __restrict__ y, int64_t ldy, double* __restrict__ state, double decay, unsigned* __restrict__ seen) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t u0 = (int64_t)blockIdx.x * L, u1 = min(wz3_groups(BM) * RB, u0 + L);
   for (int64_t ub = u0; ub < u1;) {  // the range's piece of group G: runs [q0, q1) of each of its bands
@@ -322,7 +323,8 @@ static __global__ void __launch_bounds__(kWarpsPerCta * 32, 2)
     const bool shared = c_lo != c_hi;
     band_write<1, 8, 32>(z, lane, 4 * I, M, shared ? ws + (I * maxseg + (blockIdx.x - c_lo)) * 32 : nullptr, y, ldy,
                          state, decay, true);
-    if (shared) finish_shared_band(seen, ws, I, M, (int)(c_hi - c_lo + 1), maxseg, 8, y, ldy, state, decay);
+    if (shared)
+      finish_shared_band(seen, ws, I, M, (int)(blockIdx.x - c_lo), (int)(c_hi - c_lo + 1), maxseg, 8, y, ldy, state, decay);
   }
 }
 
