@@ -184,7 +184,8 @@ int whff_info(const whff_handle* h, int* fmt, int* rate, int64_t* M, int64_t* N,
 /* Launch plan of a resident matrix: *ksplit = column splits per 4-row band
  * (1 for matrices with enough rows to fill the GPU), *launches = kernel
  * launches of one CUDA-core whff_step pass: the fused kernel, the epilogue of
- * split-K (or of shared bands, bulk-staged) if any, and the (2G)^T x transform of x
+ * split-K (or of shared bands: bulk-staged, and above 2^21 blocks with four or
+ * eight blocks in flight) if any, and the (2G)^T x transform of x
  * where the fused kernel reads it: FIXED_ACC, and FIXED_LIFT unless the kernel
  * transforms x itself (two blocks in flight, up to 2^24 blocks at rate 8, 2^25 at 12, else 2^26). */
 int whff_plan(const whff_handle* h, int* ksplit, int* launches);

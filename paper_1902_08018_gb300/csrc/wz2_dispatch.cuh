@@ -7,9 +7,9 @@
 
 namespace whff {
 
-template <int RATE, bool LIFT, int R, int U, int GL = 32, bool PRE = LIFT>
+template <int RATE, bool LIFT, int R, int U, int GL = 32, bool PRE = LIFT, bool FIN = true>
 static void wz2_launch_one(const Wz2Step& a, cudaStream_t st) {
-  dev::wz2_gemv_kernel<RATE, LIFT, R, U, GL, PRE><<<(unsigned)a.ctas, dev::kWarpsPerCta * 32, 0, st>>>(
+  dev::wz2_gemv_kernel<RATE, LIFT, R, U, GL, PRE, FIN><<<(unsigned)a.ctas, dev::kWarpsPerCta * 32, 0, st>>>(
       a.stream, a.M, a.N, a.BM, a.BN, a.x, a.ldx, a.x_vec_ok, a.L, a.maxseg, a.ws, a.y, a.ldy, a.state, a.decay,
       a.red32, a.seen);
 }
@@ -28,6 +28,23 @@ static int wz2_stream_smem_attr() {
   return 0;
 }
 
+static inline void wz2_launch_epilogue(const Wz2Step& a, cudaStream_t st) {
+  if (a.maxseg > 1)
+    dev::wz2_segment_epilogue<<<(unsigned)((dev::segment_epilogue_threads(a.M, a.BN, a.L) + 255) / 256), 256, 0, st>>>(
+        a.ws, a.M, a.BN, a.L, a.maxseg, a.R, a.y, a.ldy, a.state, a.decay);
+}
+
+// One column, U (4 or 8) blocks in flight.
+template <int RATE, bool LIFT, int U>
+static void wz2_launch_deep(const Wz2Step& a, cudaStream_t st) {
+  if (a.BM * a.BN <= wz2_finish_blocks(U)) {
+    wz2_launch_one<RATE, LIFT, 1, U>(a, st);
+  } else {
+    wz2_launch_one<RATE, LIFT, 1, U, 32, LIFT, false>(a, st);
+    wz2_launch_epilogue(a, st);
+  }
+}
+
 template <int RATE, bool LIFT>
 static int wz2_launch_lift(const Wz2Step& a, cudaStream_t st) {
   if (a.staged && a.R == 1 && !a.groups8) {
@@ -35,9 +52,7 @@ static int wz2_launch_lift(const Wz2Step& a, cudaStream_t st) {
     dev::wz2_stream_kernel<RATE, LIFT><<<(unsigned)a.ctas, dev::kWarpsPerCta * 32, dev::Wz2Stream<RATE>::kSmemBytes,
                                          st>>>(a.stream, a.M, a.N, a.BM, a.BN, a.x, a.ldx, a.x_vec_ok, a.L, a.maxseg,
                                                a.ws, a.y, a.ldy, a.state, a.decay, a.red32, a.status);
-    if (a.maxseg > 1)
-      dev::wz2_segment_epilogue<<<(unsigned)((dev::segment_epilogue_threads(a.M, a.BN, a.L) + 255) / 256), 256, 0, st>>>(
-          a.ws, a.M, a.BN, a.L, a.maxseg, a.R, a.y, a.ldy, a.state, a.decay);
+    wz2_launch_epilogue(a, st);
   } else if (a.groups8) {  // short bands: four 8-lane groups per warp, two blocks in flight per lane
     switch (a.R) {
       case 1: wz2_launch_one<RATE, LIFT, 1, 2, 8>(a, st); break;
@@ -48,8 +63,8 @@ static int wz2_launch_lift(const Wz2Step& a, cudaStream_t st) {
     }
   } else switch (a.R) {
     case 1:
-      if (a.unroll == 8) wz2_launch_one<RATE, LIFT, 1, 8>(a, st);
-      else if (a.unroll == 4) wz2_launch_one<RATE, LIFT, 1, 4>(a, st);
+      if (a.unroll == 8) wz2_launch_deep<RATE, LIFT, 8>(a, st);
+      else if (a.unroll == 4) wz2_launch_deep<RATE, LIFT, 4>(a, st);
       else wz2_launch_one<RATE, LIFT, 1, 2>(a, st);
       break;
     case 2: wz2_launch_one<RATE, LIFT, 2, 2>(a, st); break;

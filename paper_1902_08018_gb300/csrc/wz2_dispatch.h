@@ -23,6 +23,17 @@ constexpr uint32_t kWaitPolls = 1u << 22;
 // the others gain up to there, the longest measured.
 constexpr int64_t wz2_fuse_blocks(int rate) { return (int64_t)1 << (rate == 8 ? 24 : rate == 12 ? 25 : 26); }
 
+// Blocks up to which the one-column kernels with four or eight blocks in flight add the
+// segments of shared bands themselves.  The fence and the atomics of that make the loop
+// before them slower, a launch of its own costs 2 us.  In the kernel / launched, us:
+//   378 x 32768, rate 16, four in flight: 20.6 / 22.6; eight: 18.5 / 20.6
+//   8192^2 (2^22 blocks): 35.9 / 36.0; 40.1 / 38.3
+//   16384^2, rates 8 12 16, four: 82.1 86.2 95.8 / 78.0 81.6 94.0
+//   32768^2: 285.2 293.0 334.7 / 258.9 275.8 329.2; rate 8, eight: 278.4 / 253.8
+// With two in flight the loop gains nothing (16384^2: 84.2 84.3 94.1 / 86.2 87.7 96.0;
+// 32768^2: 282.3 282.1 332.4 / 280.1 287.7 330.2), so they always add their own.
+constexpr int64_t wz2_finish_blocks(int unroll) { return unroll == 2 ? INT64_MAX : (int64_t)1 << 21; }
+
 struct Wz2Step {
   const uint8_t* stream;
   int64_t M, N, BM, BN;

@@ -484,8 +484,9 @@ __device__ __forceinline__ void finish_shared_groups(unsigned* __restrict__ seen
 // groups take the next four pieces at once (short bands, where a warp per
 // band would spend its time folding).  PRE: x is the transformed vector of
 // wz2_xt_kernel (4 BN floats per right-hand side); otherwise, with the lift, every
-// block transforms its own four values.
-template <int RATE, bool LIFT, int R, int UNROLL, int GL, bool PRE>
+// block transforms its own four values.  FIN: the band's last warp adds its segments
+// here; otherwise wz2_segment_epilogue does (see wz2_finish_blocks).
+template <int RATE, bool LIFT, int R, int UNROLL, int GL, bool PRE, bool FIN>
 __device__ __forceinline__ void wz2_gemv_body(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM,
                                               int64_t BN, const float* __restrict__ x, int64_t ldx, bool x_vec_ok,
                                               int64_t L, int maxseg, double* __restrict__ ws, double* __restrict__ y,
@@ -520,7 +521,7 @@ __device__ __forceinline__ void wz2_gemv_body(const uint8_t* __restrict__ stream
       const bool shared = g_lo != g_hi;
       band_finish<LIFT ? 1 : 2, R>(hi, lo, lane, 4 * I, M, shared ? ws + (I * maxseg + (self - g_lo)) * R * 4 : nullptr,
                                    y, ldy, state, decay, red32);
-      if (shared)
+      if (FIN && shared)
         finish_shared_band(seen, ws, I, M, (int)(self - g_lo), (int)(g_hi - g_lo + 1), maxseg, R, y, ldy, state, decay);
       b0 = piece_end;
     } else {  // lane group lane / GL takes the piece of band b0 / BN + lane / GL
@@ -552,13 +553,13 @@ __host__ __device__ constexpr int wz2_ctas_per_sm(int unroll) {
   return unroll == 8 ? (RATE <= 8 ? 3 : RATE <= 20 ? 2 : 1) : unroll == 4 ? (RATE <= 16 ? 3 : 2) : RATE <= 16 ? 4 : 3;
 }
 
-template <int RATE, bool LIFT, int R, int UNROLL, int GL, bool PRE = LIFT>
+template <int RATE, bool LIFT, int R, int UNROLL, int GL, bool PRE = LIFT, bool FIN = true>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? wz2_ctas_per_sm<RATE>(UNROLL) : 1)
     wz2_gemv_kernel(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM, int64_t BN,
                     const float* __restrict__ x, int64_t ldx, bool x_vec_ok, int64_t L, int maxseg,
                     double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
                     double decay, bool red32, unsigned* __restrict__ seen) {
-  wz2_gemv_body<RATE, LIFT, R, UNROLL, GL, PRE>(stream, M, N, BM, BN, x, ldx, x_vec_ok, L, maxseg, ws, y, ldy, state,
+  wz2_gemv_body<RATE, LIFT, R, UNROLL, GL, PRE, FIN>(stream, M, N, BM, BN, x, ldx, x_vec_ok, L, maxseg, ws, y, ldy, state,
                                            decay, red32, seen);
 }
 
