@@ -132,6 +132,7 @@ __device__ __forceinline__ void band_finish(const float (&hi)[4][R], const float
                                             int64_t M, double* __restrict__ part, double* __restrict__ y, int64_t ldy,
                                             double* __restrict__ state, double decay, bool red32, bool active = true) {
   constexpr int N = 4 * R;
+  if constexpr (R > 1) asm volatile("" : "+r"(lane));  // the fold's lane constants stay out of the caller's loops
   float h[N], l[N];
 #pragma unroll
   for (int k = 0; k < N; ++k) h[k] = hi[k & 3][k >> 2], l[k] = lo[k & 3][k >> 2];

@@ -145,11 +145,19 @@ __device__ __forceinline__ void scaled_piece(const uint8_t* __restrict__ payload
   }
 }
 
+// CTAs per SM that the kernels are held to: the occupancy that the one-column plans
+// count on, and two for the few columns that fit 128 registers (two columns in BF16 at
+// 10000^2: 50 us; 65 us at one CTA per SM).
+template <int FMT, int R, int GL>
+__host__ __device__ constexpr int scaled_ctas_per_sm() {
+  return R == 1 ? (FMT == 7 && GL == 32 ? 3 : 2) : (R == 2 && FMT != 4) || (R == 4 && FMT == 7) ? 2 : 1;
+}
+
 // GL = 32: the warp takes one piece of a band at a time; GL = 8: four lane
 // groups take the next four pieces at once (short bands, where a warp per
 // band would spend its time folding).
 template <int FMT, int R, int GL>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, R > 1 ? 1 : FMT == 7 && GL == 32 ? 3 : 2)
+__global__ void __launch_bounds__(kWarpsPerCta * 32, scaled_ctas_per_sm<FMT, R, GL>())
     scaled_range_kernel(const uint8_t* __restrict__ payload, const float* __restrict__ scales, int64_t M, int64_t N,
                         int64_t ld, int64_t TN, const float* __restrict__ x, int64_t ldx, bool x_vec_ok, int64_t L,
                         int maxseg, double* __restrict__ ws, double* __restrict__ y, int64_t ldy,

@@ -553,8 +553,10 @@ __host__ __device__ constexpr int wz2_ctas_per_sm(int unroll) {
   return unroll == 8 ? (RATE <= 8 ? 3 : RATE <= 20 ? 2 : 1) : unroll == 4 ? (RATE <= 16 ? 3 : 2) : RATE <= 16 ? 4 : 3;
 }
 
+// Four columns: two CTAs per SM (rate 16, 10000^2: 140 us; 209 us with the 158 registers
+// that one would allow).
 template <int RATE, bool LIFT, int R, int UNROLL, int GL, bool PRE = LIFT, bool FIN = true>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? wz2_ctas_per_sm<RATE>(UNROLL) : 1)
+__global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? wz2_ctas_per_sm<RATE>(UNROLL) : R == 4 ? 2 : 1)
     wz2_gemv_kernel(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM, int64_t BN,
                     const float* __restrict__ x, int64_t ldx, bool x_vec_ok, int64_t L, int maxseg,
                     double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
@@ -620,7 +622,7 @@ __device__ __forceinline__ void batch_band_span(const BatchEntry& e, int64_t I, 
 // One column: held to the CTAs per SM that its grid is made for (wz2_occupancy);
 // at three where the grid counts on four, a quarter of it ran alone at the end.
 template <int RATE, bool LIFT, int R, int UNROLL>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? wz2_ctas_per_sm<RATE>(UNROLL) : 1)
+__global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? wz2_ctas_per_sm<RATE>(UNROLL) : R == 4 ? 2 : 1)
     wz2_batched_kernel(const BatchEntry* __restrict__ entries, int nentries, int64_t total, int64_t L) {
   constexpr int64_t kBlockBytes = 4 * Wz2Layout<RATE>::kWords;
   const int lane = threadIdx.x & 31;
