@@ -10,19 +10,6 @@
 
 namespace whff {
 
-// Raise a kernel's dynamic shared-memory limit.  The limit belongs to the kernel on
-// one device (and context): every launch sets it, as one process may use several.
-template <class K>
-static int scaled_set_smem(K kern, int bytes) {
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
-      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
-          cudaSuccess) {
-    cudaGetLastError();
-    return -1;
-  }
-  return 0;
-}
-
 template <int FMT, int NR>
 static int scaled_mma_one(const ScaledMmaStep& a, cudaStream_t st) {
   using S = dev::ScaledMmaSmem<FMT, NR>;
@@ -30,9 +17,9 @@ static int scaled_mma_one(const ScaledMmaStep& a, cudaStream_t st) {
   constexpr bool kF16 = FMT == 3;
   const bool tma = (FMT == 2 || FMT == 3) && a.tmap != nullptr;
   const bool fp8 = FMT == 4 && a.tmap != nullptr;
-  if (fp8   ? scaled_set_smem(dev::fp8_mma_kernel<NR>, dev::Fp8Smem<NR>::kBytes)
-      : tma ? scaled_set_smem(dev::scaled_mma_tma_kernel<NR, kF16>, dev::TmaSmem<NR>::kBytes)
-            : scaled_set_smem(kern, S::kBytes))
+  if (fp8   ? raise_smem<dev::fp8_mma_kernel<NR>>(dev::Fp8Smem<NR>::kBytes, false)
+      : tma ? raise_smem<dev::scaled_mma_tma_kernel<NR, kF16>>(dev::TmaSmem<NR>::kBytes, true)
+            : raise_smem<dev::scaled_mma_kernel<FMT, NR>>(S::kBytes, true))
     return -1;
   const int nstages = (int)((a.N + 63) / 64);
   const int tiles = (int)((a.M + 127) / 128);
@@ -90,7 +77,7 @@ static int scaled_mma_occ_one() {
   auto kern = dev::scaled_mma_kernel<FMT, NR>;
   cudaFuncAttributes fa;
   int dev = 0, smem_sm = 0, regs_sm = 0, reserved = 0;
-  if (scaled_set_smem(kern, S::kBytes) ||
+  if (raise_smem<dev::scaled_mma_kernel<FMT, NR>>(S::kBytes, true) ||
       cudaFuncGetAttributes(&fa, kern) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess ||
@@ -113,7 +100,8 @@ static int scaled_tma_occ_one() {
   auto kern = dev::scaled_mma_tma_kernel<NR, F16>;
   cudaFuncAttributes fa;
   int dev = 0, smem_sm = 0, regs_sm = 0, reserved = 0;
-  if (scaled_set_smem(kern, dev::TmaSmem<NR>::kBytes) || cudaFuncGetAttributes(&fa, kern) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
+  if (raise_smem<dev::scaled_mma_tma_kernel<NR, F16>>(dev::TmaSmem<NR>::kBytes, true) ||
+      cudaFuncGetAttributes(&fa, kern) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess) {

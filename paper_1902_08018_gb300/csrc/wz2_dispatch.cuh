@@ -16,16 +16,7 @@ static void wz2_launch_one(const Wz2Step& a, cudaStream_t st) {
 
 template <int RATE, bool LIFT>
 static int wz2_stream_smem_attr() {
-  static int done = 0;  // once per instantiation and process (the attribute is per function)
-  if (!done) {
-    if (cudaFuncSetAttribute(dev::wz2_stream_kernel<RATE, LIFT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             dev::Wz2Stream<RATE>::kSmemBytes) != cudaSuccess) {
-      cudaGetLastError();
-      return -1;
-    }
-    done = 1;
-  }
-  return 0;
+  return raise_smem<dev::wz2_stream_kernel<RATE, LIFT>>(dev::Wz2Stream<RATE>::kSmemBytes, false);
 }
 
 static inline void wz2_launch_epilogue(const Wz2Step& a, cudaStream_t st) {

@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 
 #include "wz2_batch.h"
@@ -12,6 +13,30 @@ namespace whff {
 // Polls of a bounded device-side wait (tensor-core kernels) before it gives up
 // and records WHFF_ETIMEOUT: about a second of try_wait.
 constexpr uint32_t kWaitPolls = 1u << 22;
+
+// Raise the dynamic shared-memory limit of a kernel.  The limit belongs to the kernel on
+// one device, and a process may use several; it is set on a device's first launch (the
+// two calls cost 1 to 2 us, which a small pass would see).  carveout: ask for all of the
+// SM's memory as shared memory, too.
+template <auto Kern>
+int raise_smem(int bytes, bool carveout) {
+  static std::atomic<uint64_t> done{0};  // a bit per device; devices from 64 on always set it
+  int d = -1;
+  if (cudaGetDevice(&d) != cudaSuccess) {
+    cudaGetLastError();
+    return -1;
+  }
+  const uint64_t bit = d < 64 ? 1ull << d : 0;
+  if (done.load(std::memory_order_acquire) & bit) return 0;
+  if (cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
+      (carveout && cudaFuncSetAttribute(Kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                        cudaSharedmemCarveoutMaxShared) != cudaSuccess)) {
+    cudaGetLastError();
+    return -1;
+  }
+  done.fetch_or(bit, std::memory_order_release);
+  return 0;
+}
 
 // Blocks up to which a one-column pass of the lift transforms x in its kernel: that
 // saves a launch and costs seven additions per block.  Transform launched / fused, us:

@@ -60,6 +60,10 @@ int main() {
         a.maxseg = 4, a.ldy = 256, a.spin = 1, a.map = map;
         if (whff::mma_launch(a, nullptr)) return 3;
       }
+    whff::Wz2Step b{};  // the bulk-staged pass
+    b.M = 256, b.N = 256, b.BM = 64, b.BN = 64, b.ldx = 256, b.L = 4096, b.maxseg = 1, b.ldy = 256, b.ctas = 1, b.unroll = 2;
+    b.lift = true, b.R = 1, b.staged = true;
+    if (whff::wz2_launch<8>(b, nullptr) || whff::wz2_launch<16>(b, nullptr) || whff::wz2_launch<24>(b, nullptr)) return 6;
   }
   std::printf("%d launches, %d large, %d refused\n", g_launches, g_large, g_refused);
   return g_large < 20 ? 4 : g_refused ? 5 : 0;
