@@ -141,10 +141,15 @@ void choose_ranges(whff_handle* h) {
   h->chunk = U;
 }
 
+// Workspace bytes that the 8-column plan needs for its shared groups.
+size_t ws_need_wz3_8(const whff_handle* h) {
+  return h->wz3_maxseg8 > 1 ? (size_t)h->BM * (size_t)h->wz3_maxseg8 * 32 * 8 : 0;
+}
+
 // Fixed accuracy, 8 columns: two CTAs per SM share the (group of 8 bands, run)
 // units in equal ranges, fewer where the partials of shared groups would not
-// fit the workspace (one CTA shares nothing).
-void plan_wz3_8(whff_handle* h) {
+// fit `room` bytes (one CTA shares nothing).
+void plan_wz3_8(whff_handle* h, size_t room) {
   const int64_t RB = ceil_div(h->BN, 32), groups = ceil_div(h->BM, 8), units = groups * RB;
   for (int64_t ctas = std::min<int64_t>(2 * h->sm_count, units);; ctas = std::max<int64_t>(1, ctas * 3 / 4)) {
     h->wz3_L8 = ceil_div(units, ctas);
@@ -153,7 +158,7 @@ void plan_wz3_8(whff_handle* h) {
     for (int64_t G = 0; G < groups; ++G)
       h->wz3_maxseg8 = std::max<int>(h->wz3_maxseg8,
                                      (int)(((G + 1) * RB - 1) / h->wz3_L8 - (G * RB) / h->wz3_L8 + 1));
-    if (h->wz3_maxseg8 == 1 || (size_t)h->BM * (size_t)h->wz3_maxseg8 * 32 * 8 <= h->ws_bytes) break;
+    if (ws_need_wz3_8(h) <= room) break;
   }
 }
 
@@ -526,7 +531,10 @@ int create_impl(const BlobInfo& info, const uint8_t* src, int max_rhs, unsigned 
   if (h->maxseg > 1)
     h->ws_bytes = (size_t)h->BM * (size_t)h->maxseg * (size_t)std::min(max_rhs, kMaxRhsKernel) * 4 * 8;
   h->ws_rhs = std::min(max_rhs, kMaxRhsKernel);
-  if (is_wz3(info.fmt)) plan_wz3_8(h);
+  if (is_wz3(info.fmt) && max_rhs >= 8) {  // its own partials: the one-column plan may share no band at all
+    plan_wz3_8(h, SIZE_MAX);
+    h->ws_bytes = std::max(h->ws_bytes, ws_need_wz3_8(h));
+  }
   const bool wz2 = info.fmt == WHFF_FMT_FIXED_LIFT || info.fmt == WHFF_FMT_FIXED_BFP;
   const bool scaled16 = info.fmt == WHFF_FMT_BF16 || info.fmt == WHFF_FMT_FP16 || info.fmt == WHFF_FMT_FP8E4M3;
   if ((wz2 || scaled16) && max_rhs >= 2) {
@@ -730,7 +738,7 @@ int step_view(const whff_handle* h, int64_t row0, int64_t nrows, const float* x,
     v.ctas_per_sm = --c;
     choose_ranges(&v);
   }
-  if (is_wz3(fmt)) plan_wz3_8(&v);
+  if (is_wz3(fmt) && R >= 8) plan_wz3_8(&v, h->ws_bytes);
   if (h->d_ws_mma) {
     int64_t ctas = (int64_t)h->sm_count * h->mma_occ;
     for (plan_mma(&v, ctas); mma_ws_need(&v, std::min(R, 32)) > h->ws_mma_cap && ctas > 1;
