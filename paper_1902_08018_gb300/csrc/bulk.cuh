@@ -36,27 +36,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
   return false;
 }
 
-// As mbar_try_wait, with the thread suspended for up to ns nanoseconds.
-__device__ __forceinline__ bool mbar_try_wait_for(uint32_t bar, uint32_t parity, uint32_t ns) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity), "r"(ns)
-      : "memory");
-  return ok != 0;
-}
-
 // Bounded wait that also gives up when the CTA's abort flag is raised:
-// 1 done, 0 timed out, -1 aborted elsewhere.  kSuspend: nanoseconds that a poll
-// may suspend the thread, where many warps wait: polling takes issue slots.
-template <uint32_t kSuspend = 0>
+// 1 done, 0 timed out, -1 aborted elsewhere.
 __device__ __forceinline__ int mbar_wait_or_abort(uint32_t bar, uint32_t parity, uint32_t limit,
                                                   const volatile int* abort_flag) {
   for (uint32_t it = 0; it < limit; ++it) {
-    if (kSuspend ? mbar_try_wait_for(bar, parity, kSuspend) : mbar_try_wait(bar, parity)) return 1;
+    if (mbar_try_wait(bar, parity)) return 1;
     if (*abort_flag) return -1;
   }
   return 0;

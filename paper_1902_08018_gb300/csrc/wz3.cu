@@ -15,16 +15,15 @@ int wz3_launch(const Wz3Step& a, cudaStream_t st) {
                                                                 a.L, a.maxseg, a.ws, a.y, a.ldy, a.state, a.decay, a.seen);
     return 0;
   }
-  const int64_t ldt = 4 * a.BN;
-  dev::wz2_xt_kernel<<<(unsigned)((a.BN + 255) / 256), 256, 0, st>>>(a.x, a.ldx, a.N, 1, a.BN, a.xt, ldt);
-  dev::wz3_gemv_kernel<1><<<(unsigned)a.ctas, threads, 0, st>>>(index, a.area, a.M, a.BM, (int)a.BN, (int)a.RB, a.xt,
-                                                                ldt, a.L, a.maxseg, a.ws, a.y, a.ldy, a.state, a.decay, a.seen);
+  dev::wz2_xt_kernel<<<(unsigned)((a.BN + 255) / 256), 256, 0, st>>>(a.x, a.ldx, a.N, 1, a.BN, a.xt, 4 * a.BN);
+  dev::wz3_gemv_kernel<<<(unsigned)a.ctas, threads, 0, st>>>(index, a.area, a.M, a.BM, (int)a.BN, (int)a.RB, a.xt,
+                                                                a.L, a.maxseg, a.ws, a.y, a.ldy, a.state, a.decay, a.seen);
   return 0;
 }
 
 int wz3_occupancy() {
   int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, dev::wz3_gemv_kernel<1>, dev::kWarpsPerCta * 32, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, dev::wz3_gemv_kernel, dev::kWarpsPerCta * 32, 0) !=
       cudaSuccess) {
     cudaGetLastError();
     return 0;

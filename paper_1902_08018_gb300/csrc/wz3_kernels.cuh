@@ -100,9 +100,9 @@ __device__ __forceinline__ void wz3_load_run(const uint8_t* __restrict__ area, u
   }
 }
 
-// A block's products added into the lane's sums: for each r,
-// p_i = s * sum_b V[i][b] xt_r[b] (xt the transformed x of the block's column
-// chunk J, ldt floats per column), then hi/lo[i][r] += p_i by TwoSum.  Rows
+// A block's products added into the lane's sums (one column): p_i = s * sum_b
+// V[i][b] xt[b] (xt the transformed x of the block's column chunk J), then
+// hi/lo[i][0] += p_i by TwoSum.  Rows
 // (0, 1) and (2, 3) go in packed FP32 pairs; each half rounds as the scalar
 // chain (product, three FMAs in b order, the scale, TwoSum) would.
 // wz3_values gives V[h][b] = (value (2h, b), value (2h + 1, b)) and s.
@@ -127,25 +127,21 @@ __device__ __forceinline__ void wz3_values(const uint32_t (&w)[16], int W, float
   s = E ? __uint_as_float((E + K - 27u) << 23) : 0.f;  // 2^(E+K-154); E >= 28 for a nonzero block
 }
 
-template <int R>
-__device__ __forceinline__ void wz3_accumulate(const float2 (&V)[2][4], float s, const float* __restrict__ xt,
-                                               int64_t ldt, int J, float (&hi)[4][R], float (&lo)[4][R]) {
+__device__ __forceinline__ void wz3_accumulate(const float2 (&V)[2][4], float s, const float* __restrict__ xt, int J,
+                                               float (&hi)[4][1], float (&lo)[4][1]) {
   const float2 s2 = make_float2(s, s);
+  const float4 x = __ldg(reinterpret_cast<const float4*>(xt + 4 * J));
+  const float2 x0 = make_float2(x.x, x.x), x1 = make_float2(x.y, x.y), x2 = make_float2(x.z, x.z),
+               x3 = make_float2(x.w, x.w);
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const float4 x = __ldg(reinterpret_cast<const float4*>(xt + (int64_t)r * ldt + 4 * J));
-    const float2 x0 = make_float2(x.x, x.x), x1 = make_float2(x.y, x.y), x2 = make_float2(x.z, x.z),
-                 x3 = make_float2(x.w, x.w);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float2 q = mul_f2(V[h][0], x0);
-      q = fma_f2(V[h][1], x1, q);
-      q = fma_f2(V[h][2], x2, q);
-      q = fma_f2(V[h][3], x3, q);
-      float2 H = make_float2(hi[2 * h][r], hi[2 * h + 1][r]), Lo = make_float2(lo[2 * h][r], lo[2 * h + 1][r]);
-      two_sum_acc2(H, Lo, mul_f2(q, s2));
-      hi[2 * h][r] = H.x, hi[2 * h + 1][r] = H.y, lo[2 * h][r] = Lo.x, lo[2 * h + 1][r] = Lo.y;
-    }
+  for (int h = 0; h < 2; ++h) {
+    float2 q = mul_f2(V[h][0], x0);
+    q = fma_f2(V[h][1], x1, q);
+    q = fma_f2(V[h][2], x2, q);
+    q = fma_f2(V[h][3], x3, q);
+    float2 H = make_float2(hi[2 * h][0], hi[2 * h + 1][0]), Lo = make_float2(lo[2 * h][0], lo[2 * h + 1][0]);
+    two_sum_acc2(H, Lo, mul_f2(q, s2));
+    hi[2 * h][0] = H.x, hi[2 * h + 1][0] = H.y, lo[2 * h][0] = Lo.x, lo[2 * h + 1][0] = Lo.y;
   }
 }
 
@@ -154,12 +150,11 @@ __device__ __forceinline__ void wz3_accumulate(const float2 (&V)[2][4], float s,
 // being band0 + I of the matrix (index points at band0's first entry).  A
 // band whose runs all lie in the range is finished here (y, state); a band
 // shared by several ranges leaves one FP64 partial per range in
-// ws[(I maxseg + seg) R + r][4] for the segment epilogue.  The index entry of
-// the next run is read while the lanes decode the current one.
-template <int R>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
+// ws[I maxseg + seg][4], which its last warp adds up.  The index entry of
+// the next run is read while the lanes decode the current one.  One column.
+static __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
     wz3_gemv_kernel(const uint64_t* __restrict__ index, const uint8_t* __restrict__ area, int64_t M, int64_t BM,
-                    int BN, int RB, const float* __restrict__ xt, int64_t ldt, int64_t L, int maxseg,
+                    int BN, int RB, const float* __restrict__ xt, int64_t L, int maxseg,
                     double* __restrict__ ws, double* __restrict__ y, int64_t ldy, double* __restrict__ state,
                     double decay, unsigned* __restrict__ seen) {
   const int lane = threadIdx.x & 31;
@@ -168,11 +163,9 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
   const int64_t u0 = g * L, u1 = min(total, u0 + L);
   if (u0 >= u1) return;  // warp-uniform; nothing below synchronises across warps
   int64_t I = u0 / RB;  // band of the current piece
-  float hi[4][R], lo[4][R];
+  float hi[4][1], lo[4][1];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int r = 0; r < R; ++r) hi[i][r] = lo[i][r] = 0.f;
+  for (int i = 0; i < 4; ++i) hi[i][0] = lo[i][0] = 0.f;
   uint64_t e_nxt = __ldg(index + u0);  // the same word for every lane
   for (int64_t ub = u0; ub < u1;) {  // the range's piece of band I: runs [ub, ue)
     const int64_t ue = min(u1, (I + 1) * RB);
@@ -189,19 +182,17 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
         float2 V[2][4];
         float s;
         wz3_values(w, W, V, s);
-        wz3_accumulate<R>(V, s, xt, ldt, 32 * q + lane, hi, lo);
+        wz3_accumulate(V, s, xt, 32 * q + lane, hi, lo);
       }
     }
     const int64_t g_lo = div64(I * RB, L), g_hi = div64((I + 1) * RB - 1, L);
     const bool shared = g_lo != g_hi;
-    band_finish<1, R>(hi, lo, lane, 4 * I, M, shared ? ws + (I * maxseg + (g - g_lo)) * R * 4 : nullptr, y, ldy, state,
+    band_finish<1, 1>(hi, lo, lane, 4 * I, M, shared ? ws + (I * maxseg + (g - g_lo)) * 4 : nullptr, y, ldy, state,
                       decay, false);
     if (shared)
-      finish_shared_band(seen, ws, I, M, (int)(g - g_lo), (int)(g_hi - g_lo + 1), maxseg, R, y, ldy, state, decay);
+      finish_shared_band(seen, ws, I, M, (int)(g - g_lo), (int)(g_hi - g_lo + 1), maxseg, 1, y, ldy, state, decay);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int r = 0; r < R; ++r) hi[i][r] = lo[i][r] = 0.f;
+    for (int i = 0; i < 4; ++i) hi[i][0] = lo[i][0] = 0.f;
     ++I;
     ub = ue;
   }
