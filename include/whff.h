@@ -332,7 +332,8 @@ void whff_fields_destroy(whff_fields* f);
  * change the arithmetic; CTAs per SM (the warp ranges) and the fold flags
  * change its rounding within the bar.
  * whff_tune times every candidate on the resident matrix (iters steps each,
- * R = 1, CUDA events on the stream) and keeps the fastest; *best_ms (optional)
+ * R = 1, CUDA events on the stream) and keeps the fastest, of a near tie (0.5 us, or
+ * 1.5 % where that is less) the one with the fewest CTAs per SM; *best_ms (optional)
  * receives its step time.  With tensor-core passes available it then sets
  * the engine crossover: the fewest columns (2..8) for which one tensor-core
  * pass is no slower than the CUDA-core passes, else 9.  whff_get_config / whff_set_config read and apply a

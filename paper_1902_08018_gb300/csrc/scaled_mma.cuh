@@ -13,8 +13,9 @@
 // multiplied by s (the product's rounding error kept exactly with an FMA) and
 // drained into TwoSum FP32 registers.
 //
-// Same persistent pipeline as wz2_mma_kernel: items are (tile of 128 rows,
-// stage of 64 columns), CTA g takes items [g L, g L + L), two stages in
+// This is the register-fed kernel, for host-resident matrices (device-resident ones
+// take scaled_mma_tma_kernel and fp8_mma_kernel).  Persistent: items are (tile of
+// 128 rows, stage of 64 columns), CTA g takes items [g L, g L + L), two stages in
 // flight (A and B tiles of buffer k % 2), the B tiles prebuilt per pass and
 // brought in with cp.async.bulk.  The A tile needs no decode for BF16: a
 // thread moves 16 bytes (8 values of one row) from HBM to one 16-byte row of

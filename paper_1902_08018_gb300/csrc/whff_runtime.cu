@@ -1259,7 +1259,7 @@ extern "C" int whff_set_crossover(whff_handle* h, int min_rhs) {
 }
 
 // Time every (unroll, CTAs per SM, lane fold) candidate on this matrix with
-// R = 1 and keep the fastest.  Uses the handle's own staging buffers (x = 0).
+// R = 1 and keep the fastest (of a near tie, the one with the fewest CTAs).  Uses the handle's own staging buffers (x = 0).
 extern "C" int whff_tune(whff_handle* h, int iters, void* stream, double* best_ms) {
   if (!h || !is_wz2(h) || iters < 1) {
     set_error("whff_tune: WZ2 handles only, iters >= 1");
@@ -1298,9 +1298,10 @@ extern "C" int whff_tune(whff_handle* h, int iters, void* stream, double* best_m
     if (err) break;
     float ms = 0.f;
     cudaEventElapsedTime(&ms, e0, e1);
-    // Within the events' noise of the fastest so far, the shape with fewer CTAs: 0.5 us,
-    // and 1.5 % on short passes.  A share alone gave long passes away: 32768^2 at rate
-    // 16 took a shape of 339 us where another has 335.
+    // Which of two shapes within the events' noise (0.5 us, 1.5 % on short passes) is the
+    // fastest changes from run to run; of those the one with fewer CTAs is kept.  It costs
+    // at most that much, and its CTA count is one that every number of blocks in flight
+    // can be set to (whff_set_config refuses more than fit an SM).
     const double t = ms / iters, tie = std::min(0.015 * fastest, 0.0005);
     const bool take = c < bc ? t < fastest + tie : c > bc ? t < fastest - tie : t < best;
     fastest = std::min(fastest, t);

@@ -1,5 +1,5 @@
 // wz1_decode.cuh -- per-thread decoder of one WZ1 block (zfp-style fixed rate,
-// Sec. 4.3), entirely in registers.
+// Sec. 4.3).
 //
 // Steps: header (nonzero flag, biased exponent) -> embedded plane decode up
 // to the 16*rate-9 bit budget (verbatim prefix bits + group tests, last
