@@ -46,7 +46,14 @@ int raise_smem(int bytes, bool carveout) {
 //   32768^2 (2^26): 277.1 290.4 334.5 410.5 467.6 / 286.7 292.7 332.1 410.0 463.2
 // Rate 8, bound by decode instructions, loses from 20480^2 on; rate 12 at 32768^2;
 // the others gain up to there, the longest measured.
-constexpr int64_t wz2_fuse_blocks(int rate) { return (int64_t)1 << (rate == 8 ? 24 : rate == 12 ? 25 : 26); }
+// An x that the kernel cannot take 16 bytes at a time (N not a multiple of 4, or an
+// unaligned x; the transform's own output always is) is read word by word for every
+// block, which pays only up to 2^22 blocks:
+//   4095^2, rates 8 12 16: 25.7 25.7 25.7 / 18.2 18.5 18.6;  8191^2: 37.5 38.2 40.5 / 35.0 36.7 39.0
+//   12289^2: 59.5 59.6 65.1 / 64.3 65.8 71.5;  16383^2: 89.1 90.8 101.8 / 105.9 107.3 116.5
+constexpr int64_t wz2_fuse_blocks(int rate, bool x_fast) {
+  return (int64_t)1 << (!x_fast ? 22 : rate == 8 ? 24 : rate == 12 ? 25 : 26);
+}
 
 // Blocks up to which the one-column kernels with four or eight blocks in flight add the
 // segments of shared bands themselves.  The fence and the atomics of that make the loop
