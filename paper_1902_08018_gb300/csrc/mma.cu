@@ -8,16 +8,11 @@ namespace whff {
 
 constexpr int kMaxMembers = 64;  // members of one batched tensor-core launch (their table sits in smem)
 
+// Shared memory of the kernel, with room for the largest table if it takes one.
 template <int RATE, bool LIFT, int NR, bool TABLE>
-static int mma_set_smem(int bytes) {
-  auto kern = dev::wz2_mma_kernel<RATE, LIFT, NR, TABLE>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
-      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
-          cudaSuccess) {
-    cudaGetLastError();
-    return -1;
-  }
-  return 0;
+static int mma_set_smem(int device = -1) {
+  return raise_smem<dev::wz2_mma_kernel<RATE, LIFT, NR, TABLE>>(
+      dev::MmaSmem<RATE, NR>::kBytes + (TABLE ? kMaxMembers * (int)sizeof(dev::MmaMember) : 0), true, device);
 }
 
 // CTAs that take `ranges` item ranges, kMmaRanges each.
@@ -30,7 +25,7 @@ template <int RATE, bool LIFT, int NR>
 static int mma_one(const MmaStep& a, cudaStream_t st) {
   using S = dev::MmaSmem<RATE, NR>;
   const int smem = S::kBytes;
-  if (mma_set_smem<RATE, LIFT, NR, false>(smem)) return -1;
+  if (mma_set_smem<RATE, LIFT, NR, false>(a.device)) return -1;
   const int nstages = (int)((a.BN + dev::kMmaStageBlocks - 1) / dev::kMmaStageBlocks);
   const int tiles = (int)((a.BM + dev::kMmaBands - 1) / dev::kMmaBands);
   const dev::MmaMember mem{a.stream, a.btiles, a.ws, a.BM, a.BN, 0, nstages, tiles, a.R, a.maxseg, a.map, a.paired, a.band0};
@@ -61,7 +56,7 @@ template <int RATE, bool LIFT, int NR>
 static int mma_batch_one(const MmaBatchStep& a, cudaStream_t st) {
   using S = dev::MmaSmem<RATE, NR>;
   const int smem = S::kBytes + a.nmem * (int)sizeof(dev::MmaMember);
-  if (mma_set_smem<RATE, LIFT, NR, true>(smem)) return -1;
+  if (mma_set_smem<RATE, LIFT, NR, true>(a.device)) return -1;
   const dev::MmaMember m0{};
   const dev::MmaPass p0{};
   dev::wz2_mma_btiles<LIFT, NR><<<(unsigned)((a.bt_threads + 255) / 256), 256, 0, st>>>(p0, a.passes, a.nmem,
@@ -110,9 +105,8 @@ int mma_launch(const MmaStep& a, cudaStream_t st) {
 // CTA takes them one after another.
 template <int RATE, bool LIFT, int NR>
 static int mma_occ_one() {
-  using S = dev::MmaSmem<RATE, NR>;
   cudaFuncAttributes fa;
-  if (mma_set_smem<RATE, LIFT, NR, true>(S::kBytes + kMaxMembers * (int)sizeof(dev::MmaMember)) ||
+  if (mma_set_smem<RATE, LIFT, NR, true>() ||
       cudaFuncGetAttributes(&fa, dev::wz2_mma_kernel<RATE, LIFT, NR, true>) != cudaSuccess ||
       fa.maxThreadsPerBlock < dev::kMmaDecodeThreads) {
     cudaGetLastError();

@@ -17,9 +17,9 @@ static int scaled_mma_one(const ScaledMmaStep& a, cudaStream_t st) {
   constexpr bool kF16 = FMT == 3;
   const bool tma = (FMT == 2 || FMT == 3) && a.tmap != nullptr;
   const bool fp8 = FMT == 4 && a.tmap != nullptr;
-  if (fp8   ? raise_smem<dev::fp8_mma_kernel<NR>>(dev::Fp8Smem<NR>::kBytes, false)
-      : tma ? raise_smem<dev::scaled_mma_tma_kernel<NR, kF16>>(dev::TmaSmem<NR>::kBytes, true)
-            : raise_smem<dev::scaled_mma_kernel<FMT, NR>>(S::kBytes, true))
+  if (fp8   ? raise_smem<dev::fp8_mma_kernel<NR>>(dev::Fp8Smem<NR>::kBytes, false, a.device)
+      : tma ? raise_smem<dev::scaled_mma_tma_kernel<NR, kF16>>(dev::TmaSmem<NR>::kBytes, true, a.device)
+            : raise_smem<dev::scaled_mma_kernel<FMT, NR>>(S::kBytes, true, a.device))
     return -1;
   const int nstages = (int)((a.N + 63) / 64);
   const int tiles = (int)((a.M + 127) / 128);

@@ -15,8 +15,8 @@ static void wz2_launch_one(const Wz2Step& a, cudaStream_t st) {
 }
 
 template <int RATE, bool LIFT>
-static int wz2_stream_smem_attr() {
-  return raise_smem<dev::wz2_stream_kernel<RATE, LIFT>>(dev::Wz2Stream<RATE>::kSmemBytes, false);
+static int wz2_stream_smem_attr(int device = -1) {
+  return raise_smem<dev::wz2_stream_kernel<RATE, LIFT>>(dev::Wz2Stream<RATE>::kSmemBytes, false, device);
 }
 
 static inline void wz2_launch_epilogue(const Wz2Step& a, cudaStream_t st) {
@@ -39,7 +39,7 @@ static void wz2_launch_deep(const Wz2Step& a, cudaStream_t st) {
 template <int RATE, bool LIFT>
 static int wz2_launch_lift(const Wz2Step& a, cudaStream_t st) {
   if (a.staged && a.R == 1 && !a.groups8) {
-    if (wz2_stream_smem_attr<RATE, LIFT>()) return -1;
+    if (wz2_stream_smem_attr<RATE, LIFT>(a.device)) return -1;
     dev::wz2_stream_kernel<RATE, LIFT><<<(unsigned)a.ctas, dev::kWarpsPerCta * 32, dev::Wz2Stream<RATE>::kSmemBytes,
                                          st>>>(a.stream, a.M, a.N, a.BM, a.BN, a.x, a.ldx, a.x_vec_ok, a.L, a.maxseg,
                                                a.ws, a.y, a.ldy, a.state, a.decay, a.red32, a.status);

@@ -16,17 +16,16 @@ constexpr uint32_t kWaitPolls = 1u << 22;
 
 // Raise the dynamic shared-memory limit of a kernel.  The limit belongs to the kernel on
 // one device, and a process may use several; it is set on a device's first launch (the
-// two calls cost 1 to 2 us, which a small pass would see).  carveout: ask for all of the
-// SM's memory as shared memory, too.
+// two calls cost 1 to 2 us, which a small pass would see).  device: the current one, -1 asks.
+// carveout: ask for all of the SM's memory as shared memory, too.
 template <auto Kern>
-int raise_smem(int bytes, bool carveout) {
+int raise_smem(int bytes, bool carveout, int device = -1) {
   static std::atomic<uint64_t> done{0};  // a bit per device; devices from 64 on always set it
-  int d = -1;
-  if (cudaGetDevice(&d) != cudaSuccess) {
+  if (device < 0 && cudaGetDevice(&device) != cudaSuccess) {
     cudaGetLastError();
     return -1;
   }
-  const uint64_t bit = d < 64 ? 1ull << d : 0;
+  const uint64_t bit = device < 64 ? 1ull << device : 0;
   if (done.load(std::memory_order_acquire) & bit) return 0;
   if (cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
       (carveout && cudaFuncSetAttribute(Kern, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -89,6 +88,7 @@ struct Wz2Step {
   bool staged;     // R = 1: stream each warp's range through shared memory by bulk copies
   int* status;     // device status word (bounded waits of the staged kernel)
   unsigned* seen;  // per band: counts the segments of the pass (see finish_shared_band)
+  int device;      // the current one, where the handle lives
 };
 
 // Bytes a handle's device stream allocation carries past the stream, so that
@@ -161,6 +161,7 @@ struct MmaStep {
   const void* map; // CUtensorMap in device memory of the whole stored matrix, or null
   int paired;      // two maps, 128 bytes apart: the even and the odd bands
   int64_t band0;   // first band of this pass in it (row views)
+  int device;      // the current one, where the handle lives
 };
 int mma_launch(const MmaStep& a, cudaStream_t st);
 
@@ -178,6 +179,7 @@ struct MmaBatchStep {
   int64_t bt_threads, fin_threads;
   int* status;
   uint32_t spin;
+  int device;        // the current one, where the handles live
 };
 int mma_batch_launch(const MmaBatchStep& a, cudaStream_t st);
 int mma_max_members();  // most members of one batched launch
@@ -209,6 +211,7 @@ struct ScaledMmaStep {
   const void* tmap;  // CUtensorMap of the whole stored matrix (A tiles by TMA), or null
   int64_t row0;      // first row of this pass within that matrix (row views)
   int* colexp;       // FP16 with tmap: 32 ints of scratch for the per-column exponents of x
+  int device;        // the current one, where the handle lives
 };
 int scaled_mma_launch(const ScaledMmaStep& a, cudaStream_t st);
 // Host: encode the TMA map of a WZ2 stream (BM bands of BN blocks, box one stage:

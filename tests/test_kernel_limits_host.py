@@ -50,19 +50,19 @@ int main() {
         for (const void* tmap : {(const void*)map, (const void*)nullptr}) {
           whff::ScaledMmaStep a{};
           a.fmt = fmt, a.M = 256, a.N = 256, a.ld = 256, a.TN = 2, a.ldx = 256, a.R = R, a.L = 1, a.ctas = 8, a.maxseg = 4;
-          a.ldy = 256, a.spin = 1, a.tmap = tmap;
+          a.ldy = 256, a.spin = 1, a.tmap = tmap, a.device = device;
           if (whff::scaled_mma_launch(a, nullptr)) return 2;
         }
     for (int rate = 8; rate <= 24; rate += 4)
       for (int R : {8, 32}) {
         whff::MmaStep a{};
         a.rate = rate, a.lift = true, a.M = 256, a.N = 256, a.BM = 64, a.BN = 64, a.ldx = 256, a.R = R, a.L = 1, a.ctas = 8;
-        a.maxseg = 4, a.ldy = 256, a.spin = 1, a.map = map;
+        a.maxseg = 4, a.ldy = 256, a.spin = 1, a.map = map, a.device = device;
         if (whff::mma_launch(a, nullptr)) return 3;
       }
     whff::Wz2Step b{};  // the bulk-staged pass
     b.M = 256, b.N = 256, b.BM = 64, b.BN = 64, b.ldx = 256, b.L = 4096, b.maxseg = 1, b.ldy = 256, b.ctas = 1, b.unroll = 2;
-    b.lift = true, b.R = 1, b.staged = true;
+    b.lift = true, b.R = 1, b.staged = true, b.device = device;
     if (whff::wz2_launch<8>(b, nullptr) || whff::wz2_launch<16>(b, nullptr) || whff::wz2_launch<24>(b, nullptr)) return 6;
   }
   std::printf("%d launches, %d large, %d refused\n", g_launches, g_large, g_refused);
