@@ -15,12 +15,6 @@ static int mma_set_smem(int device = -1) {
       dev::MmaSmem<RATE, NR>::kBytes + (TABLE ? kMaxMembers * (int)sizeof(dev::MmaMember) : 0), true, device);
 }
 
-// CTAs that take `ranges` item ranges, kMmaRanges each.
-template <int RATE>
-static unsigned mma_grid(int ranges) {
-  return (unsigned)((ranges + dev::kMmaRanges<RATE> - 1) / dev::kMmaRanges<RATE>);
-}
-
 template <int RATE, bool LIFT, int NR>
 static int mma_one(const MmaStep& a, cudaStream_t st) {
   using S = dev::MmaSmem<RATE, NR>;
@@ -32,8 +26,9 @@ static int mma_one(const MmaStep& a, cudaStream_t st) {
   const dev::MmaPass pass{a.x, a.y, a.btiles, a.ws, a.ldx, a.ldy, a.N, a.M, 0, 0, 0, nstages, tiles, a.R, a.maxseg};
   const int64_t bthreads = (int64_t)nstages * dev::kMmaStageBlocks * NR;
   dev::wz2_mma_btiles<LIFT, NR><<<(unsigned)((bthreads + 255) / 256), 256, 0, st>>>(pass, nullptr, 1, bthreads);
-  dev::wz2_mma_kernel<RATE, LIFT, NR, false><<<mma_grid<RATE>(a.ctas), dev::kMmaDecodeThreads, smem, st>>>(
-      mem, nullptr, 1, (int64_t)tiles * nstages, a.L, a.status, a.spin);
+  const int per = dev::mma_ranges_per_cta(a.ctas, a.sms, dev::kMmaRanges<RATE>);
+  dev::wz2_mma_kernel<RATE, LIFT, NR, false><<<(unsigned)((a.ctas + per - 1) / per), dev::kMmaDecodeThreads, smem, st>>>(
+      mem, nullptr, 1, (int64_t)tiles * nstages, a.L, per, a.status, a.spin);
   const int64_t fin_threads = (int64_t)tiles * a.R * 32;
   dev::wz2_mma_finish<LIFT><<<(unsigned)((fin_threads + 255) / 256), 256, 0, st>>>(pass, nullptr, 1, fin_threads,
                                                                                   a.L);
@@ -61,9 +56,9 @@ static int mma_batch_one(const MmaBatchStep& a, cudaStream_t st) {
   const dev::MmaPass p0{};
   dev::wz2_mma_btiles<LIFT, NR><<<(unsigned)((a.bt_threads + 255) / 256), 256, 0, st>>>(p0, a.passes, a.nmem,
                                                                                        a.bt_threads);
-  dev::wz2_mma_kernel<RATE, LIFT, NR, true><<<mma_grid<RATE>(a.ctas), dev::kMmaDecodeThreads, smem, st>>>(m0, a.members, a.nmem,
-                                                                                            a.total, a.L, a.status,
-                                                                                            a.spin);
+  const int per = dev::mma_ranges_per_cta(a.ctas, a.sms, dev::kMmaRanges<RATE>);
+  dev::wz2_mma_kernel<RATE, LIFT, NR, true><<<(unsigned)((a.ctas + per - 1) / per), dev::kMmaDecodeThreads, smem, st>>>(
+      m0, a.members, a.nmem, a.total, a.L, per, a.status, a.spin);
   dev::wz2_mma_finish<LIFT><<<(unsigned)((a.fin_threads + 255) / 256), 256, 0, st>>>(p0, a.passes, a.nmem,
                                                                                     a.fin_threads, a.L);
   return 0;

@@ -141,11 +141,15 @@ struct MmaSmem {
   static constexpr int kBytes = kBars + 256;
 };
 
-// Ranges that a CTA of wz2_mma_kernel takes one after another.  The ranges, and
-// the accumulator groups that end with them, are those of a grid of two CTAs per
+// Ranges that a CTA of wz2_mma_kernel takes one after another, at most.  The ranges,
+// and the accumulator groups that end with them, are those of a grid of two CTAs per
 // SM (one where A takes three pieces).
 template <int RATE>
 constexpr int kMmaRanges = MmaPieces<RATE>::kA == 3 ? 1 : 2;
+
+// Ranges per CTA of a pass of `ranges`: one while there is an SM for each (512^2 in
+// FP8, 32 columns, replayed: 16.4 us with two, 14.4 with one).
+inline int mma_ranges_per_cta(int ranges, int sms, int most) { return ranges <= sms ? 1 : most; }
 
 // Eight columns of the three accumulators at ta, ta + stride, ta + 2 stride,
 // summed big + (small + smaller): one wait for the three loads, tied to their
@@ -332,7 +336,7 @@ __device__ __forceinline__ void tmem_store_16x256(uint32_t taddr, uint32_t r0, u
 // Persistent grid over the item sequence of one or more passes (members):
 // member k owns items [item_begin, item_begin + tiles S), item = item_begin +
 // tile S + stage; range v is items [v L, v L + L), and CTA g takes the
-// kMmaRanges ranges from kMmaRanges g on.  ws[((tile * maxseg + seg) * R + r) *
+// per_cta ranges from per_cta g on.  ws[((tile * maxseg + seg) * R + r) *
 // 128 + m] of a member receives the FP64 partial of coefficient row a of band b
 // of the tile, m = 32a + b, for the range's segment seg = v - (item_begin + tile
 // S) / L.  Accumulator groups end with a range, so a result does not depend on
@@ -342,7 +346,7 @@ __device__ __forceinline__ void tmem_store_16x256(uint32_t taddr, uint32_t r0, u
 template <int RATE, bool LIFT, int NR, bool TABLE>
 __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
     wz2_mma_kernel(MmaMember single, const MmaMember* __restrict__ table, int nmem, int64_t total, int64_t L,
-                   int* __restrict__ status, uint32_t spin) {
+                   int per_cta, int* __restrict__ status, uint32_t spin) {
   using SM = MmaSmem<RATE, NR>;
   constexpr int PA = MmaPieces<RATE>::kA, NB = SM::kNB, NA = SM::kNA, NQ = kMmaQuartets;
   constexpr int NW = Wz2Layout<RATE>::kWords;
@@ -362,8 +366,8 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
 
   // broadcast, so that the compiler knows the roles to be warp-uniform
   const int t = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, t >> 5, 0), lane = t & 31;
-  const int64_t it0 = (int64_t)blockIdx.x * kMmaRanges<RATE> * L;
-  const int n = (int)max((int64_t)0, min(total, it0 + kMmaRanges<RATE> * L) - it0);  // stages of this CTA
+  const int64_t it0 = (int64_t)blockIdx.x * per_cta * L;
+  const int n = (int)max((int64_t)0, min(total, it0 + per_cta * L) - it0);  // stages of this CTA
   const int len = (int)L;
   if constexpr (TABLE)
     for (int i = t; i < nmem; i += kMmaDecodeThreads) tab[i] = table[i];
@@ -500,7 +504,7 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
 #pragma unroll
     for (int r = 0; r < HALF; ++r) hi[r] = lo[r] = 0.f;
     int cur_m = c_m, cur_tile = c_tile;  // member and tile of the sums
-    int v = (int)blockIdx.x * kMmaRanges<RATE>, left = len;  // the range, and its items from here on
+    int v = (int)blockIdx.x * per_cta, left = len;  // the range, and its items from here on
     auto flush = [&](int range) {
       const MmaMember& me = mb(cur_m);
       const int64_t seg = range - (me.item_begin + (int64_t)cur_tile * me.S) / L;

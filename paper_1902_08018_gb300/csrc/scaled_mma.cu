@@ -33,10 +33,10 @@ static int scaled_mma_one(const ScaledMmaStep& a, cudaStream_t st) {
     dev::wz2_mma_btiles<false, NR><<<(unsigned)((bthreads + 255) / 256), 256, 0, st>>>(pass, nullptr, 1, bthreads);
   }
   if (fp8) {
-    dev::fp8_mma_kernel<NR><<<(unsigned)((a.ctas + dev::kFp8Ranges - 1) / dev::kFp8Ranges), dev::kMmaDecodeThreads,
-                              dev::Fp8Smem<NR>::kBytes, st>>>(*static_cast<const CUtensorMap*>(a.tmap), a.row0, a.scales,
-                                                              a.TN, a.btiles, a.ws, nstages, a.R, a.maxseg,
-                                                              (int64_t)tiles * nstages, a.L, a.status, a.spin);
+    const int per = dev::mma_ranges_per_cta(a.ctas, a.sms, dev::kFp8Ranges);
+    dev::fp8_mma_kernel<NR><<<(unsigned)((a.ctas + per - 1) / per), dev::kMmaDecodeThreads, dev::Fp8Smem<NR>::kBytes, st>>>(
+        *static_cast<const CUtensorMap*>(a.tmap), a.row0, a.scales, a.TN, a.btiles, a.ws, nstages, a.R, a.maxseg,
+        (int64_t)tiles * nstages, a.L, per, a.status, a.spin);
   } else if (tma) {
     dev::scaled_mma_tma_kernel<NR, kF16><<<(unsigned)a.ctas, dev::kTmaThreads, dev::TmaSmem<NR>::kBytes, st>>>(
         *static_cast<const CUtensorMap*>(a.tmap), a.row0, a.scales, a.TN, a.btiles, a.ws, nstages, a.R, a.maxseg,

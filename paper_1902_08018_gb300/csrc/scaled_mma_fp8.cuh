@@ -17,7 +17,7 @@
 namespace whff {
 namespace dev {
 
-// Item ranges of a CTA: those of a grid of two CTAs per SM (see kMmaRanges).
+// Item ranges of a CTA at most: those of a grid of two CTAs per SM (see kMmaRanges).
 constexpr int kFp8Ranges = 2;
 
 template <int NR>
@@ -41,7 +41,7 @@ template <int NR>
 __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
     fp8_mma_kernel(const __grid_constant__ CUtensorMap tmap, int64_t row0, const float* __restrict__ scales, int64_t TN,
                    const uint8_t* __restrict__ btiles, double* __restrict__ ws, int S, int R, int maxseg, int64_t total,
-                   int64_t L, int* __restrict__ status, uint32_t spin) {
+                   int64_t L, int per_cta, int* __restrict__ status, uint32_t spin) {
   using SM = Fp8Smem<NR>;
   constexpr int NB = SM::kNB, NA = SM::kNA, NQ = kMmaQuartets;
   constexpr int HALF = NR / 2;  // columns drained by each of the two warps on a lane quarter
@@ -59,8 +59,8 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
 
   // broadcast, so that the compiler knows the roles to be warp-uniform
   const int t = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, t >> 5, 0), lane = t & 31;
-  const int64_t it0 = (int64_t)blockIdx.x * kFp8Ranges * L;
-  const int n = (int)max((int64_t)0, min(total, it0 + kFp8Ranges * L) - it0);  // stages of this CTA
+  const int64_t it0 = (int64_t)blockIdx.x * per_cta * L;
+  const int n = (int)max((int64_t)0, min(total, it0 + per_cta * L) - it0);  // stages of this CTA
   const int len = (int)L;
   if (t == 0) {
     for (int i = 0; i < NB; ++i)
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(kMmaDecodeThreads, 1)
 #pragma unroll
     for (int r = 0; r < HALF; ++r) hi[r] = lo[r] = 0.f;
     int cur_tile = c_tile;  // tile of the sums
-    int v = (int)blockIdx.x * kFp8Ranges, left = len;  // the range, and its items from here on
+    int v = (int)blockIdx.x * per_cta, left = len;  // the range, and its items from here on
     auto flush = [&](int range) {
       const int64_t seg = range - ((int64_t)cur_tile * S) / L;
       double* dst = ws + (((int64_t)cur_tile * maxseg + seg) * R) * 128 + 32 * quarter + lane;

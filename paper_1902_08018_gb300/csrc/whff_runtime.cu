@@ -633,14 +633,14 @@ int launch_mma(const whff_handle* h, const float* x, int R, int64_t ldx, double*
   if (is_blocked(h->info.fmt)) {
     MmaStep a{h->info.rate, h->info.fmt == WHFF_FMT_FIXED_LIFT, h->d_stream, h->info.M, h->info.N, h->BM, h->BN,
               x, ldx, R, h->mma_L, h->mma_ctas, h->mma_maxseg, h->d_ws_mma, h->d_btiles, y, ldy, state, decay,
-              h->d_status, h->wait_polls, h->d_map, h->map_count == 2, h->band0, h->device};
+              h->d_status, h->wait_polls, h->d_map, h->map_count == 2, h->band0, h->device, h->sm_count};
     e = mma_launch(a, st);
   } else {
     ScaledMmaStep a{h->info.fmt, h->d_stream, h->d_scales, h->info.M, h->info.N, scaled_ld(h->info.N),
                     ceil_div(h->info.N, kScaleTile), x, ldx, R, h->mma_L, h->mma_ctas, h->mma_maxseg,
                     h->d_ws_mma, h->d_btiles, y, ldy, state, decay, h->d_status, h->wait_polls,
                     h->has_tmap ? h->tmap : nullptr, h->tma_row0,
-                    reinterpret_cast<int*>(h->d_btiles + h->btile_bytes), h->device};
+                    reinterpret_cast<int*>(h->d_btiles + h->btile_bytes), h->device, h->sm_count};
     e = scaled_mma_launch(a, st);
   }
   if (e) {
@@ -1692,7 +1692,7 @@ extern "C" int whff_batch_step(whff_batch* b, const float* const* x, const int64
     WHFF_CUDA_TRY(cudaMemcpyAsync(g.d_passes, g.pinned, sizeof(dev::MmaPass) * n, cudaMemcpyHostToDevice, st));
     const whff_handle* h0 = b->hs[g.of[0]];
     MmaBatchStep a{b->rate, b->lift, g.nr, g.d_members, g.d_passes, n, g.total, g.L, g.ctas, g.bt_threads,
-                   g.fin_threads, h0->d_status, h0->wait_polls, h0->device};
+                   g.fin_threads, h0->d_status, h0->wait_polls, h0->device, h0->sm_count};
     if (mma_batch_launch(a, st)) {
       set_error("whff_batch_step: tensor-core launch failed");
       return WHFF_ECUDA;

@@ -162,6 +162,7 @@ struct MmaStep {
   int paired;      // two maps, 128 bytes apart: the even and the odd bands
   int64_t band0;   // first band of this pass in it (row views)
   int device;      // the current one, where the handle lives
+  int sms;         // its SMs
 };
 int mma_launch(const MmaStep& a, cudaStream_t st);
 
@@ -180,6 +181,7 @@ struct MmaBatchStep {
   int* status;
   uint32_t spin;
   int device;        // the current one, where the handles live
+  int sms;         // its SMs
 };
 int mma_batch_launch(const MmaBatchStep& a, cudaStream_t st);
 int mma_max_members();  // most members of one batched launch
@@ -212,6 +214,7 @@ struct ScaledMmaStep {
   int64_t row0;      // first row of this pass within that matrix (row views)
   int* colexp;       // FP16 with tmap: 32 ints of scratch for the per-column exponents of x
   int device;        // the current one, where the handle lives
+  int sms;         // its SMs
 };
 int scaled_mma_launch(const ScaledMmaStep& a, cudaStream_t st);
 // Host: encode the TMA map of a WZ2 stream (BM bands of BN blocks, box one stage:
