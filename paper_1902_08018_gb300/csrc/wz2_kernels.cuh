@@ -444,34 +444,44 @@ __device__ __forceinline__ void sum_segments(const double* __restrict__ ws, int6
 // none can leave anything to the next one, even if two of them overlapped; a counter that
 // the last warp sets back is off for good after that.
 constexpr unsigned kSeenPeriod = 1u << 20;
+__device__ __forceinline__ bool count_segment(unsigned* __restrict__ seen, int64_t I, int seg, int nseg) {
+  const unsigned add = seg == 0 ? kSeenPeriod - (unsigned)(nseg - 1) : 1u;
+  return (atomicAdd(seen + I, add) + add) % kSeenPeriod == 0;
+}
+
 __device__ __forceinline__ void finish_shared_band(unsigned* __restrict__ seen, const double* __restrict__ ws, int64_t I,
                                                    int64_t M, int seg, int nseg, int maxseg, int R, double* __restrict__ y,
                                                    int64_t ldy, double* __restrict__ state, double decay) {
   __threadfence();
   __syncwarp();
   int last = 0;
-  if ((threadIdx.x & 31) == 0) {
-    const unsigned add = seg == 0 ? kSeenPeriod - (unsigned)(nseg - 1) : 1u;
-    last = (atomicAdd(seen + I, add) + add) % kSeenPeriod == 0;
-  }
+  if ((threadIdx.x & 31) == 0) last = count_segment(seen, I, seg, nseg);
   last = __shfl_sync(0xffffffffu, last, 0);
   if (!last) return;
   __threadfence();
   sum_segments(ws, I, M, nseg, maxseg, R, y, ldy, state, decay, true);
 }
 
-// The same for the four lane groups of a warp, each with a piece of a band of its own.
+// The same for the lane groups of a warp, each with a piece of a band of its own: they
+// count side by side.
 template <int GL>
 __device__ __forceinline__ void finish_shared_groups(unsigned* __restrict__ seen, const double* __restrict__ ws, int64_t I,
                                                      int64_t M, int seg, int nseg, bool shared, int maxseg, int R,
                                                      double* __restrict__ y, int64_t ldy, double* __restrict__ state,
                                                      double decay) {
   if (!__any_sync(0xffffffffu, shared)) return;
+  __threadfence();
+  __syncwarp();
+  bool last = false;
+  if (shared && threadIdx.x % GL == 0) last = count_segment(seen, I, seg, nseg);
+  unsigned done = __ballot_sync(0xffffffffu, last);  // the groups whose band is complete
+  if (!done) return;
+  __threadfence();
 #pragma unroll 1
-  for (int g = 0; g < 32; g += GL) {
-    if (!__shfl_sync(0xffffffffu, (int)shared, g)) continue;
-    finish_shared_band(seen, ws, __shfl_sync(0xffffffffu, I, g), M, __shfl_sync(0xffffffffu, seg, g),
-                       __shfl_sync(0xffffffffu, nseg, g), maxseg, R, y, ldy, state, decay);
+  for (; done; done &= done - 1) {
+    const int g = __ffs((int)done) - 1;
+    sum_segments(ws, __shfl_sync(0xffffffffu, I, g), M, __shfl_sync(0xffffffffu, nseg, g), maxseg, R, y, ldy, state,
+                 decay, true);
   }
 }
 
