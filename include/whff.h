@@ -188,7 +188,8 @@ int whff_info(const whff_handle* h, int* fmt, int* rate, int64_t* M, int64_t* N,
  * eight blocks in flight) if any, and the (2G)^T x transform of x
  * where the fused kernel reads it: FIXED_ACC, and FIXED_LIFT unless the kernel
  * transforms x itself (two blocks in flight, up to 2^24 blocks at rate 8, 2^25 at 12, else 2^26;
- * 2^22 with an N that is not a multiple of 4, or an x off 16 bytes, which is not counted here). */
+ * 2^22, with lane groups 2^19, with an N that is not a multiple of 4 or an x off 16 bytes;
+ * the latter is not counted here). */
 int whff_plan(const whff_handle* h, int* ksplit, int* launches);
 
 /* One control step (Sec. 2.1 / Sec. 4.4): y[:,r] = Ahat * x[:,r] for r < R,

@@ -661,7 +661,7 @@ extern "C" int whff_plan(const whff_handle* h, int* ksplit, int* launches) {
   if (ksplit) *ksplit = h->ksplit;
   if (launches)
     *launches = (h->ksplit > 1 || (h->maxseg > 1 && (h->bulk || h->BM * h->BN > wz2_finish_blocks(h->unroll))) ? 2 : 1) +
-                ((h->info.fmt == WHFF_FMT_FIXED_LIFT && (h->BM * h->BN > wz2_fuse_blocks(h->info.rate, h->info.N % 4 == 0) || h->bulk ||
+                ((h->info.fmt == WHFF_FMT_FIXED_LIFT && (h->BM * h->BN > wz2_fuse_blocks(h->info.rate, h->info.N % 4 == 0, h->groups8) || h->bulk ||
                                                          (h->unroll != 2 && !h->groups8))) ||
                          is_wz3(h->info.fmt)
                      ? 1

@@ -72,7 +72,7 @@ int wz2_launch(const Wz2Step& a, cudaStream_t st) {
   // One column of a small matrix: the kernel transforms x block by block, which
   // costs less than a launch of its own (see wz2_fuse_blocks); the same operations,
   // so the same bits.
-  if (a.R == 1 && !a.staged && (a.groups8 || a.unroll == 2) && a.BM * a.BN <= wz2_fuse_blocks(RATE, a.x_vec_ok && a.N % 4 == 0)) {
+  if (a.R == 1 && !a.staged && (a.groups8 || a.unroll == 2) && a.BM * a.BN <= wz2_fuse_blocks(RATE, a.x_vec_ok && a.N % 4 == 0, a.groups8)) {
     if (a.groups8) wz2_launch_one<RATE, true, 1, 2, 8, false>(a, st);
     else wz2_launch_one<RATE, true, 1, 2, 32, false>(a, st);
     return 0;

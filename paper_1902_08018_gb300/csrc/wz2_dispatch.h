@@ -50,8 +50,11 @@ int raise_smem(int bytes, bool carveout, int device = -1) {
 // block, which pays only up to 2^22 blocks:
 //   4095^2, rates 8 12 16: 25.7 25.7 25.7 / 18.2 18.5 18.6;  8191^2: 37.5 38.2 40.5 / 35.0 36.7 39.0
 //   12289^2: 59.5 59.6 65.1 / 64.3 65.8 71.5;  16383^2: 89.1 90.8 101.8 / 105.9 107.3 116.5
-constexpr int64_t wz2_fuse_blocks(int rate, bool x_fast) {
-  return (int64_t)1 << (!x_fast ? 22 : rate == 8 ? 24 : rate == 12 ? 25 : 26);
+// Lane groups (groups8), whose rows are short, have less to hide such loads behind: up to
+// 2^19 blocks.  Rate 16: 16000 x 378 (380000) 17.4 / 15.5, 32000 x 378 16.2 / 18.7,
+// 64000 x 378 20.3 / 24.0, 20000 x 999 30.4 / 37.6.
+constexpr int64_t wz2_fuse_blocks(int rate, bool x_fast, bool groups8) {
+  return (int64_t)1 << (!x_fast ? (groups8 ? 19 : 22) : rate == 8 ? 24 : rate == 12 ? 25 : 26);
 }
 
 // Blocks up to which the one-column kernels with four or eight blocks in flight add the

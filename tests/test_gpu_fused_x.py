@@ -8,8 +8,11 @@ pytestmark = pytest.mark.gpu
 
 
 # blocks: 2048^2 = 2^22 and one column of blocks more
-@pytest.mark.parametrize("N,launches", [(8192, 1), (8191, 1), (8196, 1), (8195, 2), (8193, 2)])
-def test_route_and_bits(N, launches):
+@pytest.mark.parametrize("M,N,launches", [(8192, 8192, 1), (8192, 8191, 1), (8192, 8196, 1), (8192, 8195, 2),
+                                          (8192, 8193, 2),
+                                          # lane groups: 20971 x 25 blocks (2^19 less 13), 20972 x 25, aligned
+                                          (83884, 99, 1), (83888, 99, 2), (83888, 100, 1)])
+def test_route_and_bits(M, N, launches):
     import ctypes
 
     import torch
@@ -18,7 +21,6 @@ def test_route_and_bits(N, launches):
         pytest.fail("GPU tests need CUDA")
     import paper_1902_08018_gb300 as W
 
-    M = 8192
     A = np.random.default_rng(N).standard_normal((M, N), dtype=np.float32).astype(np.float64)
     buf = torch.from_numpy(np.random.default_rng(M).standard_normal(N + 1).astype(np.float32)).cuda()
     with W.whff_create(W.whff_compress(A, 5, 8), max_rhs=1) as h:
@@ -27,8 +29,8 @@ def test_route_and_bits(N, launches):
         assert n.value == launches
         out = []
         for x in (buf[1:].clone(), buf[1:]):  # aligned, 4 bytes off
-            for unroll in (2, 4):
-                h.set_config(unroll, 1, 0)  # four blocks in flight always take the transform's launch
+            for unroll, fold in ((2, h.config()[2]), (4, 0)) if N > 1000 else ((2, 2),):
+                h.set_config(unroll, 1, fold)  # four blocks in flight always take the transform's launch
                 y = torch.zeros(M, dtype=torch.float64, device="cuda")
                 h.step(x, y)
                 out.append(y)
