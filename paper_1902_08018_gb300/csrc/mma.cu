@@ -8,18 +8,27 @@ namespace whff {
 
 constexpr int kMaxMembers = 64;  // members of one batched tensor-core launch (their table sits in smem)
 
-// Shared memory of the kernel, with room for the largest table if it takes one.
-template <int RATE, bool LIFT, int NR, bool TABLE>
-static int mma_set_smem(int device = -1) {
-  return raise_smem<dev::wz2_mma_kernel<RATE, LIFT, NR, TABLE>>(
-      dev::MmaSmem<RATE, NR>::kBytes + (TABLE ? kMaxMembers * (int)sizeof(dev::MmaMember) : 0), true, device);
+// Shared memory of a batch's kernel, which grows with its table: set for every launch.
+// (Raised once for the largest table, the calls saved had a batch of ten matrices of 1024
+// to 8192 take 200 us a pass among others instead of 192: the pace of the submissions
+// matters there, a pause of the host in their place gave 192 as well.)
+template <int RATE, bool LIFT, int NR>
+static int mma_set_batch_smem(int bytes) {
+  auto kern = dev::wz2_mma_kernel<RATE, LIFT, NR, true>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
+      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
+          cudaSuccess) {
+    cudaGetLastError();
+    return -1;
+  }
+  return 0;
 }
 
 template <int RATE, bool LIFT, int NR>
 static int mma_one(const MmaStep& a, cudaStream_t st) {
   using S = dev::MmaSmem<RATE, NR>;
   const int smem = S::kBytes;
-  if (mma_set_smem<RATE, LIFT, NR, false>(a.device)) return -1;
+  if (raise_smem<dev::wz2_mma_kernel<RATE, LIFT, NR, false>>(smem, true, a.device)) return -1;
   const int nstages = (int)((a.BN + dev::kMmaStageBlocks - 1) / dev::kMmaStageBlocks);
   const int tiles = (int)((a.BM + dev::kMmaBands - 1) / dev::kMmaBands);
   const dev::MmaMember mem{a.stream, a.btiles, a.ws, a.BM, a.BN, 0, nstages, tiles, a.R, a.maxseg, a.map, a.paired, a.band0};
@@ -51,7 +60,7 @@ template <int RATE, bool LIFT, int NR>
 static int mma_batch_one(const MmaBatchStep& a, cudaStream_t st) {
   using S = dev::MmaSmem<RATE, NR>;
   const int smem = S::kBytes + a.nmem * (int)sizeof(dev::MmaMember);
-  if (mma_set_smem<RATE, LIFT, NR, true>(a.device)) return -1;
+  if (mma_set_batch_smem<RATE, LIFT, NR>(smem)) return -1;
   const dev::MmaMember m0{};
   const dev::MmaPass p0{};
   dev::wz2_mma_btiles<LIFT, NR><<<(unsigned)((a.bt_threads + 255) / 256), 256, 0, st>>>(p0, a.passes, a.nmem,
@@ -101,7 +110,7 @@ int mma_launch(const MmaStep& a, cudaStream_t st) {
 template <int RATE, bool LIFT, int NR>
 static int mma_occ_one() {
   cudaFuncAttributes fa;
-  if (mma_set_smem<RATE, LIFT, NR, true>() ||
+  if (mma_set_batch_smem<RATE, LIFT, NR>(dev::MmaSmem<RATE, NR>::kBytes + kMaxMembers * (int)sizeof(dev::MmaMember)) ||
       cudaFuncGetAttributes(&fa, dev::wz2_mma_kernel<RATE, LIFT, NR, true>) != cudaSuccess ||
       fa.maxThreadsPerBlock < dev::kMmaDecodeThreads) {
     cudaGetLastError();

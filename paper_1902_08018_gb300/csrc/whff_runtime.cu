@@ -1692,7 +1692,7 @@ extern "C" int whff_batch_step(whff_batch* b, const float* const* x, const int64
     WHFF_CUDA_TRY(cudaMemcpyAsync(g.d_passes, g.pinned, sizeof(dev::MmaPass) * n, cudaMemcpyHostToDevice, st));
     const whff_handle* h0 = b->hs[g.of[0]];
     MmaBatchStep a{b->rate, b->lift, g.nr, g.d_members, g.d_passes, n, g.total, g.L, g.ctas, g.bt_threads,
-                   g.fin_threads, h0->d_status, h0->wait_polls, h0->device, h0->sm_count};
+                   g.fin_threads, h0->d_status, h0->wait_polls, h0->sm_count};
     if (mma_batch_launch(a, st)) {
       set_error("whff_batch_step: tensor-core launch failed");
       return WHFF_ECUDA;

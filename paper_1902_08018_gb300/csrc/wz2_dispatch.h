@@ -183,8 +183,7 @@ struct MmaBatchStep {
   int64_t bt_threads, fin_threads;
   int* status;
   uint32_t spin;
-  int device;        // the current one, where the handles live
-  int sms;         // its SMs
+  int sms;           // SMs of the device
 };
 int mma_batch_launch(const MmaBatchStep& a, cudaStream_t st);
 int mma_max_members();  // most members of one batched launch
