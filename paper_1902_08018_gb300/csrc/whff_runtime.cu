@@ -1658,6 +1658,14 @@ extern "C" int whff_batch_create(whff_handle* const* hs, const int* R, int count
     set_error("whff_batch_create: pinned staging allocation failed");
     return WHFF_ENOMEM;
   }
+  // the tables went up from pageable memory, whose copies may still be on their way: a
+  // step on a non-blocking stream is not ordered behind them
+  if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+    cudaGetLastError();
+    whff_batch_destroy(b);
+    set_error("whff_batch_create: table upload failed");
+    return WHFF_ECUDA;
+  }
   *out = b;
   return WHFF_OK;
 }

@@ -40,3 +40,37 @@ def test_create_beside_a_busy_legacy_stream(orc, fmt, rate):
     h.destroy()
     for r in range(R):
         assert np.linalg.norm(got[r] - ref[r]) <= 1e-6 * np.linalg.norm(ref[r])
+
+
+def test_batches_step_at_once_on_a_stream_of_their_own(orc):
+    """The batch's tables are on the device when whff_batch_create returns: its first step
+    may run on a non-blocking stream (shown by reading; a copy still under way is a race)."""
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need CUDA")
+    import paper_1902_08018_gb300 as W
+
+    side = torch.cuda.Stream()
+    work = []
+    for k, (M, N, R) in enumerate([(256, 260, 16), (132, 516, 1), (300, 128, 5)]):
+        rng = np.random.default_rng(k)
+        blob = W.whff_compress(rng.standard_normal((M, N)), 5, 12)
+        X = rng.standard_normal((R, N)).astype(np.float32)
+        work.append((W.whff_create(blob, max_rhs=16, stream=side), torch.from_numpy(X).cuda(),
+                     torch.zeros((R, M), dtype=torch.float64, device="cuda"),
+                     X.astype(np.float64) @ orc.decode(blob.tobytes()).T))
+    torch.cuda.synchronize()
+    for _ in range(4):
+        for w in work:
+            w[2].zero_()
+        torch.cuda.synchronize()
+        with W.Batch([w[0] for w in work], [w[1].shape[0] for w in work]) as b:
+            b.step([w[1] for w in work], [w[2] for w in work], None, stream=side)
+            side.synchronize()
+        for w in work:
+            got = w[2].cpu().numpy()
+            for r in range(len(got)):
+                assert np.linalg.norm(got[r] - w[3][r]) <= 1e-6 * np.linalg.norm(w[3][r])
+    for w in work:
+        w[0].destroy()
