@@ -147,7 +147,7 @@ __device__ __forceinline__ void scaled_piece(const uint8_t* __restrict__ payload
 
 // CTAs per SM that the kernels are held to: the occupancy that the one-column plans
 // count on, and two for the few columns that fit 128 registers (two columns in BF16 at
-// 10000^2: 50 us; 65 us at one CTA per SM).
+// 10000^2: 44 us; 65 us at one CTA per SM).
 template <int FMT, int R, int GL>
 __host__ __device__ constexpr int scaled_ctas_per_sm() {
   return R == 1 ? (FMT == 7 && GL == 32 ? 3 : 2) : (R == 2 && FMT != 4) || (R == 4 && FMT == 7) ? 2 : 1;

@@ -490,12 +490,13 @@ __device__ __forceinline__ void finish_shared_groups(unsigned* __restrict__ seen
 // blocks.  A range covers pieces of one to a few 4-row bands; for every piece
 // the lanes' sums are folded and either y (and the state) is written
 // directly, when the band lies inside one range, or the piece's partial goes
-// to ws[band][segment], and the band's last warp adds its segments in order.  GL = 32: the warp takes one piece at a time; GL = 8: four lane
-// groups take the next four pieces at once (short bands, where a warp per
-// band would spend its time folding).  PRE: x is the transformed vector of
-// wz2_xt_kernel (4 BN floats per right-hand side); otherwise, with the lift, every
-// block transforms its own four values.  FIN: the band's last warp adds its segments
-// here; otherwise wz2_segment_epilogue does (see wz2_finish_blocks).
+// to ws[band][segment], and the band's last warp adds its segments in order.
+// GL = 32: the warp takes one piece at a time; GL = 8: four lane groups take the next
+// four pieces at once (short bands, where a warp per band would spend its time folding).
+// PRE: x is the transformed vector of wz2_xt_kernel (4 BN floats per right-hand side);
+// otherwise, with the lift, every block transforms its own four values.  FIN: the band's
+// last warp adds its segments here; otherwise wz2_segment_epilogue does (see
+// wz2_finish_blocks).
 template <int RATE, bool LIFT, int R, int UNROLL, int GL, bool PRE, bool FIN>
 __device__ __forceinline__ void wz2_gemv_body(const uint8_t* __restrict__ stream, int64_t M, int64_t N, int64_t BM,
                                               int64_t BN, const float* __restrict__ x, int64_t ldx, bool x_vec_ok,
@@ -563,7 +564,7 @@ __host__ __device__ constexpr int wz2_ctas_per_sm(int unroll) {
   return unroll == 8 ? (RATE <= 8 ? 3 : RATE <= 20 ? 2 : 1) : unroll == 4 ? (RATE <= 16 ? 3 : 2) : RATE <= 16 ? 4 : 3;
 }
 
-// Four columns: two CTAs per SM (rate 16, 10000^2: 140 us; 209 us with the 158 registers
+// Four columns: two CTAs per SM (rate 16, 10000^2: 118 us; 209 us with the 158 registers
 // that one would allow).
 template <int RATE, bool LIFT, int R, int UNROLL, int GL, bool PRE = LIFT, bool FIN = true>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, R == 1 ? wz2_ctas_per_sm<RATE>(UNROLL) : R == 4 ? 2 : 1)
