@@ -81,14 +81,14 @@ __device__ __forceinline__ void fold_level(float (&h)[N], float (&l)[N], float (
   if constexpr (O > 1) fold_level<N, kHalf, O / 2, TRIPLE>(h, l, m, lane);
 }
 
-// GUARD: sums that might leave FP32's range go down by 2^5 first (FP64 held them).
-template <int N, int GL, bool TRIPLE, bool GUARD = TRIPLE>
+// Triples: sums that might leave FP32's range go down by 2^5 first (FP64 held them).
+template <int N, int GL, bool TRIPLE>
 __device__ __forceinline__ void fold_lanes(float (&h)[N], float (&l)[N], int lane, double (&z)[N >= GL ? N / GL : 1]) {
   float m[TRIPLE ? N : 1];
 #pragma unroll
   for (int k = 0; k < (TRIPLE ? N : 1); ++k) m[k] = 0.f;
   bool big = false;
-  if constexpr (GUARD) {
+  if constexpr (TRIPLE) {
     float top = 0.f;
 #pragma unroll
     for (int k = 0; k < N; ++k) top = fmaxf(top, fabsf(h[k]));
@@ -106,7 +106,7 @@ __device__ __forceinline__ void fold_lanes(float (&h)[N], float (&l)[N], int lan
     } else {
       z[k] = widen(h[k]) + widen(l[k]);
     }
-    if (GUARD && big) z[k] *= 32.0;
+    if (TRIPLE && big) z[k] *= 32.0;
   }
 }
 
